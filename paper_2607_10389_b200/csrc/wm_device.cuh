@@ -342,6 +342,14 @@ __device__ __forceinline__ uint32_t mbar_try(uint32_t bar_s, uint32_t parity)
                  : "=r"(done) : "r"(bar_s), "r"(parity), "r"(200000u) : "memory");
     return done;
 }
+// The same question without waiting at all.
+__device__ __forceinline__ uint32_t mbar_test(uint32_t bar_s, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar_s), "r"(parity) : "memory");
+    return done;
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_first()
 {
     uint64_t pol;

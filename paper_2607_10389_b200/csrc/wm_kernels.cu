@@ -113,6 +113,7 @@ static const DeviceState* device_state()
     }
     if (cudaFuncSetAttribute(k_tile_digests<kTeamsPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(k_meta_crc, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
+    if (cudaFuncSetAttribute(k_xxh64_paced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXSmem) != cudaSuccess) return nullptr;
     for (int k = 0; k < 4; k++)
         for (int j = 0; j < 2; j++)
             if (cudaEventCreate(&s.ev[k][j]) != cudaSuccess) return nullptr;
@@ -285,11 +286,20 @@ wm_status wm_checksum_xxh64(const void* cache, uint64_t nbytes, uint32_t chunk_b
 {
     Geo g;
     if (!cache || !hash_out || !make_geo(nbytes, chunk_bytes, g) || !aligned16(cache)) return WM_ERR_ARG;
-    if (!device_state()) return WM_ERR_CUDA;
-    const uint32_t threads = 4u * g.n_chunks;
-    k_xxh64<<<(threads + 31u) / 32u, 32, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const unsigned char*>(cache), nbytes, chunk_bytes, g.n_chunks, seed,
-        reinterpret_cast<unsigned long long*>(hash_out));
+    const DeviceState* ds = device_state();
+    if (!ds) return WM_ERR_CUDA;
+    const unsigned char* c = static_cast<const unsigned char*>(cache);
+    unsigned long long* out = reinterpret_cast<unsigned long long*>(hash_out);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // The paced kernel takes eight chunks per block and two blocks per SM (its ring is 98 KiB): while
+    // all blocks fit at once, each chain runs at its step's latency: 162 us against 275 for 214 blocks
+    // (400 MB in 240 KiB chunks), 82 against 78 for 300, and from there on the other kernel is ahead
+    // (427 blocks: 311 against 289).
+    const uint32_t octets = (g.n_chunks + kXRows - 1u) / kXRows, n_sm = (uint32_t)ds->sm_count;
+    if (octets <= 2u * n_sm)
+        k_xxh64_paced<<<octets, kXThreads, kXSmem, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, n_sm, g.wait_ns);
+    else
+        k_xxh64<<<(4u * g.n_chunks + 31u) / 32u, 32, 0, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out);
     g_launches = 1;
     return launch_status();
 }

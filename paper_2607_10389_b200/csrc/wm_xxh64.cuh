@@ -3,13 +3,14 @@
 //
 // XXH64 takes its input in 32-byte stripes into four accumulators; lane k of a stripe feeds
 // accumulator k through  acc = rotl(acc + in * P2, 31) * P1,  a serial chain over the whole chunk
-// (digests of pieces cannot be combined, unlike a CRC).  So a chunk offers four threads of work
-// and the parallelism is across chunks: thread 4c + k owns accumulator k of chunk c, a warp
-// holds eight chunks, and one warp load fetches eight full 32-byte sectors.  What bounds the
-// kernel with large chunks is the latency of that chain, so the loads run two batches of 32
-// stripes ahead of it, in registers, and the product in * P2 is taken as a value arrives (off
-// the chain: only the add, the rotate and the multiplication by P1 depend on the accumulator).
-// With many small chunks (64 KiB) there are enough chains and the kernel runs at the memory rate.
+// (digests of pieces cannot be combined, unlike a CRC).  So a chunk offers four threads of work and
+// the parallelism is across chunks; a warp holds eight of them.  There are two kernels.
+//   k_xxh64        a warp loads its chunks' data into registers two batches ahead and walks the
+//                  chains.  With many chunks (64 KiB each, say) there are chains enough to cover
+//                  the loads and the products, and it runs at the memory rate (6.2 TB/s).
+//   k_xxh64_paced  for few chunks, where a scheduler has one chain warp at most and the latency of
+//                  one chain step bounds the call: the chain warp does nothing but chain steps,
+//                  other warps bring the data in and take the products.
 #pragma once
 
 namespace wm {
@@ -25,6 +26,34 @@ __device__ __forceinline__ unsigned long long x_round(unsigned long long acc, un
 __device__ __forceinline__ unsigned long long x_merge(unsigned long long h, unsigned long long v)
 {
     return (h ^ x_round(0ull, v)) * kXP1 + kXP4;
+}
+
+// The four accumulators merged, the bytes behind the last whole stripe, the avalanche.
+__device__ __forceinline__ unsigned long long x_finish(const unsigned char* base, uint64_t len, unsigned long long seed,
+                                                       unsigned long long v1, unsigned long long v2, unsigned long long v3,
+                                                       unsigned long long v4)
+{
+    unsigned long long h;
+    if (len >= 32u) {
+        h = x_rotl(v1, 1) + x_rotl(v2, 7) + x_rotl(v3, 12) + x_rotl(v4, 18);
+        h = x_merge(h, v1); h = x_merge(h, v2); h = x_merge(h, v3); h = x_merge(h, v4);
+    } else {
+        h = seed + kXP5;
+    }
+    h += len;
+    const unsigned char* t = base + (len & ~31ull);
+    uint32_t left = (uint32_t)len & 31u;
+    while (left >= 8u) {
+        h = x_rotl(h ^ x_round(0ull, *reinterpret_cast<const unsigned long long*>(t)), 27) * kXP1 + kXP4;
+        t += 8; left -= 8u;
+    }
+    if (left >= 4u) {
+        h = x_rotl(h ^ ((unsigned long long)*reinterpret_cast<const uint32_t*>(t) * kXP1), 23) * kXP2 + kXP3;
+        t += 4; left -= 4u;
+    }
+    while (left) { h = x_rotl(h ^ ((unsigned long long)*t * kXP5), 11) * kXP1; t++; left--; }
+    h ^= h >> 33; h *= kXP2; h ^= h >> 29; h *= kXP3; h ^= h >> 32;
+    return h;
 }
 
 constexpr int kXBatch = 32;       // stripes per batch of loads
@@ -82,27 +111,214 @@ k_xxh64(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk
     const unsigned long long v1 = __shfl_sync(0xFFFFFFFFu, v, q0), v2 = __shfl_sync(0xFFFFFFFFu, v, q0 + 1u),
                              v3 = __shfl_sync(0xFFFFFFFFu, v, q0 + 2u), v4 = __shfl_sync(0xFFFFFFFFu, v, q0 + 3u);
     if (!live || k != 0u) return;
-    unsigned long long h;
-    if (len >= 32u) {
-        h = x_rotl(v1, 1) + x_rotl(v2, 7) + x_rotl(v3, 12) + x_rotl(v4, 18);
-        h = x_merge(h, v1); h = x_merge(h, v2); h = x_merge(h, v3); h = x_merge(h, v4);
-    } else {
-        h = seed + kXP5;
+    out[c] = x_finish(base, len, seed, v1, v2, v3, v4);
+}
+
+// ---- few chunks: one warp walks the chains, the others feed it
+constexpr uint32_t kXRows = 8;                          // chunks a block works on at a time
+constexpr uint32_t kXSeg = 64;                          // stripes of every chunk in one slot of the ring
+constexpr uint32_t kXRowBytes = 32u * kXSeg;
+constexpr uint32_t kXPitch = kXRowBytes + 32u;          // (rows 32 bytes apart modulo 128: the chains' reads meet no bank twice)
+constexpr uint32_t kXSlot = kXRows * kXPitch;
+constexpr uint32_t kXSlots = 6, kXAhead = 4;            // slots of the ring; slots whose copies are under way
+constexpr uint32_t kXSmem = kXSlots * kXSlot;
+static_assert(kXAhead + 2u <= kXSlots, "a slot is handed over before the ring comes round to it");
+constexpr uint32_t kXFeeders = 4;                       // warps that bring the data in and multiply it
+constexpr uint32_t kXThreads = 256;                     // (warps 0, 1: chains; 2, 3, 6, 7: feeders, on the other two schedulers)
+
+// A warp's bounded wait for a phase of a barrier in shared memory; the answer is the same in every
+// lane.  The call has no result record to say that it failed, so a block that was merely descheduled
+// for a while must not be taken for one: a wait ends only when the budget has passed AND the barrier
+// has been tried 16,384 times (the warps that wait for each other are of one block and stand still
+// together).
+__device__ __forceinline__ bool x_wait(uint32_t bar, uint32_t parity, uint32_t budget_ns, volatile uint32_t* fail)
+{
+    bool ok = mbar_try(bar, parity) != 0u;
+    if (!ok) {
+        const uint32_t t0 = now_ns();
+        uint32_t tries = 0;
+        do {
+            ok = mbar_try(bar, parity) != 0u;
+        } while (!ok && *fail == 0u && (++tries < 16384u || now_ns() - t0 <= budget_ns));
     }
-    h += len;
-    const unsigned char* t = base + stripes * 32u;
-    uint64_t left = len - stripes * 32u;
-    while (left >= 8u) {
-        h = x_rotl(h ^ x_round(0ull, *reinterpret_cast<const unsigned long long*>(t)), 27) * kXP1 + kXP4;
-        t += 8; left -= 8u;
+    ok = __all_sync(0xFFFFFFFFu, ok);
+    if (!ok) *fail = 1u;
+    return ok;
+}
+__device__ __forceinline__ void x_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// One step of a chain: s' = rotl(s, 31) * P1 + x.  Written out in 32-bit halves: behind the rotation
+// (two funnel shifts) stand one wide product with x as its addend and, beside it, the two products
+// that only reach the high half; one add joins them.  23 cycles a step, where the plain formula
+// takes 28 as it is compiled.
+__device__ __forceinline__ unsigned long long x_step(unsigned long long s, unsigned long long x)
+{
+    const uint32_t p1lo = (uint32_t)kXP1, p1hi = (uint32_t)(kXP1 >> 32);
+    const uint32_t lo = (uint32_t)s, hi = (uint32_t)(s >> 32);
+    const uint32_t rl = __funnelshift_r(hi, lo, 1), rh = __funnelshift_r(lo, hi, 1);       // rotl 31 = halves swapped, one to the right
+    unsigned long long w;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(w) : "r"(rl), "r"(p1lo), "l"(x));
+    const uint32_t b = rh * p1lo + rl * p1hi;
+    return (unsigned long long)(uint32_t)w | ((unsigned long long)((uint32_t)(w >> 32) + b) << 32);
+}
+
+// x_step(x_before(v), x) is v + x: the state in front of a chain's first stripe.
+constexpr unsigned long long x_inverse(unsigned long long p)      // modulo 2^64 (Newton; p odd)
+{
+    unsigned long long r = p;
+    for (int i = 0; i < 6; i++) r *= 2u - p * r;
+    return r;
+}
+constexpr unsigned long long kXP1Inverse = x_inverse(kXP1);
+__device__ __forceinline__ unsigned long long x_before(unsigned long long v) { return x_rotl(v * kXP1Inverse, 33); }
+
+__device__ __forceinline__ void x_load16(unsigned long long (&x)[16], uint32_t a)
+{
+#pragma unroll
+    for (int i = 0; i < 16; i++) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(x[i]) : "r"(a + 32u * i));
+}
+
+// One block per eight chunks.  n_sm: blocks up to that number are alone on their SM, the ones above
+// share one; their chains are walked by different warps, so that two chains never share a scheduler.
+// Measured (one chain step per 32-byte stripe): 34 ns a stripe with k_xxh64, 15 ns here with a block
+// alone on its SM and 18 ns with two; 1.67 GB in 1 MiB chunks (200 blocks) 1.14 -> 0.61 ms, 8 GiB
+// of 4 MiB chunks is bound by the same chain.  What is left is the step's own latency (23 cycles,
+// 12 ns) and the hand-over of a slot every 64 steps.
+__global__ void __launch_bounds__(kXThreads)
+k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk_bytes, uint32_t n_chunks,
+              unsigned long long seed, unsigned long long* __restrict__ out, uint32_t n_sm, uint32_t wait_ns)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(8) unsigned long long s_full[kXSlots], s_empty[kXSlots];
+    __shared__ uint32_t s_fail;
+    const uint32_t warp = threadIdx.x / 32u, lane = threadIdx.x % 32u;
+    const uint32_t chain_warp = (blockIdx.x / n_sm) & 1u;
+    if (threadIdx.x == 0) {
+        for (uint32_t i = 0; i < kXSlots; i++) { mbar_init(&s_full[i], kXFeeders); mbar_init(&s_empty[i], 1); }
+        s_fail = 0;
     }
-    if (left >= 4u) {
-        h = x_rotl(h ^ ((unsigned long long)*reinterpret_cast<const uint32_t*>(t) * kXP1), 23) * kXP2 + kXP3;
-        t += 4; left -= 4u;
+    __syncthreads();
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem);
+    const uint32_t full = (uint32_t)__cvta_generic_to_shared(s_full), empty = (uint32_t)__cvta_generic_to_shared(s_empty);
+    auto length = [&](uint32_t c) -> uint32_t {          // bytes of chunk c (0: there is none)
+        if (c >= n_chunks) return 0u;
+        const uint64_t left = nbytes - (uint64_t)c * chunk_bytes;
+        return left < chunk_bytes ? (uint32_t)left : chunk_bytes;
+    };
+    const uint32_t n_seg = (length(blockIdx.x * kXRows) / 32u + kXSeg - 1u) / kXSeg;      // (the first of the eight is the longest)
+
+    if (warp & 2u) {
+        // ---- the warps that feed the ring, two chunks each: sixteen lanes take 256 consecutive bytes of
+        // one chunk, and every lane waits for its own copies only
+        const uint32_t feeder = (warp & 1u) + (warp >> 2) * 2u;
+        const uint32_t row = 2u * feeder + lane / 16u, col = 16u * (lane % 16u);
+        const uint32_t mine = ring + row * kXPitch + col;
+        constexpr uint32_t kUnits = kXRowBytes / 256u;   // 16-byte pieces of a slot per lane
+        const uint32_t c = blockIdx.x * kXRows + row;
+        const uint32_t whole = length(c) & ~31u;         // bytes in whole stripes
+        const unsigned char* p = cache + (uint64_t)(whole ? c : 0u) * chunk_bytes + col;
+        auto hand_over = [&](uint32_t s) {               // the products, in place (all loads before the first store)
+            const uint32_t a = mine + (s % kXSlots) * kXSlot;
+            unsigned long long u[kUnits], v[kUnits];
+#pragma unroll
+            for (uint32_t i = 0; i < kUnits; i++) asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(u[i]), "=l"(v[i]) : "r"(a + 256u * i));
+#pragma unroll
+            for (uint32_t i = 0; i < kUnits; i++)
+                asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a + 256u * i), "l"(u[i] * kXP2), "l"(v[i] * kXP2) : "memory");
+            __syncwarp();
+            if (lane == 0) x_arrive(full + 8u * (s % kXSlots));
+        };
+        uint32_t done = 0;
+        for (uint32_t s = 0; s < n_seg; s++) {
+            if (s >= kXSlots && !x_wait(empty + 8u * (s % kXSlots), ((s / kXSlots) & 1u) ^ 1u, wait_ns, &s_fail)) {
+                cp_async_wait_all();
+                return;
+            }
+            const uint32_t a = mine + (s % kXSlots) * kXSlot;
+            const uint32_t at = s * kXRowBytes;
+#pragma unroll
+            for (uint32_t i = 0; i < kUnits; i++)
+                if (at + 256u * i + col < whole)
+                    asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(a + 256u * i), "l"(p + at + 256u * i) : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (s + 1u - done > kXAhead) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(kXAhead) : "memory");
+                hand_over(done++);
+            }
+        }
+        cp_async_wait_all();
+        while (done < n_seg) hand_over(done++);
+        return;
     }
-    while (left) { h = x_rotl(h ^ ((unsigned long long)*t * kXP5), 11) * kXP1; t++; left--; }
-    h ^= h >> 33; h *= kXP2; h ^= h >> 29; h *= kXP3; h ^= h >> 32;
-    out[c] = h;
+    if (warp != chain_warp) return;
+
+    // ---- the chains: lane 4 r + k is accumulator k of chunk r of the eight
+    const uint32_t k = lane & 3u, row = lane >> 2;
+    const uint32_t mine = ring + row * kXPitch + 8u * k;
+    const uint32_t c = blockIdx.x * kXRows + row;
+    const uint32_t len = length(c), stripes = len / 32u;
+    // A segment in whose midst a chunk ends (only the cache's last chunk can) is walked with a test
+    // per stripe.  Behind its chunk's end a chain runs on with whatever lies in its row, its result
+    // having been put aside.
+    const uint32_t uneven = __ballot_sync(0xFFFFFFFFu, stripes % kXSeg != 0u);
+    const uint32_t odd_seg = uneven ? __shfl_sync(0xFFFFFFFFu, stripes, __ffs(uneven) - 1) / kXSeg : 0xFFFFFFFFu;
+    // the state is the accumulator with the next product already added; the last step adds 0
+    unsigned long long v = k == 0u ? seed + kXP1 + kXP2 : k == 1u ? seed + kXP2 : k == 2u ? seed : seed - kXP1;
+    unsigned long long s = x_before(v), at_end = 0ull;
+    unsigned long long x0[16], x1[16];
+    auto steps = [&](const unsigned long long (&x)[16]) {
+#pragma unroll
+        for (int i = 0; i < 16; i++) s = x_step(s, x[i]);
+    };
+    bool ok = n_seg == 0u || x_wait(full, 0u, wait_ns, &s_fail);
+    if (n_seg) x_load16(x0, mine);
+    uint32_t slot = 0, parity = 0, a = mine;             // of segment g
+    for (uint32_t g = 0; g < n_seg && ok; g++) {
+        const bool wrap = slot + 1u == kXSlots;
+        const uint32_t n_slot = wrap ? 0u : slot + 1u, n_parity = parity ^ (wrap ? 1u : 0u), n_a = wrap ? mine : a + kXSlot;
+        const bool more = g + 1u < n_seg;
+        // whether the next segment is there is asked, and its first words are fetched, while this one's
+        // last quarter is still to be walked: nothing waits at the seam
+        uint32_t ready = 1u;
+        if (g != odd_seg) {
+            x_load16(x1, a + 512u);
+            steps(x0);
+            x_load16(x0, a + 1024u);
+            steps(x1);
+            x_load16(x1, a + 1536u);
+            if (more) ready = mbar_test(full + 8u * n_slot, n_parity);
+            steps(x0);
+        } else {
+            ready = 0u;
+            for (uint32_t i = 0; i < kXSeg; i++) {
+                unsigned long long x;
+                asm volatile("ld.shared.u64 %0, [%1];" : "=l"(x) : "r"(a + 32u * i));
+                const unsigned long long n = x_step(s, x);
+                if (g * kXSeg + i < stripes) s = n;
+            }
+        }
+        if (more) {
+            if (!__all_sync(0xFFFFFFFFu, ready != 0u)) ok = x_wait(full + 8u * n_slot, n_parity, wait_ns, &s_fail);
+            x_load16(x0, n_a);
+        }
+        if (g != odd_seg) steps(x1);
+        if ((stripes + kXSeg - 1u) / kXSeg == g + 1u) at_end = s;
+        __syncwarp();
+        if (lane == 0) x_arrive(empty + 8u * slot);
+        slot = n_slot; parity = n_parity; a = n_a;
+    }
+    if (stripes) v = x_step(at_end, 0ull);
+
+    // the quad's four accumulators to its first thread
+    const uint32_t q0 = lane & ~3u;
+    const unsigned long long v1 = __shfl_sync(0xFFFFFFFFu, v, q0), v2 = __shfl_sync(0xFFFFFFFFu, v, q0 + 1u),
+                             v3 = __shfl_sync(0xFFFFFFFFu, v, q0 + 2u), v4 = __shfl_sync(0xFFFFFFFFu, v, q0 + 3u);
+    if (k != 0u || c >= n_chunks) return;
+    // (fail closed: no hash of data that never arrived)
+    out[c] = ok ? x_finish(cache + (uint64_t)c * chunk_bytes, len, seed, v1, v2, v3, v4) : 0ull;
 }
 
 }  // namespace wm

@@ -64,3 +64,17 @@ def test_gpu_xxh64_engine_cache_and_bad_arguments():
     assert got.tolist() == lib_all                                  # and every chunk against the package
     with pytest.raises(wm.WmError, match="ERR_ARG"):
         wm.wm_checksum_xxh64(cache.cuda()[:100], 1000, 0, out)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_chunks", [7, 8, 9, 2 * 148 * 8, 2 * 148 * 8 + 11])       # eight chunks a block; the last size takes the other kernel
+@pytest.mark.parametrize("last", [5, 31, 2047, 2048 + 32, TILE - 9, TILE])             # the ring's slots hold 2048 bytes of a chunk
+def test_gpu_xxh64_octets_and_ring_edges(n_chunks, last):
+    import torch
+    from paper_2607_10389_b200 import binding as wm
+    n = (n_chunks - 1) * TILE + last
+    a = _bytes(n, n_chunks + last)
+    out = torch.full((n_chunks,), 5, dtype=torch.int64, device="cuda")
+    wm.wm_checksum_xxh64(torch.from_numpy(a).cuda(), TILE, 99, out)
+    want = [xxhash.xxh64(a[o:o + TILE].tobytes(), seed=99).intdigest() for o in range(0, n, TILE)]
+    assert out.cpu().numpy().view(np.uint64).tolist() == want
