@@ -8,12 +8,14 @@
 // (x^1024, table G); the lane's place inside the row and the warp's place inside the tile
 // are folded in once per tile with two small nibble tables (NK, NW).
 //
-// Table lookups are the inner loop (one per byte), so their address arithmetic is reduced to
-// a single byte permute: the tables sit at a 64 KiB-aligned shared address, entry b of a
-// table starts at b*256 and holds one copy per lane (lane l only ever touches bank l: no
-// bank conflicts on data-dependent indices), so address = base | b << 8 | lane*4 is
-// PRMT(value, base | lane*4).  The second table of a pair lives 128 bytes further and is
-// reached through the load's immediate offset.
+// Table lookups are the inner loop (one per byte), so their address arithmetic is reduced to one
+// instruction, and to one that does not queue up with the rest: an entry of a table is 128 bytes and
+// holds one copy per lane (lane l only ever touches bank l: no bank conflicts on data-dependent
+// indices), so the address base + 128 * byte + 4 * lane is the dot product of the word's four bytes
+// with a vector that picks one of them times 128 (dp4a).  That instruction runs on the multiplier's
+// pipe.  The XORs, shifts, permutes and logic of everything else here share the other integer pipe,
+// which is what these kernels fill first (measured, warp instructions per cycle and SM: permutes and
+// logic together 2.0, dp4a and logic together 3.9).
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -25,27 +27,23 @@ namespace wm {
 constexpr uint32_t kTile = 16384;
 constexpr uint32_t kTeamThreads = 256;
 constexpr uint32_t kWordsPerLane = 16;
-// Dynamic shared memory every table-using kernel asks for: the 144 KiB image plus 81 KiB
-// that the 64 KiB alignment splits into a part below and a part above the image (with the
-// window starting at 1 KiB: 63 KiB below, 18 KiB above; a stage of the leaf-mode kernels is
-// 16 bytes longer than a tile, and one of the four has to fit above).  227 KiB is the per-block
-// maximum for static and dynamic shared memory together; the kernels' static part is below 1 KiB.
-constexpr uint32_t kDynSmem = kImgBytes + 0x10000 + 0x4400;
+// Dynamic shared memory every table-using kernel asks for: the 144 KiB image and 81 KiB for stages and
+// control blocks.  227 KiB is the per-block maximum for static and dynamic shared memory together;
+// the kernels' static part is below 1 KiB.
+constexpr uint32_t kDynSmem = kImgBytes + 0x14400;
 
 struct Smem {
-    uint32_t L01, L23, LNK;      // shared-window address of A01 / A23 / NK, or'ed with lane*4
+    uint32_t L;                  // shared-window address of the image + lane * 4
     const uint32_t* NW;          // warp-position nibble tables [8][8][16]
-    unsigned char* lo; uint32_t lo_bytes;    // free space below the image
-    unsigned char* hi; uint32_t hi_bytes;    // free space above the image
+    unsigned char* free; uint32_t free_bytes;    // what is left behind the image
     bool ok;
 
     // carve `bytes` (multiple of 16) from the free space; nullptr when it does not fit
     __device__ unsigned char* take(uint32_t bytes)
     {
-        unsigned char* p = nullptr;
-        if (lo_bytes >= bytes) { p = lo; lo += bytes; lo_bytes -= bytes; }
-        else if (hi_bytes >= bytes) { p = hi; hi += bytes; hi_bytes -= bytes; }
-        else ok = false;
+        if (free_bytes < bytes) { ok = false; return nullptr; }
+        unsigned char* p = free;
+        free += bytes; free_bytes -= bytes;
         return p;
     }
 };
@@ -54,14 +52,10 @@ struct Smem {
 __device__ __forceinline__ Smem setup_smem(unsigned char* smem, const Tables* __restrict__ tab)
 {
     Smem s;
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
-    const uint32_t tab0 = (base + 0xFFFFu) & ~0xFFFFu;
-    unsigned char* img = smem + (tab0 - base);
     s.ok = true;
-    s.lo = smem; s.lo_bytes = tab0 - base;
-    s.hi = img + kImgBytes; s.hi_bytes = kDynSmem - kImgBytes - (tab0 - base);
+    s.free = smem + kImgBytes; s.free_bytes = kDynSmem - kImgBytes;
     const uint4* src = reinterpret_cast<const uint4*>(tab->image);
-    uint4* dst = reinterpret_cast<uint4*>(img);
+    uint4* dst = reinterpret_cast<uint4*>(smem);
     for (uint32_t i = threadIdx.x; i < kImgBytes / 16; i += blockDim.x) dst[i] = src[i];
     uint32_t* nw = reinterpret_cast<uint32_t*>(s.take(8 * 8 * 16 * 4));
     if (nw) {
@@ -69,10 +63,7 @@ __device__ __forceinline__ Smem setup_smem(unsigned char* smem, const Tables* __
         for (uint32_t i = threadIdx.x; i < 8 * 8 * 16; i += blockDim.x) nw[i] = gNW[i];
     }
     s.NW = nw;
-    const uint32_t lane4 = (threadIdx.x & 31u) * 4u;
-    s.L01 = (tab0 + kImgA01) | lane4;
-    s.L23 = (tab0 + kImgA23) | lane4;
-    s.LNK = (tab0 + kImgNK) | lane4;
+    s.L = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x & 31u) * 4u;
     __syncthreads();
     return s;
 }
@@ -151,22 +142,26 @@ __device__ __forceinline__ void team_bar(uint32_t team)
 // One chain step: (state ^ word) advanced over 128 bytes.
 __device__ __forceinline__ uint32_t chain_step(const Smem& S, uint32_t x)
 {
-    const uint32_t a = lds_off<0>(__byte_perm(x, S.L01, 0x7604));
-    const uint32_t b = lds_off<128>(__byte_perm(x, S.L01, 0x7614));
-    const uint32_t c = lds_off<0>(__byte_perm(x, S.L23, 0x7624));
-    const uint32_t d = lds_off<128>(__byte_perm(x, S.L23, 0x7634));
+    const uint32_t a = lds_off<0 * kImgTable>(__dp4a(x, kImgEntry, S.L));
+    const uint32_t b = lds_off<1 * kImgTable>(__dp4a(x, kImgEntry << 8, S.L));
+    const uint32_t c = lds_off<2 * kImgTable>(__dp4a(x, kImgEntry << 16, S.L));
+    const uint32_t d = lds_off<3 * kImgTable>(__dp4a(x, kImgEntry << 24, S.L));
     return a ^ b ^ c ^ d;
 }
 
-// Lane finish: x advanced over 128 - 4*lane bytes (eight nibble lookups).
+// Lane finish: x advanced over 128 - 4*lane bytes (eight nibble lookups; an odd nibble is 16 times its
+// value in its byte, so its entry's place is 8 times that).
+template <int N>
+__device__ __forceinline__ uint32_t nibble_entry(const Smem& S, uint32_t xe, uint32_t xo)
+{
+    return lds_off<kImgNK + N * kImgNibble>((N & 1) ? __dp4a(xo, (kImgEntry / 16u) << (8 * (N / 2)), S.L)
+                                                    : __dp4a(xe, kImgEntry << (8 * (N / 2)), S.L));
+}
 __device__ __forceinline__ uint32_t lane_finish(const Smem& S, uint32_t x)
 {
-    const uint32_t xe = x & 0x0F0F0F0Fu, xo = (x >> 4) & 0x0F0F0F0Fu;
-    uint32_t r = lds_off<0x0000>(__byte_perm(xe, S.LNK, 0x7604)) ^ lds_off<0x0080>(__byte_perm(xo, S.LNK, 0x7604));
-    r ^= lds_off<0x1000>(__byte_perm(xe, S.LNK, 0x7614)) ^ lds_off<0x1080>(__byte_perm(xo, S.LNK, 0x7614));
-    r ^= lds_off<0x2000>(__byte_perm(xe, S.LNK, 0x7624)) ^ lds_off<0x2080>(__byte_perm(xo, S.LNK, 0x7624));
-    r ^= lds_off<0x3000>(__byte_perm(xe, S.LNK, 0x7634)) ^ lds_off<0x3080>(__byte_perm(xo, S.LNK, 0x7634));
-    return r;
+    const uint32_t xe = x & 0x0F0F0F0Fu, xo = x & 0xF0F0F0F0u;
+    return nibble_entry<0>(S, xe, xo) ^ nibble_entry<1>(S, xe, xo) ^ nibble_entry<2>(S, xe, xo) ^ nibble_entry<3>(S, xe, xo) ^
+           nibble_entry<4>(S, xe, xo) ^ nibble_entry<5>(S, xe, xo) ^ nibble_entry<6>(S, xe, xo) ^ nibble_entry<7>(S, xe, xo);
 }
 
 // CRC state (zero start) of a warp's 2048-byte block from the 16 words each lane holds.
@@ -196,7 +191,7 @@ __device__ __forceinline__ void load_small_chain_tables(uint32_t* sG, const Tabl
 {
     for (uint32_t i = threadIdx.x; i < 1024; i += blockDim.x) {
         const uint32_t k = i >> 8, b = i & 255u;
-        sG[i] = tab->image[((k < 2 ? kImgA01 : kImgA23) + b * 256u + (k & 1u) * 128u) / 4u];
+        sG[i] = tab->image[(k * kImgTable + b * kImgEntry) / 4u];
     }
     __syncthreads();
 }
@@ -213,7 +208,7 @@ __device__ __forceinline__ uint32_t tile_digest_part_small(const uint32_t* sG, c
     uint32_t r = 0;
 #pragma unroll
     for (uint32_t n = 0; n < 8; n++)
-        r ^= __ldg(&tab->image[(kImgNK + (n / 2u) * 0x1000u + ((x >> (4u * n)) & 15u) * 256u + (n & 1u) * 128u) / 4u + lane]);
+        r ^= __ldg(&tab->image[(kImgNK + n * kImgNibble + ((x >> (4u * n)) & 15u) * kImgEntry) / 4u + lane]);
     const uint32_t digest = __reduce_xor_sync(0xFFFFFFFFu, r);
     uint32_t v = 0;
     if (lane < 8) v = __ldg(&tab->NW[warp][lane][(digest >> (4 * lane)) & 15u]);

@@ -12,14 +12,13 @@ namespace wm {
 constexpr uint32_t kPolyReflected = 0x82F63B78u;   // CRC32C (Castagnoli), the checksum of the wire format
 constexpr uint32_t kPolyZlib = 0xEDB88320u;        // CRC-32 of zlib, an option of the checksum call only
 
-// Byte offsets inside the shared-memory table image.  The image is placed at an address that
-// is a multiple of 64 KiB inside the shared window, so that "table base | value << 8 | lane
-// slot" can be put together with one byte permute.
-//   A01: entry b at b*256: 32 lane copies of G[0][b] (bytes 0..127), then of G[1][b]
-//   A23: the same for G[2], G[3]
-//   NK : four 4 KiB arrays, array j = nibbles 2j and 2j+1 of the lane-finish table:
-//        entry v at v*256: NK[lane][2j][v] for the 32 lanes, then NK[lane][2j+1][v]
-constexpr uint32_t kImgA01 = 0x00000, kImgA23 = 0x10000, kImgNK = 0x20000, kImgBytes = 0x24000;
+// Byte offsets inside the shared-memory table image.  An entry is 128 bytes, one 32-bit copy per
+// lane, so the address of entry v is base + 128 v + 4 lane, one integer dot product of the word that
+// holds v (see chain_step).
+//   G  : table k at k * kImgTable, 256 entries: G[k][b]
+//   NK : array n at kImgNK + n * kImgNibble, 16 entries: entry v is NK[lane][n][v]
+constexpr uint32_t kImgEntry = 128, kImgTable = 256 * kImgEntry, kImgNibble = 16 * kImgEntry;
+constexpr uint32_t kImgNK = 4 * kImgTable, kImgBytes = kImgNK + 8 * kImgNibble;
 
 // Tables shared by all kernels; one copy lives in device memory per device.
 struct Tables {
@@ -61,7 +60,7 @@ inline void build_tables(Tables& t, uint32_t poly = kPolyReflected)
     for (uint32_t k = 0; k < 4; k++)
         for (uint32_t b = 0; b < 256; b++) {
             const uint32_t g = mulmod(b << (8 * k), k128, poly);
-            uint32_t* dst = t.image + ((k < 2 ? kImgA01 : kImgA23) + b * 256 + (k & 1) * 128) / 4;
+            uint32_t* dst = t.image + (k * kImgTable + b * kImgEntry) / 4;
             for (uint32_t l = 0; l < 32; l++) dst[l] = g;
             t.HT[k][b] = mulmod(b << (8 * k), kTile, poly);
         }
@@ -71,7 +70,7 @@ inline void build_tables(Tables& t, uint32_t poly = kPolyReflected)
         const uint32_t kl = x_pow_bytes(128 - 4 * l, poly);
         for (uint32_t n = 0; n < 8; n++)
             for (uint32_t v = 0; v < 16; v++)
-                t.image[(kImgNK + (n / 2) * 0x1000 + v * 256 + (n & 1) * 128) / 4 + l] = mulmod(v << (4 * n), kl, poly);
+                t.image[(kImgNK + n * kImgNibble + v * kImgEntry) / 4 + l] = mulmod(v << (4 * n), kl, poly);
     }
     for (uint32_t w = 0; w < 8; w++) {
         const uint32_t kw = x_pow_bytes(2048u * (7 - w), poly);
