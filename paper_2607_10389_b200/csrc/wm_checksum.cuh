@@ -35,12 +35,17 @@ k_tile_digests(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tabl
     tc += team;
     const uint64_t stride = (uint64_t)gridDim.x * TEAMS;
     const uint64_t pol = l2_policy_evict_first();
-    auto full = [&](uint64_t tile) { return tile < g.n_tiles && g.nbytes - tile * kTile >= kTile; };
     auto start_copy = [&](uint64_t tile) {     // one thread of the team
-        if (full(tile) && !(g.inject & kInjectNoCopy)) bulk_load(stage, cache + tile * kTile, kTile, &tc->mbar, pol);
+        if (tile < g.n_full_tiles && !(g.inject & kInjectNoCopy)) bulk_load(stage, cache + tile * kTile, kTile, &tc->mbar, pol);
     };
 
     uint64_t t = (uint64_t)blockIdx.x * TEAMS + team;
+    // the ragged last tile: by the team that comes by next in turn, before its loop
+    if (g.tail_len && t == g.n_full_tiles % stride) {
+        const uint32_t v = ragged_tile_digest(S, g, stage, cache + (uint64_t)g.n_full_tiles * kTile, tc->wdig[0], team, tt);
+        if (tt == 0) ws.dig[g.n_full_tiles] = v;
+        team_bar(team);
+    }
     if (tt == 64u) { mbar_init(&tc->mbar, 1); start_copy(t); }
     team_bar(team);
     uint32_t phase = 0, par = 0;
@@ -48,22 +53,16 @@ k_tile_digests(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tabl
     // One team barrier per tile.  The single-lane chores sit on different warps (the team waits
     // for whichever warp has the most to do): warp 2 starts the next copy, warp 1 folds and
     // stores the previous tile's digest once the barrier has made its parts complete.
-    for (; t < g.n_tiles; t += stride) {
+    for (; t < g.n_full_tiles; t += stride) {
         const bool first = first_in_chunk(g, (uint32_t)t);
         uint32_t d[kWordsPerLane];
-        bool fold = first;
-        if (full(t)) {
-            wait_for_copy<false>(&tc->mbar, phase, g.wait_ns, ws.ctrl, (g.inject & kInjectNoCopy) != 0u);
-            phase ^= 1u;
-            read_staged_words(stage, warp, lane, d);
-        } else {
-            load_tile_words_guarded(cache + t * kTile, (uint32_t)(g.nbytes - t * kTile), first, warp, lane, d);
-            fold = false;
-        }
+        wait_for_copy<false>(&tc->mbar, phase, g.wait_ns, ws.ctrl, (g.inject & kInjectNoCopy) != 0u);
+        phase ^= 1u;
+        read_staged_words(stage, warp, lane, d);
         team_bar(team);                          // stage free; the previous tile's digest parts complete
         if (tt == 64u) start_copy(t + stride);
         if (tt == 32u && t_done != ~0ull) ws.dig[t_done] = xor8(tc->wdig[par ^ 1u]);
-        const uint32_t v = tile_digest_part(S, d, fold, warp, lane);
+        const uint32_t v = tile_digest_part(S, d, first, warp, lane);
         if (lane == 0) tc->wdig[par][warp] = v;
         t_done = t;
         par ^= 1u;

@@ -295,7 +295,7 @@ k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g,
 }
 
 struct DecSlot {                 // what the team's first thread prepares for a tile ahead of its turn
-    uint32_t t;                  // tile (>= n_tiles: none left)
+    uint32_t t;                  // tile (>= n_full_tiles: none left)
     uint32_t entry;              // tile table entry | (first tile of its chunk) << 16
     unsigned long long src;      // offset of the encoded tile inside the payload
 };
@@ -445,8 +445,9 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     // present chunks only; k_decode_check listed those chunks (ws.plist, in any order: nothing here
     // depends on the order of tiles), and ticket k is tile k mod tiles_per_chunk of the
     // (k / tiles_per_chunk)-th listed chunk, so a sparse image costs nothing for what it leaves
-    // out.  Only the cache's last chunk can have fewer tiles: a ticket that falls behind its end
-    // has no tile, and the claimer draws the next one at once.
+    // out.  Only the cache's last chunk can have fewer tiles: a ticket that falls behind its end (or
+    // on the ragged last tile, which is not claimed) has no tile, and the claimer draws the next one
+    // at once.
     const bool masked = ((reinterpret_cast<const uint32_t*>(wire)[1] >> 16) & 1u) != 0u;
     const uint32_t n_tickets = masked ? ld_volatile_u32(&ws.ctrl->n_present) * g.tiles_per_chunk : 0u;
     auto claim = [&]() -> uint32_t {
@@ -455,7 +456,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         while (k < n_tickets) {
             const uint32_t j = chunk_of(g, k);
             const uint32_t t = ws.plist[j] * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
-            if (t < g.n_tiles) return t;
+            if (t < g.n_full_tiles) return t;
             k = atomicAdd(&ws.ctrl->ticket, 1u);
         }
         return kNone;
@@ -465,25 +466,38 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
 
     // a tile's entry word and payload offset (blocking: prologue only)
     auto lookup = [&](uint32_t t, DecSlot* sl) {
-        if (LEAVES && t < g.n_tiles) tc->dstp[sl - tc->slot] = ws.tptr[t];
+        if (LEAVES && t < g.n_full_tiles) tc->dstp[sl - tc->slot] = ws.tptr[t];
         sl->t = t;
         sl->entry = 0; sl->src = 0;
-        if (t < g.n_tiles) {
+        if (t < g.n_full_tiles) {
             const uint32_t e = tab16_of()[t];
             sl->entry = e | (first_in_chunk(g, t) ? 0x10000u : 0u);
             if (e) sl->src = *reinterpret_cast<const unsigned long long*>(dir_of() + 16ull * chunk_of(g, t)) + ws.rel[t];
         }
     };
-    // staged tiles: full RAW and PACK tiles (everything except absent tiles and the ragged tail)
+    // staged tiles: full RAW and PACK tiles (everything except absent tiles and zero / constant ones)
     // (images with the entropy option hold ENT tiles too: entry 0x8000 | length / 32)
-    auto is_ent_entry = [](uint32_t e) { return ENT != 0 && e > 0x8000u && e != 0xFFFFu; };
+    auto is_ent_entry = [](uint32_t e) { return ENT != 0 && e > 0x8000u; };
     auto is_pack_entry = [](uint32_t e) { return ENT != 1 && e >= 258u && e < 512u; };
     auto is_staged = [&](uint32_t e) { return e == 512u || is_pack_entry(e) || is_ent_entry(e); };
     auto start_copy = [&](const DecSlot& sl) {   // leader only
         const uint32_t e = sl.entry & 0xFFFFu;
-        if (sl.t < g.n_tiles && is_staged(e) && !(g.inject & kInjectNoCopy)) bulk_load_at(stage_s, payload_of() + sl.src, 32u * (e & 0x7FFFu), tc_s + (uint32_t)offsetof(DecTeamCtl, mbar), 0);
+        if (sl.t < g.n_full_tiles && is_staged(e) && !(g.inject & kInjectNoCopy)) bulk_load_at(stage_s, payload_of() + sl.src, 32u * (e & 0x7FFFu), tc_s + (uint32_t)offsetof(DecTeamCtl, mbar), 0);
     };
 
+    // The ragged last tile (raw; entry 0 when its chunk is absent): by the team that is the last to get
+    // a ticket anyway, before its loop.
+    if (g.tail_len && blockIdx.x == gridDim.x - 1u && team == TEAMS - 1u && tab16_of()[g.n_full_tiles] == 0xFFFFu) {
+        const uint32_t t = g.n_full_tiles;
+        const unsigned char* src = payload_of() + *reinterpret_cast<const unsigned long long*>(dir_of() + 16ull * chunk_of(g, t)) + ws.rel[t];
+        // (leaf mode: the tile has a slot of its own in the side buffer)
+        if (MODE != 1) copy_ragged_tile(LEAVES ? reinterpret_cast<unsigned char*>(ws.tptr[t]) : dst + (uint64_t)t * kTile, src, g.tail_len, tt);
+        if (MODE != 2) {
+            const uint32_t v = ragged_tile_digest(S, g, stage, src, tc->wdig[0], team, tt);
+            if (tt == 0) ws.dig[t] = v;
+            team_bar(team);
+        }
+    }
     if (leader) {
         mbar_init(&tc->mbar, 1);
         lookup(claim(), &tc->slot[0]);
@@ -496,7 +510,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     uint32_t t_done = kNone;           // tile whose digest parts wait in wdig[(it - 1) & 1]
     for (uint32_t it = 0;; it++) {
         const uint32_t t = lds_now<offsetof(DecTeamCtl, slot)>(tc_s + 16u * (it & 3u));
-        if (t >= g.n_tiles) {
+        if (t >= g.n_full_tiles) {
             team_bar(team);
             if (tt == 32u && t_done != kNone) ws.dig[t_done] = xor8(TC()->wdig[(it & 1u) ^ 1u]);
             break;
@@ -678,7 +692,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         uint32_t t_look = kNone;           // warps 0 and 3: the tile claimed a step ago (two tiles ahead)
         if (leader) {                      // its table entry and offsets
             t_look = TC()->slot[(it + 2u) & 3u].t;
-            if (t_look < g.n_tiles) {
+            if (t_look < g.n_full_tiles) {
                 cp_async16(&TC()->in_tab, tab16_of() + (t_look & ~7u));
                 cp_async16(&TC()->in_rel, ws.rel + (t_look & ~3u));
                 cp_async16(&TC()->in_dir, dir_of() + 16ull * chunk_of(g, t_look));
@@ -687,7 +701,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         }
         if (tt == 96u) {                   // the ticket of the tile three ahead
             t_look = TC()->slot[(it + 2u) & 3u].t;
-            if (t_look < g.n_tiles) l_tk = claim();
+            if (t_look < g.n_full_tiles) l_tk = claim();
         }
 
         // ---- phase 2: unpack, store, checksum
@@ -699,15 +713,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                 o_leaf = v.x | ((unsigned long long)v.y << 32);
             }
             unsigned char* o = LEAVES ? reinterpret_cast<unsigned char*>(o_leaf) : dst + (uint64_t)t * kTile;
-            bool fold = (ew >> 16) != 0;
-            if (e == 0xFFFFu) {
-                const unsigned char* src = payload_of() + TC()->slot[it & 3u].src;
-                const uint32_t len = g.tail_len;
-                // (leaf mode: the ragged tile has a slot of its own in the side buffer)
-                if (MODE != 1) for (uint32_t i = tt; i < len; i += kTeamThreads) o[i] = src[i];
-                if (MODE != 2) load_tile_words_guarded(src, len, fold, warp, lane, w);
-                fold = false;
-            }
+            const bool fold = (ew >> 16) != 0;
             // where the decoded words go: word i of this lane to byte 128 i of its warp's 2 KiB.  In leaf
             // mode a tile may start off a four-byte boundary inside its leaf; it then takes halfword
             // or byte stores instead of the plain 32-bit one.
@@ -768,8 +774,8 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                     have_digest = true;
                 }
             } else if (decoded) {
-                // raw, zero and constant tiles and the ragged tail: the sixteen words are there already
-                if (MODE != 1 && e != 0xFFFFu) {
+                // raw, zero and constant tiles: the sixteen words are there already
+                if (MODE != 1) {
 #pragma unroll
                     for (int i = 0; i < 16; i++) put(i, w[i]);
                 }
@@ -785,7 +791,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
             else rest_of_step(std::integral_constant<uint32_t, 2u>());
         }
         t_done = have_digest ? t : kNone;
-        if (leader && t_look < g.n_tiles) {
+        if (leader && t_look < g.n_full_tiles) {
             cp_async_wait_all();
             DecSlot* s2 = &TC()->slot[(it + 2u) & 3u];
             const uint32_t l_e = reinterpret_cast<const volatile unsigned short*>(&TC()->in_tab)[t_look & 7u];

@@ -420,31 +420,62 @@ __device__ __forceinline__ void read_staged_words_at(uint32_t stage_s, uint32_t 
     w[12] = lds_now<1536>(p); w[13] = lds_now<1664>(p); w[14] = lds_now<1792>(p); w[15] = lds_now<1920>(p);
 }
 
-// One 32-bit word of a tile of `len` (1..16384) real bytes that is right-aligned in a virtual
-// tile whose leading 16384 - len bytes are zero (leading zeros do not change a zero-start CRC
-// state).  `vb` is the word's byte offset inside the virtual tile.  When `first_in_chunk`, the
-// chunk's first four bytes are complemented (the all-ones CRC init).  Rare path (one tile per
-// call at most), kept out of line.
-__device__ __noinline__ uint32_t guarded_word(const unsigned char* tile, uint32_t len, bool first_in_chunk, uint32_t vb)
+// ---- the ragged last tile of a cache: `len` (1..16383) real bytes, stored raw ----
+// One team handles it outside the kernels' loops, which then know full tiles only.  For the checksum
+// it goes into the team's stage right-aligned in a virtual tile whose leading 16384 - len bytes are
+// zero (leading zeros do not change a zero-start CRC state) and is read from there like any other
+// tile.  When `first_in_chunk`, the chunk's first four bytes are complemented (the all-ones CRC
+// init).  `tile` is four-byte aligned; no byte behind its end is read.  A thread takes sixteen
+// words and has all of its loads under way together: the tile is one trip to memory long, where
+// fetching its words one after the other, byte by byte, took 8 us more (decode of 8 MB: 36.8 us, 28.7
+// now), which every call waited for at its end.
+__device__ __forceinline__ void stage_ragged_tile(unsigned char* stage, const unsigned char* __restrict__ tile, uint32_t len,
+                                                  bool first_in_chunk, uint32_t tt)
 {
-    const int64_t pad = (int64_t)kTile - (int64_t)len;
-    uint32_t word = 0;
-    for (int j = 0; j < 4; j++) {
-        const int64_t rb = (int64_t)vb + j - pad;
-        if (rb >= 0) {
-            uint32_t b = tile[rb];
-            if (first_in_chunk && rb < 4) b ^= 0xFFu;
-            word |= b << (8 * j);
-        }
+    const int32_t pad = (int32_t)(kTile - len);
+    const uint32_t off = len & 3u;                     // (a virtual word starts at real byte 4 q - pad, off modulo four)
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(tile);
+    uint32_t v[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        const int32_t rb = 4 * (int32_t)(tt + kTeamThreads * i) - pad;      // the word's first real byte
+        const int32_t a = rb >> 2;
+        uint32_t lo = 0, hi = 0;
+        if (a >= 0) lo = __ldcg(p + a);
+        if (off && a >= -1 && 4 * (a + 2) <= (int32_t)len) hi = __ldcg(p + a + 1);
+        v[i] = __funnelshift_r(lo, hi, 8u * off);
     }
-    return word;
+    if (off && tt == kTeamThreads - 1u) {              // the last word: its last bytes are not a whole word of the tile
+        const uint32_t at = len & ~3u;
+        for (uint32_t j = 0; j < off; j++) v[15] |= (uint32_t)tile[at + j] << (8u * (4u - off + j));
+    }
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        const uint32_t q = tt + kTeamThreads * i;
+        const int32_t rb = 4 * (int32_t)q - pad;
+        if (first_in_chunk && rb > -4 && rb < 4)
+            v[i] ^= rb < 0 ? 0xFFFFFFFFu << (8 * -rb) : 0xFFFFFFFFu >> (8 * rb);
+        reinterpret_cast<uint32_t*>(stage)[q] = v[i];
+    }
+    // (the stage's next content comes by a bulk copy, which is another proxy)
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-__device__ __forceinline__ void load_tile_words_guarded(const unsigned char* tile, uint32_t len, bool first_in_chunk,
-                                                        uint32_t warp, uint32_t lane, uint32_t (&w)[kWordsPerLane])
+// The same tile's `len` bytes from one 16-byte aligned place to another, by a team's 256 threads.
+__device__ __forceinline__ void copy_ragged_tile(unsigned char* __restrict__ dst, const unsigned char* __restrict__ src, uint32_t len,
+                                                 uint32_t tt)
 {
+    uint4 v[4];
 #pragma unroll
-    for (int i = 0; i < 16; i++) w[i] = guarded_word(tile, len, first_in_chunk, (warp * 16 + i) * 128 + lane * 4);
+    for (int i = 0; i < 4; i++) {
+        v[i] = make_uint4(0, 0, 0, 0);
+        if (16u * (tt + kTeamThreads * i) + 16u <= len) v[i] = __ldcg(reinterpret_cast<const uint4*>(src) + tt + kTeamThreads * i);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+        if (16u * (tt + kTeamThreads * i) + 16u <= len) reinterpret_cast<uint4*>(dst)[tt + kTeamThreads * i] = v[i];
+    const uint32_t at = (len & ~15u) + tt;
+    if (at < len) dst[at] = src[at];
 }
 
 // CRC32C of a short run computed byte by byte (chunks shorter than four bytes).

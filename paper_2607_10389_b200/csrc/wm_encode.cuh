@@ -210,11 +210,6 @@ struct EncTeamCtl {
 };
 static_assert(sizeof(EncTeamCtl) % 16 == 0, "team control block keeps 16-byte alignment");
 
-__device__ __forceinline__ uint32_t tile_left(const Geo& g, uint32_t t)      // bytes of a ragged tile
-{
-    return (uint32_t)(g.nbytes - (uint64_t)t * kTile);
-}
-
 __device__ __forceinline__ void stg_u8(void* p, uint32_t v)
 {
     asm volatile("st.global.cs.u8 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -354,10 +349,10 @@ __device__ __forceinline__ uint32_t ent_parse_value(uint32_t buf, uint32_t s, ui
 // of slack that is rare, and it only delays: the teams that hold earlier tiles never depend
 // on this one.
 // A tile as a team passes it round: its number in the low 22 bits, kQFirst when it is the first
-// tile of its chunk, kQPresent when its chunk is encoded; kQNone: no tile.  Leaf mode adds, in
-// bits 22-25, how many bytes above a 16-byte boundary the tile starts.  (The codec takes caches
-// of at most 2^21 tiles, so a number never reaches kQNone or the other fields.)
-constexpr uint32_t kQPresent = 1u << 31, kQFirst = 1u << 30, kQTile = (1u << 22) - 1u, kQNone = kQTile;
+// tile of its chunk; the top bit alone (kQNone): no tile.  Leaf mode adds, in bits 22-25, how many
+// bytes above a 16-byte boundary the tile starts.  (The codec takes caches of at most 2^21 tiles.)
+// Only full tiles are passed round: the ragged last tile is the scanner's block's business.
+constexpr uint32_t kQNone = 1u << 31, kQFirst = 1u << 30, kQTile = (1u << 22) - 1u;
 constexpr uint32_t kQOffShift = 22;
 // Marks in a team's width table: on a warp's first entry, all 2 KiB of the warp's rows are zero;
 // as the sum of the widths, the tile is all zero.
@@ -370,18 +365,43 @@ constexpr uint32_t kSumEnt = 0x10000u;
 // The tile behind ticket k.  Without a mask tickets are tile numbers.  With one, only the tiles of
 // present chunks are claimed: ticket k is tile k mod tiles_per_chunk of the (k / tiles_per_chunk)-th
 // present chunk (plist, ascending, written by k_encode_init), so placement runs over tickets and a
-// sparse mask costs nothing for what it leaves out.
+// sparse mask costs nothing for what it leaves out.  n_hot: tickets of full tiles.
 template <bool MASKED>
-__device__ __forceinline__ uint32_t describe_tile(const Geo& g, const uint32_t* __restrict__ plist, uint32_t n_tickets, uint32_t k)
+__device__ __forceinline__ uint32_t describe_tile(const Geo& g, const uint32_t* __restrict__ plist, uint32_t n_hot, uint32_t k)
 {
-    if (k >= n_tickets) return kQNone;
+    if (k >= n_hot) return kQNone;
     uint32_t t = k;
     bool first = first_in_chunk(g, k);
     if (MASKED) {
         const uint32_t j = chunk_of(g, k);
         t = plist[j] * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
     }
-    return t | kQPresent | (first ? kQFirst : 0u);
+    return t | (first ? kQFirst : 0u);
+}
+
+// The ragged last tile (ticket k, behind all others), stored raw: by the second team of the scanner's
+// block, beside the scanner.  Nothing follows it, so its length is of no interest to the scanner: the
+// zero published here only asks for the tile's offset.
+__device__ __forceinline__ void encode_ragged_tile(const Smem& S, const Geo& g, const unsigned char* __restrict__ tile, unsigned char* __restrict__ wire,
+                                                uint64_t wire_cap, const Ws& ws, uint32_t k, unsigned char* slot, uint32_t* wdig)
+{
+    const uint32_t tt = threadIdx.x % kTeamThreads, t = g.n_full_tiles;
+    __shared__ unsigned long long s_excl;
+    if (tt == 0) st_relaxed_u32(ws.lbk + k, kFlagA);
+    const uint32_t v = ragged_tile_digest(S, g, slot, tile, wdig, 1, tt);
+    if (tt == 0) {
+        ws.dig[t] = v;
+        s_excl = wait_prefix(ws.lbk, k, ws.ctrl, g.wait_ns);
+    }
+    team_bar(1);
+    const unsigned long long excl = s_excl;
+    if (tt == 0) {
+        reinterpret_cast<uint16_t*>(wire + 64 + 16ull * g.n_chunks)[t] = 0xFFFFu;
+        if (first_in_chunk(g, t)) *reinterpret_cast<unsigned long long*>(wire + 64 + 16ull * chunk_of(g, t)) = excl;
+        ws.ctrl->payload_total = excl + g.tail_len;
+        if (excl + g.tail_len > wire_cap - g.meta_end) atomicOr(&ws.ctrl->err, 1u);
+    }
+    if (excl + g.tail_len <= wire_cap - g.meta_end) copy_ragged_tile(wire + g.meta_end + excl, tile, g.tail_len, tt);
 }
 
 template <int TEAMS, bool MASKED, bool LEAVES, bool ZEROS, bool ENT = false>
@@ -400,10 +420,21 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     if (LEAVES && (ld_volatile_u32(&ws.ctrl->err) & 8u)) return;      // the leaf table was rejected
     if (threadIdx.x == 0) s_scanner = atomicCAS(&ws.ctrl->scan_lock, 0u, 1u) == 0u;
     __syncthreads();
+    // Tickets: all of them, and those of full tiles (the teams').  The ragged last tile of the cache,
+    // when its chunk is present, is the last ticket.
+    const uint32_t n_tickets = MASKED ? ld_volatile_u32(&ws.ctrl->n_tickets) : g.n_tiles;
+    const bool ragged = g.tail_len != 0u && (!MASKED || dirty[g.n_chunks - 1u] != 0);
+    const uint32_t n_hot = ragged ? n_tickets - 1u : n_tickets;
     if (s_scanner) {
         uint32_t* win = reinterpret_cast<uint32_t*>(S.take(2048));      // 512 entries
+        unsigned char* slot = S.take(kTile);
+        uint32_t* wdig = reinterpret_cast<uint32_t*>(S.take(32));
+        if (!S.ok) { if (threadIdx.x == 0) atomicOr(&ws.ctrl->err, 4u); return; }
         // (test hook: with the scanner left out no offset is ever handed out, and the owners' waits run out)
-        if (threadIdx.x < 32 && win && !(g.inject & kInjectNoScanner)) scan_tile_lengths(ws.lbk, MASKED ? ld_volatile_u32(&ws.ctrl->n_tickets) : g.n_tiles, threadIdx.x, ws.ctrl, win, g.wait_ns);
+        if (threadIdx.x < 32 && !(g.inject & kInjectNoScanner)) scan_tile_lengths(ws.lbk, n_tickets, threadIdx.x, ws.ctrl, win, g.wait_ns);
+        if (ragged && threadIdx.x / kTeamThreads == 1u)
+            encode_ragged_tile(S, g, LEAVES ? reinterpret_cast<const unsigned char*>(ws.tptr[g.n_full_tiles]) : cache + (uint64_t)g.n_full_tiles * kTile,
+                               wire, wire_cap, ws, n_tickets - 1u, slot, wdig);
         return;
     }
     const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
@@ -453,10 +484,8 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     const bool leader = (tt == 0);
     uint32_t phase = 0;                // parity of the stage's next completion
 
-    auto is_tile = [](uint32_t q) { return (q & kQTile) != kQNone; };
-    auto is_hot = [&](uint32_t q) { return q >= kQPresent && (q & kQTile) < g.n_full_tiles; };   // present and full
+    auto is_tile = [](uint32_t q) { return (int32_t)q >= 0; };
     // (the placement words are indexed by ticket: with a mask that is the ring slot's ticket, else the tile number)
-    const uint32_t n_tickets = MASKED ? ld_volatile_u32(&ws.ctrl->n_tickets) : g.n_tiles;
     auto place_of = [&](uint32_t slot, uint32_t t) { return MASKED ? tc->kring[slot] : t; };
     auto publish_len = [&](uint32_t slot, uint32_t t, uint32_t len) { st_relaxed_u32(ws.lbk + place_of(slot, t), kFlagA | (len / kUnit)); };
     // where tile t lives: its address in the flat cache, or (leaf mode) the address that k_leaf_map wrote
@@ -467,13 +496,13 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     // off a 16-byte boundary; the copy then starts at the boundary below and takes 16 bytes more
     // (k_leaf_map saw to it that they belong to the leaf); the readers shift by the remainder.
     auto start_copy = [&](uint32_t q, unsigned long long src) {
-        if (!is_hot(q)) return;
+        if (!is_tile(q)) return;
         const unsigned long long a = LEAVES ? src & ~15ull : src;
         bulk_load(stage, reinterpret_cast<const void*>(a), (LEAVES && a != src) ? kTile + 16u : kTile, &tc->mbar, pol_once);
     };
     // leaf mode, handing a claimed tile on: its word carries the start's remainder
     auto with_mark = [](uint32_t q, unsigned long long addr) {
-        return (!LEAVES || (q & kQTile) == kQNone) ? q : q | (((uint32_t)addr & 15u) << kQOffShift);
+        return (!LEAVES || (int32_t)q < 0) ? q : q | (((uint32_t)addr & 15u) << kQOffShift);
     };
 
     // Tiles in flight, oldest first: X (packed in this step), V, W (waiting for their offsets),
@@ -500,9 +529,9 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     if (leader) {
         mbar_init(&tc->mbar, 1);
         const uint32_t k0 = next_ticket(ws.ctrl);
-        const uint32_t q0 = describe_tile<MASKED>(g, ws.plist, n_tickets, k0);
+        const uint32_t q0 = describe_tile<MASKED>(g, ws.plist, n_hot, k0);
         const uint32_t k1 = is_tile(q0) ? next_ticket(ws.ctrl) : 0xFFFFFFFFu;
-        const uint32_t q1 = is_tile(q0) ? describe_tile<MASKED>(g, ws.plist, n_tickets, k1) : kQNone;
+        const uint32_t q1 = is_tile(q0) ? describe_tile<MASKED>(g, ws.plist, n_hot, k1) : kQNone;
         claiming = is_tile(q1);
         if (MASKED) { tc->kring[3] = k0; tc->kring[4] = k1; }      // the slots in which they will be measured
         tc->next[0] = q0;
@@ -514,17 +543,17 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             tc->nptr[1] = is_tile(q1) ? tile_src(q1 & kQTile) : 0ull;
             tc->next[0] = with_mark(q0, tc->nptr[0]);
             tc->next[1] = with_mark(q1, tc->nptr[1]);
-            if (claiming) { kA = next_ticket(ws.ctrl); qA = describe_tile<MASKED>(g, ws.plist, n_tickets, kA); claiming = is_tile(qA); }
+            if (claiming) { kA = next_ticket(ws.ctrl); qA = describe_tile<MASKED>(g, ws.plist, n_hot, kA); claiming = is_tile(qA); }
         }
-        if (kLateList && claiming) { kA = next_ticket(ws.ctrl); claiming = haveA = kA < n_tickets; }
+        if (kLateList && claiming) { kA = next_ticket(ws.ctrl); claiming = haveA = kA < n_hot; }
     }
     team_bar(team);
     qY = tc->next[0];
     if (leader) start_copy(qY, LEAVES ? tc->nptr[0] : tile_src(qY & kQTile));
 
     uint32_t trouble = 0;              // sticky: the image does not fit
-    while (((qX & qV & qW & qY) & kQTile) != kQNone) {
-        const bool hotY = is_hot(qY);
+    while (is_tile(qX & qV & qW & qY)) {
+        const bool hotY = is_tile(qY);
         if (hotY) {
             wait_for_copy<!ENT>(&tc->mbar, phase, g.wait_ns, ws.ctrl);
             phase ^= 1u;
@@ -550,7 +579,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         // (half a step later than the last-arriving warp could have, which the three steps of slack
         // before the tile is packed absorb; but no warp waits for a counter in the measuring step
         // and the sum is off the path of whichever warp was slowest there).
-        if (warp == 6u && is_hot(qW)) {
+        if (warp == 6u && is_tile(qW)) {
             const uint32_t slW = (sl + 2u) & 7u;
             const uint32_t wt = tc->wtab[slW][lane];
             const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u);
@@ -588,7 +617,6 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
 
         // ---- Y: digest, exponent ranges, length out, words parked
         const uint32_t slY = (sl + 3u) & 7u;
-        const uint32_t tYn = qY & kQTile;
         if (hotY) {
             const uint32_t v = tile_digest_part(S, d, (qY & kQFirst) != 0, warp, lane);
             // From here on the words are kept rotated left by one bit: each half then reads
@@ -652,21 +680,11 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 if (ENT) tc->etab[slY][warp] = ent_w;
             }
             tmem_store16(tmem_warp + 16u * (step & 3u), d);
-        } else if (is_tile(qY)) {
-            // rare: a tile of an absent chunk (length 0) or the ragged last tile (stored raw)
-            const bool present = qY >= kQPresent;
-            if (tt == 0) publish_len(slY, tYn, present ? tile_left(g, tYn) : 0u);
-            if (present) {
-                // (leaf mode: the ragged tile has a slot of its own in the side buffer)
-                load_tile_words_guarded(reinterpret_cast<const unsigned char*>(tile_src(tYn)), tile_left(g, tYn), (qY & kQFirst) != 0, warp, lane, d);
-                const uint32_t v = tile_digest_part(S, d, false, warp, lane);
-                if (lane == 0) tc->wdig[slY][warp] = v;
-            }
         }
 
         // ---- X: its words back from tensor memory, packed straight into the wire image
         const uint32_t tXn = qX & kQTile;
-        if (is_hot(qX)) {
+        if (is_tile(qX)) {
             tmem_load16(tmem_warp + 16u * ((step + 1u) & 3u), d);
             const uint32_t Smark = tc->ssum[sl];
             const bool ent_form = ENT && (Smark & kSumEnt) != 0u;
@@ -792,39 +810,22 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
 #pragma unroll
                 for (int i = 0; i < 16; i++) st_stream_u32(q + i * 128, __funnelshift_r(d[i], d[i], 1));
             }
-        } else if (qX >= kQPresent) {
-            // rare: the ragged last tile, stored raw
-            const uint32_t enc_len = tile_left(g, tXn);
-            if (exclX + enc_len > room) {
-                trouble |= 1u;
-            } else {
-                const unsigned char* src = reinterpret_cast<const unsigned char*>(tile_src(tXn));
-                unsigned char* dst = payload + exclX;
-                for (uint32_t i = tt; i < enc_len; i += kTeamThreads) dst[i] = src[i];
-            }
         }
 
         // What is left to note about X is done by two other warps' first lanes (the leader's
         // warp is the one the team waits for): the digest by warp 1; the table entry, where its
         // chunk starts and the total by warp 7 (not warp 4: warps w and w + 4 issue through the same
         // scheduler, and warp 4 would share the end of the step with the leader's hand-over).
-        if (tt == 32u && qX >= kQPresent && is_tile(qX)) ws.dig[tXn] = xor8(tc->wdig[sl]);
+        if (tt == 32u && is_tile(qX)) ws.dig[tXn] = xor8(tc->wdig[sl]);
         if (tt == 224u && is_tile(qX)) {
-            uint32_t entry = 0, enc_len = 0;
-            if (qX >= kQPresent) {
-                if (tXn < g.n_full_tiles) {
-                    const uint32_t Ssum = tc->ssum[sl];
-                    if (ENT && (Ssum & kSumEnt)) {
-                        enc_len = ent_tile_bytes(Ssum & 0xFFFFu);
-                        entry = 0x8000u | (enc_len / 32u);
-                    } else {
-                        entry = Ssum <= 253u ? 258u + Ssum : (ZEROS && Ssum == kSumZeroTile) ? 1u : (ZEROS && Ssum == kSumConstTile) ? 2u : 512u;
-                        enc_len = (ZEROS && entry <= 2u) ? 32u * (entry - 1u) : 32u * entry;
-                    }
-                } else {
-                    entry = 0xFFFFu;
-                    enc_len = tile_left(g, tXn);
-                }
+            uint32_t entry, enc_len;
+            const uint32_t Ssum = tc->ssum[sl];
+            if (ENT && (Ssum & kSumEnt)) {
+                enc_len = ent_tile_bytes(Ssum & 0xFFFFu);
+                entry = 0x8000u | (enc_len / 32u);
+            } else {
+                entry = Ssum <= 253u ? 258u + Ssum : (ZEROS && Ssum == kSumZeroTile) ? 1u : (ZEROS && Ssum == kSumConstTile) ? 2u : 512u;
+                enc_len = (ZEROS && entry <= 2u) ? 32u * (entry - 1u) : 32u * entry;
             }
             tile_tab[tXn] = (uint16_t)entry;
             if (qX & kQFirst) *reinterpret_cast<unsigned long long*>(dir + 16ull * chunk_of(g, tXn)) = exclX;
@@ -834,16 +835,16 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             uint32_t qn = kQNone;
             if (haveA) {
                 const uint32_t j = chunk_of(g, kA);
-                qn = (plA * g.tiles_per_chunk + (kA - j * g.tiles_per_chunk)) | kQPresent | (first_in_chunk(g, kA) ? kQFirst : 0u);
+                qn = (plA * g.tiles_per_chunk + (kA - j * g.tiles_per_chunk)) | (first_in_chunk(g, kA) ? kQFirst : 0u);
             }
             tc->next[par] = qn;
             tc->kring[(sl + 5u) & 7u] = kA;
-            haveA = claiming && tk < n_tickets;
+            haveA = claiming && tk < n_hot;
             claiming = haveA;
             kA = tk;
         } else if (leader) {
             uint32_t qn2 = kQNone;
-            if (claiming) { qn2 = describe_tile<MASKED>(g, ws.plist, n_tickets, tk); claiming = is_tile(qn2); }
+            if (claiming) { qn2 = describe_tile<MASKED>(g, ws.plist, n_hot, tk); claiming = is_tile(qn2); }
             // (the tile handed over now is measured two steps on, in ring slot sl + 5)
             if (LEAVES) {              // hand over the tile whose address arrived during this step
                 tc->next[par] = with_mark(qA, pA);

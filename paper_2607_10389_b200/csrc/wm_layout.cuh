@@ -295,6 +295,22 @@ __device__ __forceinline__ uint32_t xor8(const uint32_t* p)
     return p[0] ^ p[1] ^ p[2] ^ p[3] ^ p[4] ^ p[5] ^ p[6] ^ p[7];
 }
 
+// The digest of the cache's ragged last tile, by one whole team before its loop (its stage is empty):
+// the result is in thread 0.  wdig: eight words of shared memory.
+__device__ __forceinline__ uint32_t ragged_tile_digest(const Smem& S, const Geo& g, unsigned char* stage, const unsigned char* __restrict__ tile,
+                                                       uint32_t* wdig, uint32_t team, uint32_t tt)
+{
+    const uint32_t warp = tt / 32, lane = tt % 32;
+    stage_ragged_tile(stage, tile, g.tail_len, first_in_chunk(g, g.n_full_tiles), tt);
+    team_bar(team);
+    uint32_t w[kWordsPerLane];
+    read_staged_words(stage, warp, lane, w);
+    const uint32_t v = tile_digest_part(S, w, false, warp, lane);
+    if (lane == 0) wdig[warp] = v;
+    team_bar(team);
+    return tt == 0 ? xor8(wdig) : 0u;
+}
+
 // First byte of chunk c: in the flat buffer, or (leaf mode, flat == nullptr) where the chunk's
 // first tile is (for the only chunk ever asked for, the ragged last one, that is its slot in the
 // side buffer).  Only chunks shorter than four bytes are read through it.

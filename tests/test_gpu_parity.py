@@ -428,3 +428,33 @@ def test_constant_tiles_match_the_oracle(layout):
         want_bad = oracle.decode_verify(bad, n, chunk, dst=old, dst_crc=want_crc)[2]
         _, _, rb = g.decode(to_dev(bad), bad.size, dst=old, dst_crc=want_crc)
         assert same_result(rb, want_bad) and want_bad.status_name == "ERR_CHUNK_CRC"
+
+
+@pytest.mark.parametrize("full", [0, 3, 4, 7, 148 * 4, 148 * 4 + 1])       # full tiles: none, around a block's four teams, around all teams
+@pytest.mark.parametrize("tail", [5, 14, 4096, TILE - 3])
+def test_ragged_last_tile_wherever_it_falls(G, full, tail):
+    """The ragged tile is handled outside the loops over full tiles: present, absent (its chunk is not in
+    the mask) and alone, with bytes behind the destination that must stay as they are."""
+    from gpu_util import same_result
+    n, chunk = full * TILE + tail, 2 * TILE
+    a = _special_cache(n, n)
+    g = G(n, chunk)
+    nc = g.nc
+    src = torch.from_numpy(a).cuda()
+    assert np.array_equal(g.checksum(src), oracle.checksum(a, chunk))
+    masks = [None, np.ones(nc, np.uint8), np.array([c % 3 == 0 and c + 1 < nc for c in range(nc)], np.uint8),
+             np.array([c + 1 == nc for c in range(nc)], np.uint8)]
+    old = oracle.checksum(a, chunk)
+    for mask in masks:
+        want_wire, want_crc, want = oracle.encode(a, chunk, dirty=mask, crc_in=old)
+        wire, crc, res, wire_dev = g.encode(src, dirty=mask, crc_in=old)
+        assert same_result(res, want) and np.array_equal(crc, want_crc) and np.array_equal(wire[: res.wire_len], want_wire)
+        dst = torch.full((n + 48,), 0x5A, dtype=torch.uint8, device="cuda")
+        dst[:n] = src
+        if mask is not None:
+            for c in np.nonzero(mask)[0]:
+                dst[c * chunk: min((c + 1) * chunk, n)] = 0x11
+        dcrc = torch.from_numpy(old.view(np.int32).copy()).cuda()
+        from paper_2607_10389_b200 import binding as wm
+        wm.wm_decode_verify(wire_dev, res.wire_len, dst[:n], chunk, dcrc, g.ws, g.res)
+        assert wm.read_result(g.res).ok and torch.equal(dst[:n], src) and bool((dst[n:] == 0x5A).all())
