@@ -322,3 +322,26 @@ def test_append_only_schedule_on_the_gpu_matches_the_oracle_step_by_step():
             assert r.payload_bytes == 0
         wm.wm_decode_verify_opt(wire, r.wire_len, dst, chunk, dcrc, ws, res, 0)
         assert wm.read_result(res).ok and torch.equal(dst, cur) and torch.equal(dcrc, crc)
+
+
+@gpu
+@pytest.mark.parametrize("before", [1, 2, 3, 4 * TILE + 6])        # where the run of small leaves begins, modulo four
+def test_runs_of_every_length_and_alignment_through_the_side_buffer(before):
+    """Leaves of 1 to 59 bytes, one behind the other, then cuts at odd places of further tiles: the pieces of
+    the tiles that cross leaves have every length and every alignment of either end."""
+    sizes = list(range(1, 60)) + [TILE + 1, TILE + 2, TILE + 3, TILE + 5]
+    cuts = _flags(before, sizes)
+    nbytes = before + sum(sizes) + TILE + 7
+    torch, wm, flat, leaves = _setup(nbytes, 2 * TILE, cuts, seed=before, byte_cuts=True)
+    nc, ws, res = wm.num_chunks(nbytes, 2 * TILE), wm.new_workspace(nbytes, 2 * TILE), wm.new_result()
+    crc, dcrc = (torch.zeros(nc, dtype=torch.int32, device="cuda") for _ in range(2))
+    wire = torch.zeros(wm.wire_bound(nbytes, 2 * TILE), dtype=torch.uint8, device="cuda")
+    wm.wm_encode_leaves(wm.make_leaf_table(leaves), nbytes, 2 * TILE, None, crc, wire, ws, res)
+    r = wm.read_result(res)
+    want, want_crc, _ = oracle.encode(flat.cpu().numpy(), 2 * TILE)
+    assert r.ok and np.array_equal(wire[: r.wire_len].cpu().numpy(), want)
+    dst = [torch.full((x.numel() + 16,), 0xC3, dtype=torch.uint8, device="cuda") for x in leaves]
+    table = wm.make_leaf_table([b[: x.numel()] for b, x in zip(dst, leaves)])
+    wm.wm_decode_verify_leaves(wire, r.wire_len, table, nbytes, 2 * TILE, dcrc, ws, res)
+    assert wm.read_result(res).ok and np.array_equal(dcrc.cpu().numpy().view(np.uint32), want_crc)
+    assert all(torch.equal(b[:-16], x) and bool((b[-16:] == 0xC3).all()) for b, x in zip(dst, leaves))
