@@ -48,22 +48,34 @@ struct Smem {
     }
 };
 
-// Copy the table image into shared memory (whole block; ends with __syncthreads).
+// Put the table image into shared memory (whole block; ends with __syncthreads).  A block fetches
+// 24 KiB and makes the lanes' copies of G itself: fetching the finished image, 144 KiB for each of
+// 148 blocks at once, is 21 MB out of L2 in front of every kernel, and the caches that are small
+// enough to notice consist of such kernels.
 __device__ __forceinline__ Smem setup_smem(unsigned char* smem, const Tables* __restrict__ tab)
 {
     Smem s;
     s.ok = true;
     s.free = smem + kImgBytes; s.free_bytes = kDynSmem - kImgBytes;
-    const uint4* src = reinterpret_cast<const uint4*>(tab->image);
+    const uint32_t lane = threadIdx.x & 31u;
     uint4* dst = reinterpret_cast<uint4*>(smem);
-    for (uint32_t i = threadIdx.x; i < kImgBytes / 16; i += blockDim.x) dst[i] = src[i];
+    for (uint32_t e0 = (threadIdx.x / 32u) * 32u; e0 < 1024u; e0 += blockDim.x) {      // 32 entries per warp
+        const uint32_t x = (&tab->G[0][0])[e0 + lane];
+#pragma unroll
+        for (uint32_t j = 0; j < 8u; j++) {            // four entries of 128 bytes at a time
+            const uint32_t v = __shfl_sync(0xFFFFFFFFu, x, 4u * j + lane / 8u);
+            dst[(e0 + 4u * j) * (kImgEntry / 16u) + lane] = make_uint4(v, v, v, v);
+        }
+    }
+    const uint4* nk = reinterpret_cast<const uint4*>(&tab->NK[0][0][0]);
+    for (uint32_t i = threadIdx.x; i < (kImgBytes - kImgNK) / 16u; i += blockDim.x) dst[kImgNK / 16u + i] = nk[i];
     uint32_t* nw = reinterpret_cast<uint32_t*>(s.take(8 * 8 * 16 * 4));
     if (nw) {
         const uint32_t* gNW = &tab->NW[0][0][0];
         for (uint32_t i = threadIdx.x; i < 8 * 8 * 16; i += blockDim.x) nw[i] = gNW[i];
     }
     s.NW = nw;
-    s.L = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x & 31u) * 4u;
+    s.L = (uint32_t)__cvta_generic_to_shared(smem) + lane * 4u;
     __syncthreads();
     return s;
 }
@@ -184,15 +196,12 @@ __device__ __forceinline__ uint32_t warp_place(const Smem& S, uint32_t digest, u
 
 // ---- the same digest with small tables, for kernels that see a few hundred kilobytes ----
 // Copying the 144 KiB lane-replicated image costs more than such a kernel's whole work.  Here
-// the chain uses one copy of the four byte tables (4 KiB in shared memory, taken from lane 0's
-// column of the image; lookups may collide on a bank) and the two once-per-tile steps read the
+// the chain uses one copy of the four byte tables (4 KiB in shared memory; lookups may collide on a
+// bank) and the two once-per-tile steps read the
 // nibble tables straight from global memory.  Same result as warp_block_digest + warp_place.
 __device__ __forceinline__ void load_small_chain_tables(uint32_t* sG, const Tables* __restrict__ tab)
 {
-    for (uint32_t i = threadIdx.x; i < 1024; i += blockDim.x) {
-        const uint32_t k = i >> 8, b = i & 255u;
-        sG[i] = tab->image[(k * kImgTable + b * kImgEntry) / 4u];
-    }
+    for (uint32_t i = threadIdx.x; i < 1024; i += blockDim.x) sG[i] = (&tab->G[0][0])[i];
     __syncthreads();
 }
 __device__ __forceinline__ uint32_t tile_digest_part_small(const uint32_t* sG, const Tables* __restrict__ tab,
@@ -208,7 +217,7 @@ __device__ __forceinline__ uint32_t tile_digest_part_small(const uint32_t* sG, c
     uint32_t r = 0;
 #pragma unroll
     for (uint32_t n = 0; n < 8; n++)
-        r ^= __ldg(&tab->image[(kImgNK + n * kImgNibble + ((x >> (4u * n)) & 15u) * kImgEntry) / 4u + lane]);
+        r ^= __ldg(&tab->NK[n][(x >> (4u * n)) & 15u][lane]);
     const uint32_t digest = __reduce_xor_sync(0xFFFFFFFFu, r);
     uint32_t v = 0;
     if (lane < 8) v = __ldg(&tab->NW[warp][lane][(digest >> (4 * lane)) & 15u]);

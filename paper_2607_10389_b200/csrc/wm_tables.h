@@ -16,13 +16,15 @@ constexpr uint32_t kPolyZlib = 0xEDB88320u;        // CRC-32 of zlib, an option 
 // lane, so the address of entry v is base + 128 v + 4 lane, one integer dot product of the word that
 // holds v (see chain_step).
 //   G  : table k at k * kImgTable, 256 entries: G[k][b]
-//   NK : array n at kImgNK + n * kImgNibble, 16 entries: entry v is NK[lane][n][v]
+//   NK : array n at kImgNK + n * kImgNibble, 16 entries: entry v is NK[n][v][lane]
+// In device memory the G tables are single (4 KiB); a block makes the lanes' copies itself.
 constexpr uint32_t kImgEntry = 128, kImgTable = 256 * kImgEntry, kImgNibble = 16 * kImgEntry;
 constexpr uint32_t kImgNK = 4 * kImgTable, kImgBytes = kImgNK + 8 * kImgNibble;
 
 // Tables shared by all kernels; one copy lives in device memory per device.
 struct Tables {
-    uint32_t image[kImgBytes / 4];   // the shared-memory image described above
+    uint32_t G[4][256];              // G[k][b] = (b << 8k) advanced over 128 bytes (one row stride of the word-strided chain)
+    uint32_t NK[8][16][32];          // NK[n][v][l] = (v << 4n) advanced over 128 - 4l bytes (lane l's place inside its row)
     uint32_t NW[8][8][16];           // NW[w][n][v] = (v << 4n) advanced over 2048 (7 - w) bytes
     uint32_t HT[4][256];             // HT[k][b] = (b << 8k) advanced over 16384 bytes (one tile)
     uint32_t T0[256];                // T0[b]    = b advanced over one byte (the classic table)
@@ -56,21 +58,16 @@ inline uint32_t x_pow_bytes(uint64_t n, uint32_t poly = kPolyReflected)
 inline void build_tables(Tables& t, uint32_t poly = kPolyReflected)
 {
     const uint32_t k128 = x_pow_bytes(128, poly), kTile = x_pow_bytes(16384, poly), k1 = x_pow_bytes(1, poly);
-    // G[k][b] = (b << 8k) advanced over 128 bytes (one row stride of the word-strided chain)
     for (uint32_t k = 0; k < 4; k++)
         for (uint32_t b = 0; b < 256; b++) {
-            const uint32_t g = mulmod(b << (8 * k), k128, poly);
-            uint32_t* dst = t.image + (k * kImgTable + b * kImgEntry) / 4;
-            for (uint32_t l = 0; l < 32; l++) dst[l] = g;
+            t.G[k][b] = mulmod(b << (8 * k), k128, poly);
             t.HT[k][b] = mulmod(b << (8 * k), kTile, poly);
         }
     for (uint32_t b = 0; b < 256; b++) t.T0[b] = mulmod(b, k1, poly);
-    // NK[l][n][v] = (v << 4n) advanced over 128 - 4l bytes (a lane's place inside its row)
     for (uint32_t l = 0; l < 32; l++) {
         const uint32_t kl = x_pow_bytes(128 - 4 * l, poly);
         for (uint32_t n = 0; n < 8; n++)
-            for (uint32_t v = 0; v < 16; v++)
-                t.image[(kImgNK + n * kImgNibble + v * kImgEntry) / 4 + l] = mulmod(v << (4 * n), kl, poly);
+            for (uint32_t v = 0; v < 16; v++) t.NK[n][v][l] = mulmod(v << (4 * n), kl, poly);
     }
     for (uint32_t w = 0; w < 8; w++) {
         const uint32_t kw = x_pow_bytes(2048u * (7 - w), poly);
