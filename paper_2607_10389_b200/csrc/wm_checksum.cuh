@@ -6,9 +6,69 @@ namespace wm {
 
 // ------------------------------------------------------------------ wm_checksum
 
-// Tile digests of the whole cache: static striding over tiles.  Each team owns one 16 KiB stage
-// that bulk copies (TMA) fill; the team takes its 16 words per lane out of the stage, hands
-// the stage to the copy of its next tile and digests from registers meanwhile.
+// Three kernels, by the size of the cache (the rule, with both sides' times, is checksum_any's).
+//   k_chunk_crcs          small caches: a block takes one chunk and folds it itself; one launch
+//   k_tile_digests        a team of eight warps per tile; k_checksum_finish folds the digests
+//   k_tile_digests_stream large caches: a warp per tile; the same finish
+// What bounds the last two is the shared memory the look-ups go through (128 bytes a cycle and SM):
+// a tile is 512 look-ups of a warp in the chain, and with a team per tile 64 more at the ends of its
+// eight warps' chains.
+
+// The cleared control block: the error word in it is the call's outcome (wm_workspace_status).
+__global__ void k_checksum_init(Ctrl* ctrl)
+{
+    grid_dep_launch();
+    if (threadIdx.x < sizeof(Ctrl) / 4) reinterpret_cast<uint32_t*>(ctrl)[threadIdx.x] = 0u;
+}
+
+// Small caches.  A block takes one chunk of at most TEAMS tiles, a tile per team, straight into
+// registers (asked for before the tables are in place), and thread 0 folds the chunk.  Nothing in
+// here waits for a copy, so there is no outcome to report but success.
+template <int TEAMS>
+__global__ void __launch_bounds__(TEAMS * 256, 1)
+k_chunk_crcs(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables* __restrict__ tab, uint32_t* __restrict__ crc_out)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_wdig[TEAMS][8], s_rdig[8], s_dig[TEAMS];
+    const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
+    const uint32_t warp = tt / 32, lane = tt % 32;
+    const uint32_t c = blockIdx.x, t0 = c * g.tiles_per_chunk, t = t0 + team;
+    const uint32_t ntc = min(g.tiles_per_chunk, g.n_tiles - t0);
+    const bool full = team < ntc && t < g.n_full_tiles;
+    if (c == 0 && threadIdx.x == 0) ws.ctrl->err = 0;
+    uint32_t d[kWordsPerLane];
+    if (full) {
+        const uint32_t* p = reinterpret_cast<const uint32_t*>(cache + (uint64_t)t * kTile) + warp * 512u + lane;
+#pragma unroll
+        for (int i = 0; i < 16; i++) d[i] = __ldcs(p + 32 * i);
+    }
+    const uint32_t ht = (&tab->HT[0][0])[threadIdx.x];
+    Smem S = setup_smem(smem, tab);
+    unsigned char* const slot = S.take(kTile);
+    uint32_t* const sHT = reinterpret_cast<uint32_t*>(S.take(4096));        // (complete behind the block's barrier)
+    sHT[threadIdx.x] = ht;
+    if (full) {
+        const uint32_t v = tile_digest_part(S, d, team == 0u, warp, lane);
+        if (lane == 0) s_wdig[team][warp] = v;
+        team_bar(team);
+        if (tt == 0) s_dig[team] = xor8(s_wdig[team]);
+    } else if (team < ntc) {                   // the ragged last tile of the cache
+        const uint32_t v = ragged_tile_digest(S, g, slot, cache + (uint64_t)t * kTile, s_rdig, team, tt);
+        if (tt == 0) s_dig[team] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const uint64_t clen = chunk_len_dev(g, c);
+    if (clen < 4) {
+        crc_out[c] = crc_bytewise(tab->T0, cache + (uint64_t)c * g.chunk_bytes, (uint32_t)clen);
+        return;
+    }
+    uint32_t st = 0;
+    for (uint32_t k = 0; k < ntc; k++)
+        st = (t0 + k == g.n_full_tiles ? mulmod_dev(st, g.k_tail, g.poly) : advance_tile(sHT, st)) ^ s_dig[k];
+    crc_out[c] = ~st;
+}
+
 struct DigTeamCtl {
     uint32_t wdig[2][8];
     unsigned long long mbar;
@@ -16,13 +76,17 @@ struct DigTeamCtl {
 };
 static_assert(sizeof(DigTeamCtl) % 16 == 0, "team control block keeps 16-byte alignment");
 
+// Tile digests, a team per tile: static striding over tiles.  Each team owns one 16 KiB stage that
+// bulk copies (TMA) fill; the team takes its 16 words per lane out of the stage, hands the stage to
+// the copy of its next tile and digests from registers meanwhile.
 template <int TEAMS>
 __global__ void __launch_bounds__(TEAMS * 256, 1)
 k_tile_digests(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables* __restrict__ tab)
 {
-    grid_dep_launch();
     extern __shared__ __align__(16) unsigned char smem[];
     Smem S = setup_smem(smem, tab);
+    grid_dep_wait();
+    grid_dep_launch();
     const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
     const uint32_t warp = tt / 32, lane = tt % 32;
     unsigned char* stage = nullptr;
@@ -69,6 +133,61 @@ k_tile_digests(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tabl
     }
     team_bar(team);
     if (tt == 32u && t_done != ~0ull) ws.dig[t_done] = xor8(tc->wdig[par ^ 1u]);
+}
+
+// Tile digests, a warp per tile: its lanes' chains run over all 128 rows, so that a chain has one end
+// per tile, no warp waits for another and there is nothing to put together.  A warp owns a 2 KiB stage
+// that bulk copies fill, an eighth of a tile each; it takes 16 words per lane out of it, hands it to
+// the next copy and walks on.  Tiles are dealt out warp by warp across the SMs, so that the SMs'
+// shares differ by a tile at most.
+constexpr uint32_t kPart = kTile / 8u;
+__global__ void __launch_bounds__(1024, 1)
+k_tile_digests_stream(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables* __restrict__ tab)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    Smem S = setup_smem(smem, tab);
+    grid_dep_wait();
+    grid_dep_launch();
+    const uint32_t warp = threadIdx.x / 32u, lane = threadIdx.x % 32u;
+    unsigned char* const stages = S.take(32u * kPart);
+    unsigned long long* const bars = reinterpret_cast<unsigned long long*>(S.take(32u * 8u));
+    uint32_t* const wdig = reinterpret_cast<uint32_t*>(S.take(32u));
+    if (!S.ok) { if (threadIdx.x == 0) atomicOr(&ws.ctrl->err, 4u); return; }
+    // the ragged last tile: by the last team of the last block (one of those with the fewest tiles), whose stages make a tile's
+    if (g.tail_len && blockIdx.x == gridDim.x - 1u && warp >= 24u) {
+        const uint32_t tt = threadIdx.x - 768u;
+        const uint32_t v = ragged_tile_digest(S, g, stages + 24u * kPart, cache + (uint64_t)g.n_full_tiles * kTile, wdig, 3, tt);
+        if (tt == 0) ws.dig[g.n_full_tiles] = v;
+    }
+    const uint64_t pol = l2_policy_evict_first();
+    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stages) + warp * kPart;
+    const uint32_t bar_s = (uint32_t)__cvta_generic_to_shared(bars) + 8u * warp;
+    const uint32_t stride = 32u * gridDim.x;
+    uint32_t t = warp * gridDim.x + blockIdx.x;
+    auto start_copy = [&](uint32_t tile, uint32_t part) {      // lane 0
+        if (tile < g.n_full_tiles && !(g.inject & kInjectNoCopy))
+            bulk_load_at(stage_s, cache + (uint64_t)tile * kTile + part * kPart, kPart, bar_s, pol);
+    };
+    if (lane == 0) { mbar_init(&bars[warp], 1); start_copy(t, 0); }
+    __syncwarp();
+    uint32_t phase = 0;
+    for (; t < g.n_full_tiles; t += stride) {
+        uint32_t s = first_in_chunk(g, t) && lane == 0u ? 0xFFFFFFFFu : 0u;      // (the all-ones start value complements the chunk's first word)
+        for (uint32_t part = 0; part < 8u; part++) {
+            wait_for_copy_at<true>(bar_s, phase, g.wait_ns, ws.ctrl, (g.inject & kInjectNoCopy) != 0u);
+            phase ^= 1u;
+            uint32_t w[kWordsPerLane];
+            read_staged_words_at(stage_s, 0u, lane, w);
+            __syncwarp();
+            if (lane == 0) start_copy(part < 7u ? t : t + stride, (part + 1u) & 7u);
+            if (part) s = chain_step(S, s);
+#pragma unroll
+            for (int i = 0; i < 15; i++) s = chain_step(S, s ^ w[i]);
+            s ^= w[15];
+        }
+        const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, s));
+        if (lane == 0) ws.dig[t] = v;
+    }
 }
 
 __global__ void __launch_bounds__(1024)

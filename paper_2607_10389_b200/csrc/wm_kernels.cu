@@ -1,7 +1,7 @@
 // CUDA kernels (sm_100a) and C ABI of the session mover's data path.
 //
 // Kernel map (every call enqueues a short chain on the caller's stream, no host sync):
-//   wm_checksum      : k_tile_digests -> k_checksum_finish
+//   wm_checksum      : k_checksum_init -> k_tile_digests (or _stream) -> k_checksum_finish; small caches: k_chunk_crcs
 //   wm_dirty_diff    : k_diff_init -> k_diff -> k_diff_compact
 //   wm_encode        : k_encode_init -> k_encode (single pass; teams publish tile lengths, one
 //                      scanner warp turns them into payload offsets) -> k_encode_finish (directory, cache CRC, header)
@@ -43,6 +43,7 @@ namespace wm {
 
 constexpr int kTeams = 4;        // encode: teams per block (plus the scanner warp)
 constexpr int kTeamsPlain = 4;   // checksum / decode: teams per block
+constexpr uint32_t kStreamTiles = 112;   // checksum: tiles per SM from which a warp takes a tile of its own
 
 struct DeviceState {
     Tables* tables = nullptr;
@@ -111,7 +112,8 @@ static const DeviceState* device_state()
         for (const void* f : dec)
             if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     }
-    if (cudaFuncSetAttribute(k_tile_digests<kTeamsPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
+    for (const void* f : {(const void*)k_tile_digests<kTeamsPlain>, (const void*)k_tile_digests_stream, (const void*)k_chunk_crcs<kTeamsPlain>})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(k_meta_crc, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(k_xxh64_paced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXSmem) != cudaSuccess) return nullptr;
     for (int k = 0; k < 4; k++)
@@ -206,6 +208,46 @@ int wm_timing_read_ms(int kind, float* ms)
     return cudaEventElapsedTime(ms, ds->ev[kind][0], ds->ev[kind][1]) == cudaSuccess ? WM_OK : WM_ERR_CUDA;
 }
 
+// The checksum calls' kernels: `tab` and g's powers carry the polynomial.
+static wm_status checksum_any(const unsigned char* c, const Geo& g, const Ws& ws, const Tables* tab, uint32_t n_sm,
+                              const DeviceState* timed, uint32_t* crc_out, cudaStream_t s)
+{
+    // A chunk per block and a tile per team, when they all fit at once: one launch instead of three.
+    // Measured (us a call, this and the three): 2 MiB in 16 KiB chunks 5.2 and 8.0, 2 and 8 MiB in 64 KiB
+    // chunks 7.8 and 8.2, 8.3 and 8.8; with more chunks per block (16 MiB) 12.7 and 10.8.
+    // (The test hook for waits that run out needs a kernel that waits.)
+    if (g.n_chunks <= n_sm && g.tiles_per_chunk <= (uint32_t)kTeamsPlain && !g.inject) {
+        if (timed) {
+            MainKernelTimer timer(timed, 0, s);
+            k_chunk_crcs<kTeamsPlain><<<g.n_chunks, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, tab, crc_out);
+        } else {
+            k_chunk_crcs<kTeamsPlain><<<g.n_chunks, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, tab, crc_out);
+        }
+        g_launches = 1;
+        return launch_status();
+    }
+    k_checksum_init<<<1, 64, 0, s>>>(ws.ctrl);
+    auto digests = [&]() {
+        // A warp per tile needs enough tiles for even shares.  Measured (us a call, a team and a warp per
+        // tile): 77 MB 21 and 24, 155 MB 34 and 36, 310 MB 59 and 58, 620 MB 112 and 105, 1.67 GB 275 and 257.
+        if (g.n_tiles >= kStreamTiles * n_sm) {
+            launch_after(k_tile_digests_stream, n_sm, 1024, kDynSmem, s, c, g, ws, tab);
+        } else {
+            const uint32_t need = (g.n_tiles + kTeamsPlain - 1) / kTeamsPlain;
+            launch_after(k_tile_digests<kTeamsPlain>, need < n_sm ? need : n_sm, kTeamsPlain * 256, kDynSmem, s, c, g, ws, tab);
+        }
+    };
+    if (timed) {
+        MainKernelTimer timer(timed, 0, s);
+        digests();
+    } else {
+        digests();
+    }
+    launch_after(k_checksum_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, ws, tab, crc_out);
+    g_launches = 3;
+    return launch_status();
+}
+
 wm_status wm_checksum(const void* cache, uint64_t nbytes, uint32_t chunk_bytes, uint32_t* crc_out,
                       void* workspace, uint64_t workspace_bytes, void* stream)
 {
@@ -214,20 +256,8 @@ wm_status wm_checksum(const void* cache, uint64_t nbytes, uint32_t chunk_bytes, 
     if (!aligned16(cache) || !aligned16(workspace) || workspace_bytes < ws_layout(g).total) return WM_ERR_ARG;
     const DeviceState* ds = device_state();
     if (!ds) return WM_ERR_CUDA;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Ws ws = ws_carve(workspace, g);
-    const unsigned char* c = static_cast<const unsigned char*>(cache);
-    const uint32_t need = (g.n_tiles + kTeamsPlain - 1) / kTeamsPlain;
-    const uint32_t grid = need < (uint32_t)ds->sm_count ? need : (uint32_t)ds->sm_count;
-    // the control block starts at zero: the error word in it is this call's outcome (wm_workspace_status)
-    if (cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), s) != cudaSuccess) return WM_ERR_CUDA;
-    {
-        MainKernelTimer timer(ds, 0, s);
-        k_tile_digests<kTeamsPlain><<<grid, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, ds->tables);
-    }
-    launch_after(k_checksum_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, ws, ds->tables, crc_out);
-    g_launches = 2;
-    return launch_status();
+    return checksum_any(static_cast<const unsigned char*>(cache), g, ws_carve(workspace, g), ds->tables, (uint32_t)ds->sm_count, ds, crc_out,
+                        static_cast<cudaStream_t>(stream));
 }
 
 // The checksum call with the polynomial as an argument.  The tile kernel and the finish kernel
@@ -264,20 +294,8 @@ wm_status wm_checksum_poly(const void* cache, uint64_t nbytes, uint32_t chunk_by
     g.k_tail = x_pow_bytes(g.tail_len, kPolyZlib);
     g.k_chunk = x_pow_bytes(g.chunk_bytes, kPolyZlib);
     g.k_last_chunk = x_pow_bytes(g.last_chunk_len, kPolyZlib);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Ws ws = ws_carve(workspace, g);
-    const unsigned char* c = static_cast<const unsigned char*>(cache);
-    const uint32_t need = (g.n_tiles + kTeamsPlain - 1) / kTeamsPlain;
-    const uint32_t grid = need < (uint32_t)ds->sm_count ? need : (uint32_t)ds->sm_count;
-    // the control block starts at zero: the error word in it is this call's outcome (wm_workspace_status)
-    if (cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), s) != cudaSuccess) return WM_ERR_CUDA;
-    {
-        MainKernelTimer timer(ds, 0, s);
-        k_tile_digests<kTeamsPlain><<<grid, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, tab);
-    }
-    launch_after(k_checksum_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, ws, tab, crc_out);
-    g_launches = 2;
-    return launch_status();
+    return checksum_any(static_cast<const unsigned char*>(cache), g, ws_carve(workspace, g), tab, (uint32_t)ds->sm_count, ds, crc_out,
+                        static_cast<cudaStream_t>(stream));
 }
 
 // XXH64 of every chunk: one kernel, no workspace, no tables.
@@ -333,9 +351,8 @@ static const NoAllocState* noalloc_state()
     build_tables(host);
     if (cudaMemcpy(s.tables, &host, sizeof(Tables), cudaMemcpyHostToDevice) != cudaSuccess) return nullptr;
     if (cudaDeviceGetAttribute(&s.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
-    if (cudaFuncSetAttribute(k_tile_digests<kTeamsPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem)
-        != cudaSuccess)
-        return nullptr;
+    for (const void* f : {(const void*)k_tile_digests<kTeamsPlain>, (const void*)k_tile_digests_stream, (const void*)k_chunk_crcs<kTeamsPlain>})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem) != cudaSuccess) return nullptr;
     s.ready = true;
     return &s;
 }
@@ -356,15 +373,8 @@ wm_status wm_checksum_noalloc(const void* cache, uint64_t nbytes, uint32_t chunk
     memset(&ws, 0, sizeof ws);
     ws.ctrl = reinterpret_cast<Ctrl*>(ns->scratch);
     ws.dig = reinterpret_cast<uint32_t*>(ns->scratch + sizeof(Ctrl));
-    // the array keeps the last call's contents; only the control block has to start at zero
-    if (cudaMemsetAsync(ns->scratch, 0, sizeof(Ctrl), s) != cudaSuccess) return WM_ERR_CUDA;
-    const unsigned char* c = static_cast<const unsigned char*>(cache);
-    const uint32_t need = (g.n_tiles + kTeamsPlain - 1) / kTeamsPlain;
-    const uint32_t grid = need < (uint32_t)ns->sm_count ? need : (uint32_t)ns->sm_count;
-    k_tile_digests<kTeamsPlain><<<grid, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, ns->tables);
-    launch_after(k_checksum_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, ws, ns->tables, crc_out);
-    g_launches = 2;
-    return launch_status();
+    // (the array keeps the last call's contents; the control block is cleared on the stream)
+    return checksum_any(static_cast<const unsigned char*>(cache), g, ws, ns->tables, (uint32_t)ns->sm_count, nullptr, crc_out, s);
 }
 
 wm_status wm_dirty_diff(const void* cache, const void* prev, uint64_t nbytes, uint32_t chunk_bytes,

@@ -458,3 +458,25 @@ def test_ragged_last_tile_wherever_it_falls(G, full, tail):
         from paper_2607_10389_b200 import binding as wm
         wm.wm_decode_verify(wire_dev, res.wire_len, dst[:n], chunk, dcrc, g.ws, g.res)
         assert wm.read_result(g.res).ok and torch.equal(dst[:n], src) and bool((dst[n:] == 0x5A).all())
+
+
+@pytest.mark.parametrize("chunk,n_chunks", [(TILE, 147), (TILE, 148), (TILE, 149), (3 * TILE, 5), (4 * TILE, 148), (4 * TILE, 149), (5 * TILE, 3)])
+@pytest.mark.parametrize("last", [2, 9, TILE - 1, TILE])             # bytes of the last chunk
+def test_checksum_around_the_one_launch_kernel(G, chunk, n_chunks, last):
+    n = (n_chunks - 1) * chunk + last
+    a = _special_cache(n, n)
+    assert np.array_equal(G(n, chunk).checksum(torch.from_numpy(a).cuda()), oracle.checksum(a, chunk))
+
+
+@pytest.mark.parametrize("tiles", [112 * 148 - 1, 112 * 148, 112 * 148 + 1, 113 * 148 + 77])
+@pytest.mark.parametrize("tail", [0, 4097])
+def test_checksum_around_the_warp_per_tile_kernel(G, tiles, tail):
+    """Against the encoder's checksums of the same cache (another kernel) and the oracle on chunks at the ends."""
+    n, chunk = tiles * TILE + tail, 8 * TILE
+    src = torch.randint(0, 256, (n,), dtype=torch.uint8, device="cuda", generator=torch.Generator("cuda").manual_seed(tiles))
+    g = G(n, chunk)
+    got = g.checksum(src)
+    _, crc, res, _ = g.encode(src)
+    assert res.status == 0 and np.array_equal(got, crc)
+    for lo, hi in ((0, 3), (g.nc // 2, g.nc // 2 + 2), (g.nc - 3, g.nc)):
+        assert np.array_equal(got[lo:hi], oracle.checksum(src[lo * chunk: min(hi * chunk, n)].cpu().numpy(), chunk))
