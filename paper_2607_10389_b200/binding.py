@@ -199,9 +199,13 @@ def _dev_u8(t: torch.Tensor, what: str) -> torch.Tensor:
     return t
 
 
+# The current stream's handle without making a Stream object of it: 0.2 us instead of 3.4, where a
+# small cache's call is 6 us of host work in all.
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _stream(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    return _raw_stream(_device()) if stream is None else stream.cuda_stream
 
 
 def _check(rc: int, what: str) -> None:
