@@ -334,35 +334,42 @@ __device__ __forceinline__ PlaneWords read_group_planes(uint32_t rec, uint32_t w
     return pw;
 }
 
-// Inverse of pack_group_planes: the lane's eight exponent bytes (two words, coded order).
-template <int W>
-__device__ __forceinline__ void unpack_group_planes(const PlaneWords& pw, uint32_t base, uint32_t& ea, uint32_t& eb)
+// The eight 4-bit deltas of a plane word, one per byte (two words, coded order).
+__device__ __forceinline__ void unpack_nibbles(uint32_t a, uint32_t& da, uint32_t& db)
+{
+    const uint32_t even = a & 0x0F0F0F0Fu, odd = (a >> 4) & 0x0F0F0F0Fu;
+    da = __byte_perm(even, odd, 0x5140);
+    db = __byte_perm(even, odd, 0x7362);
+}
+
+// Inverse of pack_group_planes: the lane's eight exponent bytes (two words, coded order).  Width 4 is
+// by far the most frequent; the others share one piece of code that goes plane by plane (seven
+// pieces, four times each in the loop, were more than the instruction cache wants to hold).
+__device__ __forceinline__ void unpack_group(const PlaneWords& pw, uint32_t base, uint32_t wd, uint32_t& ea, uint32_t& eb)
 {
     uint32_t da = 0, db = 0;
-    if (W == 8) { da = pw.a; db = pw.b; }
-    else {
-        int sh = 0;
-        if (W & 4) {
-            const uint32_t t = __byte_perm(pw.a, 0, 0x1100), u = __byte_perm(pw.a, 0, 0x3322);
-            da = (t & 0x000F000Fu) | ((t >> 4) & 0x0F000F00u);
-            db = (u & 0x000F000Fu) | ((u >> 4) & 0x0F000F00u);
-            sh = 4;
-        }
-        if (W & 2) {        // byte -> four 2-bit fields, one per byte
+    if (wd == 4u) {
+        unpack_nibbles(pw.a, da, db);
+    } else if (wd == 8u) {
+        da = pw.a; db = pw.b;
+    } else {
+        if (wd & 4u) unpack_nibbles(pw.a, da, db);
+        uint32_t sh = wd & 4u;
+        if (wd & 2u) {      // byte -> four 2-bit fields, one per byte
             uint32_t xa = pw.b & 0xFFu, xb = (pw.b >> 8) & 0xFFu;
             xa = (xa * 0x1001u) & 0x000F000Fu; xa = (xa * 0x41u) & 0x03030303u;
             xb = (xb * 0x1001u) & 0x000F000Fu; xb = (xb * 0x41u) & 0x03030303u;
             da |= xa << sh; db |= xb << sh;
-            sh += 2;
+            sh += 2u;
         }
-        if (W & 1) {        // nibble -> four bits, one per byte
+        if (wd & 1u) {      // nibble -> four bits, one per byte
             const uint32_t xa = (((pw.b >> 16) & 0xFu) * 0x00204081u) & 0x01010101u;
             const uint32_t xb = (((pw.b >> 20) & 0xFu) * 0x00204081u) & 0x01010101u;
             da |= xa << sh; db |= xb << sh;
         }
     }
     const uint32_t b4 = base * 0x01010101u;
-    if (base + ((1u << W) - 1u) <= 255u) {        // no byte can wrap: plain add
+    if (base + ((1u << wd) - 1u) <= 255u) {       // no byte can wrap: plain add
         ea = da + b4; eb = db + b4;
     } else {                                      // per byte (base + d) & 0xFF
         ea = ((da & 0x7F7F7F7Fu) + (b4 & 0x7F7F7F7Fu)) ^ ((da ^ b4) & 0x80808080u);
@@ -522,7 +529,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         const bool is_pack = is_ent || is_pack_entry(e);            // a coded tile (in either form)
         bool decoded = true;
         uint32_t w[kWordsPerLane];
-        uint32_t desc = 0;
+        uint2 dd = make_uint2(0u, 0u);      // PACK tile: the descriptors of this warp's four groups, base | width << 8 each
         uint2 sm[4];
         PlaneWords pw[4];
 
@@ -619,7 +626,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                     }
                 }
             } else if (ENT != 1) {
-                desc = lds_now_u16(stage_s + 2u * lane);
+                const uint32_t desc = lds_now_u16(stage_s + 2u * lane);
                 // Whether the descriptors are sound (step 4) is one warp's business, the one without
                 // a single-lane chore: its verdict goes to the control block and decides the call's
                 // status.  The other warps do not wait for it; they only have to stay inside the
@@ -639,26 +646,19 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                 }
                 // widths of the groups before this warp's four
                 const uint32_t wv = min((desc >> 8) & 15u, 8u);
-                const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < 4u * warp ? wv : 0u);
-                {
-                    // lanes 0..3 end up with the descriptors of the warp's four groups, each with its
-                    // group's offset in the plane area in the high half
-                    const uint32_t own = __shfl_sync(0xFFFFFFFFu, desc, 4 * warp + (lane & 3u)) & 0xFFFFu;
-                    const uint32_t wo = min((own >> 8) & 15u, 8u);
-                    uint32_t off = before;                          // running offset over the four groups
-                    const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, wo, 0), w1 = __shfl_sync(0xFFFFFFFFu, wo, 1),
-                                   w2 = __shfl_sync(0xFFFFFFFFu, wo, 2);
-                    if ((lane & 3u) >= 1u) off += w0;
-                    if ((lane & 3u) >= 2u) off += w1;
-                    if ((lane & 3u) == 3u) off += w2;
-                    off = min(off, 245u);                           // (8256 + 32 * 245 + 256 bytes of planes end inside the stage)
-                    desc = (own & 0xF0FFu) | (wo << 8) | (off << 16);
+                uint32_t off = __reduce_add_sync(0xFFFFFFFFu, lane < 4u * warp ? wv : 0u);
+                // the warp's four descriptors, the same two words in every lane, and their widths (at most 8)
+                dd = lds_now_v2<0>(stage_s + 8u * warp);
+                const uint32_t w01 = min_u16x2((dd.x >> 8) & 0x000F000Fu, 0x00080008u), w23 = min_u16x2((dd.y >> 8) & 0x000F000Fu, 0x00080008u);
+                dd.x = (dd.x & 0x00FF00FFu) | (w01 << 8);
+                dd.y = (dd.y & 0x00FF00FFu) | (w23 << 8);
 #pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        const uint32_t dg = __shfl_sync(0xFFFFFFFFu, desc, j);
-                        sm[j] = j == 0 ? lds_now_v2<0>(sm_s) : j == 1 ? lds_now_v2<256>(sm_s) : j == 2 ? lds_now_v2<512>(sm_s) : lds_now_v2<768>(sm_s);
-                        pw[j] = read_group_planes(stage_s + 8256u + 32u * (dg >> 16), (dg >> 8) & 15u, 4u * lane, 2u * lane, lane);
-                    }
+                for (int j = 0; j < 4; j++) {
+                    const uint32_t wg = j == 0 ? w01 & 15u : j == 1 ? w01 >> 16 : j == 2 ? w23 & 15u : w23 >> 16;
+                    sm[j] = j == 0 ? lds_now_v2<0>(sm_s) : j == 1 ? lds_now_v2<256>(sm_s) : j == 2 ? lds_now_v2<512>(sm_s) : lds_now_v2<768>(sm_s);
+                    // (8256 + 32 * 245 + 256 bytes of planes end inside the stage)
+                    pw[j] = read_group_planes(stage_s + 8256u + 32u * min(off, 245u), wg, 4u * lane, 2u * lane, lane);
+                    off += wg;
                 }
             }
         } else if (e == 1u || e == 2u) {
@@ -736,21 +736,11 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                 uint32_t st = 0, last = 0;
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    const uint32_t dg = __shfl_sync(0xFFFFFFFFu, desc, j);
-                    const uint32_t base = dg & 0xFFu, wd = (dg >> 8) & 15u;
-                    uint32_t ea = base * 0x01010101u, eb = ea;
+                    const uint32_t dw = j < 2 ? dd.x : dd.y;
+                    const uint32_t base = (j & 1) ? (dw >> 16) & 0xFFu : dw & 0xFFu, wd = (j & 1) ? dw >> 24 : (dw >> 8) & 15u;
+                    uint32_t ea, eb;
                     if (ENT == 1 || (ENT == 2 && is_ent)) { ea = pw[j].a; eb = pw[j].b; }     // the exponent bytes are already there
-                    else if (wd == 4u) unpack_group_planes<4>(pw[j], base, ea, eb);       // by far the most frequent width
-                    else switch (wd) {     // uniform across the warp
-                        case 1: unpack_group_planes<1>(pw[j], base, ea, eb); break;
-                        case 2: unpack_group_planes<2>(pw[j], base, ea, eb); break;
-                        case 3: unpack_group_planes<3>(pw[j], base, ea, eb); break;
-                        case 5: unpack_group_planes<5>(pw[j], base, ea, eb); break;
-                        case 6: unpack_group_planes<6>(pw[j], base, ea, eb); break;
-                        case 7: unpack_group_planes<7>(pw[j], base, ea, eb); break;
-                        case 8: unpack_group_planes<8>(pw[j], base, ea, eb); break;
-                        default: break;
-                    }
+                    else unpack_group(pw[j], base, wd, ea, eb);
                     // A word rotated left by one bit reads [E | m << 1 | sign of the other half] in
                     // each half: swap bit 0 inside the byte pairs of the sign-mantissa words, put
                     // the exponent bytes beside them, rotate back.
