@@ -515,11 +515,16 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     team_bar(team);
     uint32_t phase = 0;
     uint32_t t_done = kNone;           // tile whose digest parts wait in wdig[(it - 1) & 1]
+    auto store_digest = [&](uint32_t done, uint32_t slot) {     // warp 1
+        if (warp != 1u || done == kNone) return;
+        const uint32_t v = place_warp_digests(S, tc_s + (uint32_t)offsetof(DecTeamCtl, wdig) + 32u * slot, lane);
+        if (lane == 0) ws.dig[done] = v;
+    };
     for (uint32_t it = 0;; it++) {
         const uint32_t t = lds_now<offsetof(DecTeamCtl, slot)>(tc_s + 16u * (it & 3u));
         if (t >= g.n_full_tiles) {
             team_bar(team);
-            if (tt == 32u && t_done != kNone) ws.dig[t_done] = xor8(TC()->wdig[(it & 1u) ^ 1u]);
+            store_digest(t_done, (it & 1u) ^ 1u);
             break;
         }
         const uint32_t ew = lds_now<offsetof(DecTeamCtl, slot) + 4>(tc_s + 16u * (it & 3u));
@@ -688,7 +693,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         uint32_t l_tk = kNone;
         // (spread over three warps: the team waits for whichever warp has the most to do)
         if (tt == 64u) start_copy(TC()->slot[(it + 1u) & 3u]);
-        if (tt == 32u && t_done != kNone) ws.dig[t_done] = xor8(TC()->wdig[p ^ 1u]);
+        store_digest(t_done, p ^ 1u);
         uint32_t t_look = kNone;           // warps 0 and 3: the tile claimed a step ago (two tiles ahead)
         if (leader) {                      // its table entry and offsets
             t_look = TC()->slot[(it + 2u) & 3u].t;
@@ -759,7 +764,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                     }
                 }
                 if (MODE != 2) {
-                    const uint32_t v = warp_place(S, __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, last)), warp, lane);
+                    const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, last));
                     if (lane == 0) sts_now(tc_s + (uint32_t)offsetof(DecTeamCtl, wdig) + 32u * p + 4u * warp, v);
                     have_digest = true;
                 }
@@ -770,7 +775,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                     for (int i = 0; i < 16; i++) put(i, w[i]);
                 }
                 if (MODE != 2) {
-                    const uint32_t v = tile_digest_part(S, w, fold, warp, lane);
+                    const uint32_t v = tile_digest_block(S, w, fold, warp, lane);
                     if (lane == 0) sts_now(tc_s + (uint32_t)offsetof(DecTeamCtl, wdig) + 32u * p + 4u * warp, v);
                     have_digest = true;
                 }

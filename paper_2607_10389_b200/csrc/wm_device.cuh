@@ -194,6 +194,20 @@ __device__ __forceinline__ uint32_t warp_place(const Smem& S, uint32_t digest, u
     return __reduce_xor_sync(0xFFFFFFFFu, v);
 }
 
+// The tile's digest from its eight warps' block digests (one warp, the result in every lane): lane l
+// places nibbles 2 (l mod 4) and the next of warp l / 4's digest.  In the codec kernels one warp does
+// this for the team, a step later, where each warp placing its own digest is a look-up, two reductions
+// and their wait in every warp.  wdig_s: shared-window address of the eight digests.
+__device__ __forceinline__ uint32_t place_warp_digests(const Smem& S, uint32_t wdig_s, uint32_t lane)
+{
+    const uint32_t d = lds_now<0>(wdig_s + (lane & ~3u));
+    const uint32_t n = 2u * (lane & 3u);                     // table row 8 (lane / 4) + n = 2 lane
+    const uint32_t at = S.L - 4u * lane + kImgBytes + 128u * lane;       // (the position tables stand behind the image)
+    const uint32_t b = d >> (4u * n);
+    const uint32_t v = lds_off<0>(at + 4u * (b & 15u)) ^ lds_off<64>(at + 4u * ((b >> 4) & 15u));
+    return __reduce_xor_sync(0xFFFFFFFFu, v);
+}
+
 // ---- the same digest with small tables, for kernels that see a few hundred kilobytes ----
 // Copying the 144 KiB lane-replicated image costs more than such a kernel's whole work.  Here
 // the chain uses one copy of the four byte tables (4 KiB in shared memory; lookups may collide on a

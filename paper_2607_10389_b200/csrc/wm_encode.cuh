@@ -618,7 +618,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         // ---- Y: digest, exponent ranges, length out, words parked
         const uint32_t slY = (sl + 3u) & 7u;
         if (hotY) {
-            const uint32_t v = tile_digest_part(S, d, (qY & kQFirst) != 0, warp, lane);
+            const uint32_t v = tile_digest_block(S, d, (qY & kQFirst) != 0, warp, lane);
             // From here on the words are kept rotated left by one bit: each half then reads
             // [E | mantissa | a sign bit], E in its high byte (the two sign bits of a word
             // land in each other's half; the packing step puts them right).
@@ -816,7 +816,10 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         // warp is the one the team waits for): the digest by warp 1; the table entry, where its
         // chunk starts and the total by warp 7 (not warp 4: warps w and w + 4 issue through the same
         // scheduler, and warp 4 would share the end of the step with the leader's hand-over).
-        if (tt == 32u && is_tile(qX)) ws.dig[tXn] = xor8(tc->wdig[sl]);
+        if (warp == 1u && is_tile(qX)) {
+            const uint32_t v = place_warp_digests(S, (uint32_t)__cvta_generic_to_shared(tc->wdig[sl]), lane);
+            if (lane == 0) ws.dig[tXn] = v;
+        }
         if (tt == 224u && is_tile(qX)) {
             uint32_t entry, enc_len;
             const uint32_t Ssum = tc->ssum[sl];

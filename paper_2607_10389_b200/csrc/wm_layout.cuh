@@ -290,6 +290,17 @@ __device__ __forceinline__ uint32_t tile_digest_part(const Smem& S, uint32_t (&w
     return warp_place(S, d, warp, lane);
 }
 
+// The same without its place in the tile (place_warp_digests does that for the team).
+__device__ __forceinline__ uint32_t tile_digest_block(const Smem& S, uint32_t (&w)[kWordsPerLane], bool init_fold,
+                                                      uint32_t warp, uint32_t lane)
+{
+    const uint32_t m = (init_fold && warp == 0 && lane == 0) ? 0xFFFFFFFFu : 0u;
+    w[0] ^= m;
+    const uint32_t d = warp_block_digest(S, w);
+    w[0] ^= m;
+    return d;
+}
+
 __device__ __forceinline__ uint32_t xor8(const uint32_t* p)
 {
     return p[0] ^ p[1] ^ p[2] ^ p[3] ^ p[4] ^ p[5] ^ p[6] ^ p[7];
