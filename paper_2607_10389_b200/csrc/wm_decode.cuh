@@ -313,7 +313,7 @@ struct DecTeamCtl {
 };
 static_assert(sizeof(DecTeamCtl) % 16 == 0, "team control block keeps 16-byte alignment");
 
-// The plane words of one group as stored (aligned per-lane units, see pack_group_planes):
+// The plane words of one group as stored (aligned per-lane units, see pack_group):
 // a = the 4-bit plane's word or the low half of an 8-bit plane; b = the 2-bit plane's 16 bits
 // in the low half and the 1-bit plane's byte in bits 16-23, or the high half of an 8-bit plane.
 struct PlaneWords { uint32_t a, b; };
@@ -342,7 +342,7 @@ __device__ __forceinline__ void unpack_nibbles(uint32_t a, uint32_t& da, uint32_
     db = __byte_perm(even, odd, 0x7362);
 }
 
-// Inverse of pack_group_planes: the lane's eight exponent bytes (two words, coded order).  Width 4 is
+// Inverse of pack_group: the lane's eight exponent bytes (two words, coded order).  Width 4 is
 // by far the most frequent; the others share one piece of code that goes plane by plane (seven
 // pieces, four times each in the loop, were more than the instruction cache wants to hold).
 __device__ __forceinline__ void unpack_group(const PlaneWords& pw, uint32_t base, uint32_t wd, uint32_t& ea, uint32_t& eb)

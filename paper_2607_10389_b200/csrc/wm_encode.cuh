@@ -229,38 +229,43 @@ __device__ __forceinline__ void stg_v2(void* p, uint32_t a, uint32_t b)
 // whose bit is set in W) take consecutive bits of the deltas from bit 0.  In every plane lane
 // l owns an aligned 4 / 2 / 1-byte unit at l times that size, so each warp store covers one
 // contiguous, sector-aligned run of 128 / 64 / 32 bytes and nothing needs staging.
-//   nibbles : v | v >> 4 puts two 4-bit values side by side in bytes 0 and 2 of each word
+//   nibbles : the low nibbles of v and the high ones of v >> 4 put two 4-bit values side by side in
+//             bytes 0 and 2 of each word (bits above the plane fall away)
 //   2 bits  : (t * 0x01041040) >> 24 gathers the four 2-bit fields of a word into one byte
 //   1 bit   : (t * 0x01020408) >> 24 gathers the four bits of a word into one nibble
 // (the partial products of both multiplications land on distinct bits, so no carry occurs).
-template <int W>
-__device__ __forceinline__ void pack_group_planes(uint32_t e4a, uint32_t e4b, uint32_t base, unsigned char* rec,
-                                                  uint32_t lane)
+// Width 4 is by far the most frequent; the others share one piece of code that goes plane by plane
+// (seven pieces, four times each in the loop, were more than the instruction cache wants to hold).
+__device__ __forceinline__ void pack_nibbles(uint32_t da, uint32_t db, unsigned char* p, uint32_t lane)
+{
+    const uint32_t va = (da & 0x0F0F0F0Fu) | ((da >> 4) & 0xF0F0F0F0u), vb = (db & 0x0F0F0F0Fu) | ((db >> 4) & 0xF0F0F0F0u);
+    st_stream_u32(p + 4 * lane, __byte_perm(va, vb, 0x6420));
+}
+__device__ __forceinline__ void pack_group(uint32_t wd, uint32_t e4a, uint32_t e4b, uint32_t base, unsigned char* p, uint32_t lane)
 {
     const uint32_t b4 = base * 0x01010101u;
     uint32_t da = e4a - b4, db = e4b - b4;
-    if (W == 8) {
-        stg_v2(rec + 8 * lane, da, db);
-        return;
-    }
-    unsigned char* p = rec;
-    if (W & 4) {
-        const uint32_t na = (W == 4) ? da : (da & 0x0F0F0F0Fu), nb = (W == 4) ? db : (db & 0x0F0F0F0Fu);
-        const uint32_t va = na | (na >> 4), vb = nb | (nb >> 4);
-        st_stream_u32(p + 4 * lane, __byte_perm(va, vb, 0x6420));
-        p += 128;
-        da >>= 4; db >>= 4;
-    }
-    if (W & 2) {
-        const uint32_t pa = (da & 0x03030303u) * 0x01041040u, pb = (db & 0x03030303u) * 0x01041040u;
-        stg_u16(p + 2 * lane, __byte_perm(pa, pb, 0x0073));
-        p += 64;
-        da >>= 2; db >>= 2;
-    }
-    if (W & 1) {
-        const uint32_t pa = (da & 0x01010101u) * 0x01020408u, pb = (db & 0x01010101u) * 0x01020408u;
-        const uint32_t x = __byte_perm(pa, pb, 0x0073);          // byte 0: a's nibble, byte 1: b's nibble
-        stg_u8(p + lane, x | (x >> 4));
+    if (wd == 4u) {
+        pack_nibbles(da, db, p, lane);
+    } else if (wd == 8u) {
+        stg_v2(p + 8 * lane, da, db);
+    } else {
+        if (wd & 4u) {
+            pack_nibbles(da, db, p, lane);
+            p += 128;
+            da >>= 4; db >>= 4;
+        }
+        if (wd & 2u) {
+            const uint32_t pa = (da & 0x03030303u) * 0x01041040u, pb = (db & 0x03030303u) * 0x01041040u;
+            stg_u16(p + 2 * lane, __byte_perm(pa, pb, 0x0073));
+            p += 64;
+            da >>= 2; db >>= 2;
+        }
+        if (wd & 1u) {
+            const uint32_t pa = (da & 0x01010101u) * 0x01020408u, pb = (db & 0x01010101u) * 0x01020408u;
+            const uint32_t x = __byte_perm(pa, pb, 0x0073);          // byte 0: a's nibble, byte 1: b's nibble
+            stg_u8(p + lane, x | (x >> 4));
+        }
     }
 }
 
@@ -655,8 +660,8 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 // orders like its halves and one warp reduction per bound does
                 mn = min_u16x2(mn, __byte_perm(mn, mn, 0x1032));
                 mx = max_u16x2(mx, __byte_perm(mx, mx, 0x1032));
-                const uint32_t emin = (__reduce_min_sync(0xFFFFFFFFu, mn) >> 8) & 0xFFu;
-                const uint32_t emax = (__reduce_max_sync(0xFFFFFFFFu, mx) >> 8) & 0xFFu;
+                const uint32_t emin = __reduce_min_sync(0xFFFFFFFFu, mn) >> 24;
+                const uint32_t emax = __reduce_max_sync(0xFFFFFFFFu, mx) >> 24;
                 gw[j] = emin | ((32u - __clz(emax - emin)) << 8);
             }
             }
@@ -790,17 +795,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                     const uint32_t e4a = __byte_perm(d[4 * j], d[4 * j + 1], 0x7531), e4b = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x7531);
                     unsigned char* rec = pl_dst + 32u * before;
                     before += wd;
-                    if (wd == 4u) pack_group_planes<4>(e4a, e4b, base, rec, lane);      // by far the most frequent width
-                    else switch (wd) {     // uniform across the warp
-                        case 1: pack_group_planes<1>(e4a, e4b, base, rec, lane); break;
-                        case 2: pack_group_planes<2>(e4a, e4b, base, rec, lane); break;
-                        case 3: pack_group_planes<3>(e4a, e4b, base, rec, lane); break;
-                        case 5: pack_group_planes<5>(e4a, e4b, base, rec, lane); break;
-                        case 6: pack_group_planes<6>(e4a, e4b, base, rec, lane); break;
-                        case 7: pack_group_planes<7>(e4a, e4b, base, rec, lane); break;
-                        case 8: pack_group_planes<8>(e4a, e4b, base, rec, lane); break;
-                        default: break;
-                    }
+                    pack_group(wd, e4a, e4b, base, rec, lane);
                 }
             } else if (ZEROS && Ssum == kSumConstTile) {
                 // the value (any word's low half, rotated back), then 30 zero bytes
