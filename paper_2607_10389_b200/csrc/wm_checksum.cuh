@@ -140,7 +140,6 @@ k_tile_digests(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tabl
 // that bulk copies fill, an eighth of a tile each; it takes 16 words per lane out of it, hands it to
 // the next copy and walks on.  Tiles are dealt out warp by warp across the SMs, so that the SMs'
 // shares differ by a tile at most.
-constexpr uint32_t kPart = kTile / 8u;
 __global__ void __launch_bounds__(1024, 1)
 k_tile_digests_stream(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables* __restrict__ tab)
 {
@@ -149,24 +148,24 @@ k_tile_digests_stream(const unsigned char* __restrict__ cache, Geo g, Ws ws, con
     grid_dep_wait();
     grid_dep_launch();
     const uint32_t warp = threadIdx.x / 32u, lane = threadIdx.x % 32u;
-    unsigned char* const stages = S.take(32u * kPart);
+    unsigned char* const stages = S.take(32u * kShare);
     unsigned long long* const bars = reinterpret_cast<unsigned long long*>(S.take(32u * 8u));
     uint32_t* const wdig = reinterpret_cast<uint32_t*>(S.take(32u));
     if (!S.ok) { if (threadIdx.x == 0) atomicOr(&ws.ctrl->err, 4u); return; }
     // the ragged last tile: by the last team of the last block (one of those with the fewest tiles), whose stages make a tile's
     if (g.tail_len && blockIdx.x == gridDim.x - 1u && warp >= 24u) {
         const uint32_t tt = threadIdx.x - 768u;
-        const uint32_t v = ragged_tile_digest(S, g, stages + 24u * kPart, cache + (uint64_t)g.n_full_tiles * kTile, wdig, 3, tt);
+        const uint32_t v = ragged_tile_digest(S, g, stages + 24u * kShare, cache + (uint64_t)g.n_full_tiles * kTile, wdig, 3, tt);
         if (tt == 0) ws.dig[g.n_full_tiles] = v;
     }
     const uint64_t pol = l2_policy_evict_first();
-    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stages) + warp * kPart;
+    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stages) + warp * kShare;
     const uint32_t bar_s = (uint32_t)__cvta_generic_to_shared(bars) + 8u * warp;
     const uint32_t stride = 32u * gridDim.x;
     uint32_t t = warp * gridDim.x + blockIdx.x;
     auto start_copy = [&](uint32_t tile, uint32_t part) {      // lane 0
         if (tile < g.n_full_tiles && !(g.inject & kInjectNoCopy))
-            bulk_load_at(stage_s, cache + (uint64_t)tile * kTile + part * kPart, kPart, bar_s, pol);
+            bulk_load_at(stage_s, cache + (uint64_t)tile * kTile + part * kShare, kShare, bar_s, pol);
     };
     if (lane == 0) { mbar_init(&bars[warp], 1); start_copy(t, 0); }
     __syncwarp();

@@ -26,6 +26,7 @@ namespace wm {
 
 constexpr uint32_t kTile = 16384;
 constexpr uint32_t kTeamThreads = 256;
+constexpr uint32_t kShare = 2048;           // sixteen rows of a tile: what a warp holds, 16 words per lane
 constexpr uint32_t kWordsPerLane = 16;
 // Dynamic shared memory every table-using kernel asks for: the 144 KiB image and 81 KiB for stages and
 // control blocks.  227 KiB is the per-block maximum for static and dynamic shared memory together;
@@ -208,6 +209,15 @@ __device__ __forceinline__ uint32_t place_warp_digests(const Smem& S, uint32_t w
     return __reduce_xor_sync(0xFFFFFFFFu, v);
 }
 
+// The same for a tile's four warps of 4096 bytes (rows 32 w ..): lane l places nibble l mod 8 of warp l / 8's digest.
+__device__ __forceinline__ uint32_t place_team4_digests(const Smem& S, uint32_t wdig_s, uint32_t lane)
+{
+    const uint32_t w = lane >> 3, n = lane & 7u;
+    const uint32_t d = lds_now<0>(wdig_s + 4u * w);
+    // (advancing over 4096 (3 - w) bytes is row 2 w + 1 of the tables for 2048-byte blocks)
+    return __reduce_xor_sync(0xFFFFFFFFu, lds_off<0>(S.L - 4u * lane + kImgBytes + 64u * (8u * (2u * w + 1u) + n) + 4u * ((d >> (4u * n)) & 15u)));
+}
+
 // ---- the same digest with small tables, for kernels that see a few hundred kilobytes ----
 // Copying the 144 KiB lane-replicated image costs more than such a kernel's whole work.  Here
 // the chain uses one copy of the four byte tables (4 KiB in shared memory; lookups may collide on a
@@ -360,13 +370,17 @@ __device__ __forceinline__ uint32_t mbar_try(uint32_t bar_s, uint32_t parity)
                  : "=r"(done) : "r"(bar_s), "r"(parity), "r"(200000u) : "memory");
     return done;
 }
-// The same question without waiting at all.
+// The same question without waiting at all; one arrival.
 __device__ __forceinline__ uint32_t mbar_test(uint32_t bar_s, uint32_t parity)
 {
     uint32_t done;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(done) : "r"(bar_s), "r"(parity) : "memory");
     return done;
+}
+__device__ __forceinline__ void mbar_arrive_at(uint32_t bar_s)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_s) : "memory");
 }
 __device__ __forceinline__ uint64_t l2_policy_evict_first()
 {

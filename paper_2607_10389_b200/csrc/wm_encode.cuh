@@ -189,26 +189,31 @@ __device__ __forceinline__ uint32_t desc_of(uint32_t base, uint32_t w)
     return base | (w << 8) | ((((base & 15u) ^ (base >> 4) ^ w ^ 5u) & 15u) << 12);
 }
 
+// A team of the encode kernel: four warps.  Warp w owns rows 32w .. 32w+31 of the tile, that is shares
+// (16 rows, four groups) 2w and 2w + 1, one after the other.
+constexpr uint32_t kEncTeams = 8, kEncTeamThreads = 128;
 struct EncTeamCtl {
-    uint32_t wtab[8][32];   // per group: base | w << 8 (| the all-zero mark on a warp's first entry) (a ring of
-                            // slots: one per tile in flight and spares, so that a slot is rewritten
-                            // long after its last read)
-    uint32_t wdig[8][8];    // per warp: its contribution to the tile digest
-    uint32_t spare8[8];     // (unused)
-    uint32_t ssum[8];       // sum of the 32 widths of the slot's tile (set by the publishing warp), or a mark:
+    uint32_t wtab[4][32];   // per group: base | w << 8 (| marks on a share's first entry), by step modulo 4
+    uint32_t wdig[4][4];    // per warp: its block's digest
+    uint32_t etab[4][8];    // entropy option, per share: anchor | words of its stream << 8 (0xFFFF: a strand too long for the form)
+    uint32_t ssum[4];       // sum of the 32 widths of the tile (set by the publishing warp), or a mark:
                             // zero tile, constant tile, kSumEnt | words of the streams for a tile stored in ENT form
-    uint32_t etab[8][8];    // entropy option, per warp: anchor | words of its stream << 8 (0xFFFF: a strand too long for the form)
-    uint32_t next[2];       // ticket claimed in this step (>= n_tiles: none left), by step parity
+    uint32_t next[2];       // the tile to be measured two steps after it was put here, by step parity
     uint32_t pad[2];
+    uint32_t kring[8];      // with a mask: the ticket of a tile in flight, by step modulo 8 (placement runs over tickets)
     unsigned long long excl[2];   // offset of the tile packed in the next step, by step parity
-    unsigned long long mbar;      // completion of the bulk copy into the team's stage
-    unsigned long long pad2;
     unsigned long long nptr[2];   // leaf mode: address (k_leaf_map) of the tile in next[], by step parity
-    uint32_t kring[8];            // with a mask: the ticket of the tile in each ring slot (placement runs over tickets)
-    unsigned char sbits[4][256];  // entropy option: every strand's bit length - 64, from the measuring step to the
-                                  // packing step three steps on (slot: step mod 4, as in tensor memory)
+    unsigned long long mbar[4];   // per warp: completion of the bulk copy into its stage
+    unsigned long long measured;  // the four warps' measures of the step's tile are complete
+    unsigned long long pad2;
+    unsigned char sbits[2][256];  // entropy option: every strand's bit length - 64, by step parity (a warp reads its
+                                  // own strands only, before it writes the next ones)
 };
 static_assert(sizeof(EncTeamCtl) % 16 == 0, "team control block keeps 16-byte alignment");
+__device__ __forceinline__ void enc_team_bar(uint32_t team)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(kEncTeamThreads) : "memory");
+}
 
 __device__ __forceinline__ void stg_u8(void* p, uint32_t v)
 {
@@ -327,30 +332,33 @@ __device__ __forceinline__ uint32_t ent_parse_value(uint32_t buf, uint32_t s, ui
     return s == 8u ? (buf >> 8) & 0xFFu : (anchor + base - x) & 0xFFu;
 }
 
-// Single-pass fused checksum + encode.  Each team keeps four tiles in flight:
-//     X  measured three steps ago, packed and written to the wire image in this step
-//     V, W  measured two / one steps ago, waiting for their offsets
-//     Y  checksummed and measured in this step (its length is published right after the next barrier)
-// The team owns one 16 KiB stage in shared memory that bulk copies (TMA) fill, one tile per
-// step, each copy started a whole step before its tile is needed.  A measured tile's words
-// (16 registers per lane) are parked in tensor memory until its offset is known, so a tile is
-// read from memory once and nothing waits in registers.  Per step:
-//     take Y's words from the stage | team barrier | publish len(W), the tile measured a step
-//     ago | start the copy of the next Y | digest + exponent ranges of Y | park Y | fetch X |
-//     pack X straight into the wire image
-// Meanwhile two round trips to L2 are in flight whose answers are needed a step later: the
-// ticket of the tile to measure two steps on and the offset of the tile to pack next.  These and
-// the other single-lane chores of a step sit on different warps: the team passes one barrier per
-// tile, so it runs at the pace of the warp that has the most to do.
-// Template switches: MASKED (a dirty mask was given), LEAVES (the cache is a table of tensors;
-// tickets are claimed one step further ahead so that a tile's address can be looked up on the
-// way), ZEROS (the zero / constant tile option), ENT (the entropy option: the measuring step also
+// Single-pass fused checksum + encode.  Each team keeps three tiles in flight:
+//     X  measured two steps ago, packed and written to the wire image in this step
+//     W  measured in the last step, at the end of which its length was published
+//     Y  checksummed and measured in this step
+// Every warp has a 2 KiB stage of its own in shared memory that bulk copies (TMA) fill, a share (16
+// rows) at a time; it takes 16 words per lane out of it and starts the next copy at once, so a warp
+// waits for its own data and the team meets at one barrier per tile.  A measured share's words are
+// parked in tensor memory (four shares per warp: two tiles) until the tile's offset is known, so a
+// tile is read from memory once and nothing waits in registers.  Per step:
+//     team barrier | fetch X's two shares and pack them straight into the wire image | take Y's two
+//     shares: digest, exponent ranges, park | publish len(Y)
+// The chores of a step sit on different warps: the team passes one barrier per tile, so it runs at the
+// pace of the warp that has the most to do.
+// What bounds it is the number of instructions issued, then the time an offset takes to come back.
+// Teams of eight warps with one share each and one stage per team met twice as often and did the
+// step's bookkeeping once per share: 11 % more instructions, 596 us on the engine cache (1.67 GB)
+// against 526 us, 449 -> 412 with a mask, 604 -> 565 in leaf mode, 1178 -> 1123 with the entropy option.
+// The four shares per warp that tensor memory holds leave one step between a length and its offset;
+// with lengths published behind the next team barrier, and tickets claimed a step earlier, late
+// offsets held back the lengths that other offsets waited for, and the kernel fell to 767 us.
+// Template switches: MASKED (a dirty mask was given), LEAVES (the cache is a table of tensors), ZEROS (the zero / constant tile option), ENT (the entropy option: the measuring step also
 // adds up codeword lengths, the tile takes the shorter of the two coded forms, and for the ENT
 // form the packing step writes the strands' lengths and the share's stream of words instead of bit planes).
 // Packed data goes from registers to the wire image directly: in every region of a PACK tile
 // a lane owns an aligned unit at a lane-strided place, so each warp store is one contiguous
 // sector-aligned run.  Claiming a tile before the previous offset is known means that, if the
-// scanner is late, this team waits while that tile's length is not out yet; with three steps
+// scanner is late, this team waits while that tile's length is not out yet; with a whole step
 // of slack that is rare, and it only delays: the teams that hold earlier tiles never depend
 // on this one.
 // A tile as a team passes it round: its number in the low 22 bits, kQFirst when it is the first
@@ -359,9 +367,9 @@ __device__ __forceinline__ uint32_t ent_parse_value(uint32_t buf, uint32_t s, ui
 // Only full tiles are passed round: the ragged last tile is the scanner's block's business.
 constexpr uint32_t kQNone = 1u << 31, kQFirst = 1u << 30, kQTile = (1u << 22) - 1u;
 constexpr uint32_t kQOffShift = 22;
-// Marks in a team's width table: on a warp's first entry, all 2 KiB of the warp's rows are zero;
+// Marks in a team's width table: on a share's first entry, all 2 KiB of its rows are zero;
 // as the sum of the widths, the tile is all zero.
-// kWarpConst: all 1024 elements of the warp's rows hold one value (its sign-mantissa byte rides in
+// kWarpConst: all 1024 elements of the share's rows hold one value (its sign-mantissa byte rides in
 // bits 16-23 of the entry, the exponent is the base); kSumConstTile: the tile holds one value.
 constexpr uint32_t kWarpAllZero = 0x8000u, kWarpConst = 0x4000u, kSumZeroTile = 0xFFFFu, kSumConstTile = 0xFFFEu;
 // The tile is stored in ENT form (shorter than its bit planes and than raw); low half: words of its streams.
@@ -409,8 +417,8 @@ __device__ __forceinline__ void encode_ragged_tile(const Smem& S, const Geo& g, 
     if (excl + g.tail_len <= wire_cap - g.meta_end) copy_ragged_tile(wire + g.meta_end + excl, tile, g.tail_len, tt);
 }
 
-template <int TEAMS, bool MASKED, bool LEAVES, bool ZEROS, bool ENT = false>
-__global__ void __launch_bounds__(TEAMS * 256, 1)
+template <bool MASKED, bool LEAVES, bool ZEROS, bool ENT = false>
+__global__ void __launch_bounds__(kEncTeams * kEncTeamThreads, 1)
 k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restrict__ dirty,
          unsigned char* __restrict__ wire, uint64_t wire_cap, Ws ws, const Tables* __restrict__ tab)
 {
@@ -442,17 +450,13 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                                wire, wire_cap, ws, n_tickets - 1u, slot, wdig);
         return;
     }
-    const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
-    const uint32_t warp = tt / 32, lane = tt % 32;
-    unsigned char* stage = nullptr;
-    // (leaf mode: a tile may start off a 16-byte boundary; its copy then starts at the boundary
+    const uint32_t team = threadIdx.x / kEncTeamThreads, tt = threadIdx.x % kEncTeamThreads;
+    const uint32_t wc = threadIdx.x / 32, warp = tt / 32, lane = tt % 32;
+    // (leaf mode: a tile may start off a 16-byte boundary; a copy then starts at the boundary
     // below and is 16 bytes longer, so the stage is too)
-    constexpr uint32_t kStage = LEAVES ? kTile + 16u : kTile;
-    for (int i = 0; i < TEAMS; i++) {          // every thread carves the same blocks in the same order
-        unsigned char* p = S.take(kStage);
-        if ((uint32_t)i == team) stage = p;
-    }
-    EncTeamCtl* tc = reinterpret_cast<EncTeamCtl*>(S.take(TEAMS * sizeof(EncTeamCtl)));
+    constexpr uint32_t kStage = LEAVES ? kShare + 16u : kShare;
+    unsigned char* const stages = S.take(kEncTeams * 4u * kStage);
+    EncTeamCtl* tc = reinterpret_cast<EncTeamCtl*>(S.take(kEncTeams * sizeof(EncTeamCtl)));
     // ENT: codeword length and codeword by k = E - anchor + 256 (1..511), so that a look-up is the
     // exponent added to an address the share works out once (no slot arithmetic per element); the
     // escape's codeword reads 0xFFFF (the packing step lets the exponent through its high byte)
@@ -471,74 +475,61 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
 
     // Tensor memory for the tiles in flight: allocated by the block's first warp, the address
     // goes round through shared memory.  Warp w of the block owns lanes 32 (w % 4) .. + 31 and
-    // 64 columns from 64 (w / 4): four slots of 16 columns, one per tile in flight.
+    // 64 columns from 64 (w / 4): four slots of 16 columns, two shares of two tiles.
     if (threadIdx.x < 32) tmem_alloc_all(&s_tmem);
     tmem_fence_before_sync();
     __syncthreads();
     tmem_fence_after_sync();
-    const uint32_t wc = threadIdx.x / 32;
     const uint32_t tmem_warp = s_tmem + ((32u * (wc & 3u)) << 16) + 64u * (wc >> 2);
 
-    unsigned char* const dir = wire + 64;
-    uint16_t* const tile_tab = reinterpret_cast<uint16_t*>(wire + 64 + 16ull * g.n_chunks);
     unsigned char* const payload = wire + g.meta_end;
     const uint64_t room = wire_cap - g.meta_end;                 // payload bytes that fit
     const uint64_t pol_once = l2_policy_evict_first();           // every tile is read once
-    const uint32_t* const my_words = reinterpret_cast<const uint32_t*>(stage) + warp * 512u + lane;
-    const uint32_t sm_off = 64u + 1024u * warp + 8u * lane;      // this lane's place in a group's sign-mantissa run
+    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stages) + wc * kStage;
+    const uint32_t tc_s = (uint32_t)__cvta_generic_to_shared(tc);
+    const uint32_t bar_s = tc_s + (uint32_t)offsetof(EncTeamCtl, mbar) + 8u * warp;
     const bool leader = (tt == 0);
     uint32_t phase = 0;                // parity of the stage's next completion
+    uint32_t measured_phase = 0;       // warp 3: of the measures'
 
     auto is_tile = [](uint32_t q) { return (int32_t)q >= 0; };
-    // (the placement words are indexed by ticket: with a mask that is the ring slot's ticket, else the tile number)
-    auto place_of = [&](uint32_t slot, uint32_t t) { return MASKED ? tc->kring[slot] : t; };
-    auto publish_len = [&](uint32_t slot, uint32_t t, uint32_t len) { st_relaxed_u32(ws.lbk + place_of(slot, t), kFlagA | (len / kUnit)); };
+    // (the placement words are indexed by ticket: with a mask that is the tile's entry in kring, else the tile number)
+    auto place_of = [&](uint32_t step, uint32_t q) { return MASKED ? tc->kring[step & 7u] : q & kQTile; };
     // where tile t lives: its address in the flat cache, or (leaf mode) the address that k_leaf_map wrote
     auto tile_src = [&](uint32_t t) -> unsigned long long {
         return LEAVES ? ws.tptr[t] : reinterpret_cast<unsigned long long>(cache + (uint64_t)t * kTile);
     };
-    // One thread of the team, after the barrier that frees the stage.  Leaf mode: a tile may start
-    // off a 16-byte boundary; the copy then starts at the boundary below and takes 16 bytes more
-    // (k_leaf_map saw to it that they belong to the leaf); the readers shift by the remainder.
-    auto start_copy = [&](uint32_t q, unsigned long long src) {
+    // Lane 0 of a warp, when the warp's stage is free: the copy of one of its two shares.  Leaf mode: a
+    // tile may start off a 16-byte boundary; the copy then starts at the boundary below and takes 16
+    // bytes more (k_leaf_map saw to it that they belong to the leaf); the readers shift by the remainder.
+    auto start_copy = [&](uint32_t q, unsigned long long src, uint32_t part) {
         if (!is_tile(q)) return;
-        const unsigned long long a = LEAVES ? src & ~15ull : src;
-        bulk_load(stage, reinterpret_cast<const void*>(a), (LEAVES && a != src) ? kTile + 16u : kTile, &tc->mbar, pol_once);
+        const unsigned long long a = (LEAVES ? src & ~15ull : src) + kShare * (2u * warp + part);
+        bulk_load_at(stage_s, reinterpret_cast<const void*>(a), (LEAVES && (src & 15ull)) ? kShare + 16u : kShare, bar_s, pol_once);
     };
     // leaf mode, handing a claimed tile on: its word carries the start's remainder
     auto with_mark = [](uint32_t q, unsigned long long addr) {
         return (!LEAVES || (int32_t)q < 0) ? q : q | (((uint32_t)addr & 15u) << kQOffShift);
     };
 
-    // Tiles in flight, oldest first: X (packed in this step), V, W (waiting for their offsets),
-    // Y (measured in this step).  Ring slots of the widths: X = sl, V = sl+1, W = sl+2, Y = sl+3
-    // (mod 8); tensor memory slots: Y = step mod 4, X = (step + 1) mod 4 (where it was put three
-    // steps ago).
-    uint32_t qX = kQNone, qV = kQNone, qW = kQNone, qY = kQNone;
-    uint32_t sl = 0;
-    uint32_t par = 0;                  // step parity (selects next[] / excl[])
+    // Tiles in flight, oldest first: X (packed in this step), W (its length goes out), Y (measured in
+    // this step).  Y's results go to the tables' slot step mod 4 and to tensor memory slot step mod 2.
+    uint32_t qX = kQNone, qW = kQNone, qY = kQNone;
     uint32_t step = 0;
-    uint32_t d[kWordsPerLane];
     bool claiming = false;             // leader: the last ticket it claimed was a tile
 
-    // ---- prologue: the tiles of the first two steps are claimed, the first one's copy started.
-    // Leaf mode claims one step further ahead: a tile's address is looked up in the step between
-    // its claim and its hand-over, so that the leader never waits for that answer either.
-    uint32_t qA = kQNone;              // leader, leaf mode: claimed and described, address on its way
-    uint32_t kA = 0;                   // ... and its ticket
-    // With a mask (flat cache) a ticket's tile is found through the list of present chunks.  That
-    // look-up too is started in the step after the claim and used at that step's end, so a ticket
-    // is handed over one step later than without a mask and the leader claims one step further ahead.
-    constexpr bool kLateList = MASKED && !LEAVES;
-    bool haveA = false;                // leader, kLateList: ticket kA is a tile and waits for its chunk number
+    // ---- prologue: the tiles of the first two steps are claimed.  (With few tiles only the first one:
+    // a team that takes two while another gets none is the slower way to share them out.)
     if (leader) {
-        mbar_init(&tc->mbar, 1);
-        const uint32_t k0 = next_ticket(ws.ctrl);
+        const bool many = n_hot > 2u * kEncTeams * gridDim.x;
+        const uint32_t teams = (n_hot + gridDim.x - 2u) / (gridDim.x - 1u);       // per block, when every tile has one
+        uint32_t k0 = 0xFFFFFFFFu, k1 = 0xFFFFFFFFu;
+        if (many || team < teams) k0 = next_ticket(ws.ctrl);
         const uint32_t q0 = describe_tile<MASKED>(g, ws.plist, n_hot, k0);
-        const uint32_t k1 = is_tile(q0) ? next_ticket(ws.ctrl) : 0xFFFFFFFFu;
-        const uint32_t q1 = is_tile(q0) ? describe_tile<MASKED>(g, ws.plist, n_hot, k1) : kQNone;
-        claiming = is_tile(q1);
-        if (MASKED) { tc->kring[3] = k0; tc->kring[4] = k1; }      // the slots in which they will be measured
+        if (many) k1 = next_ticket(ws.ctrl);
+        const uint32_t q1 = describe_tile<MASKED>(g, ws.plist, n_hot, k1);
+        claiming = is_tile(many ? q1 : q0);
+        if (MASKED) { tc->kring[0] = k0; tc->kring[1] = k1; }      // the steps in which they will be measured
         tc->next[0] = q0;
         tc->next[1] = q1;
         tc->excl[0] = 0ull;
@@ -548,150 +539,54 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             tc->nptr[1] = is_tile(q1) ? tile_src(q1 & kQTile) : 0ull;
             tc->next[0] = with_mark(q0, tc->nptr[0]);
             tc->next[1] = with_mark(q1, tc->nptr[1]);
-            if (claiming) { kA = next_ticket(ws.ctrl); qA = describe_tile<MASKED>(g, ws.plist, n_hot, kA); claiming = is_tile(qA); }
         }
-        if (kLateList && claiming) { kA = next_ticket(ws.ctrl); claiming = haveA = kA < n_hot; }
     }
-    team_bar(team);
+    if (lane == 0) mbar_init(&tc->mbar[warp], 1);
+    if (tt == 96u) mbar_init(&tc->measured, 4);
+    enc_team_bar(team);
     qY = tc->next[0];
-    if (leader) start_copy(qY, LEAVES ? tc->nptr[0] : tile_src(qY & kQTile));
+    unsigned long long srcY = LEAVES ? tc->nptr[0] : 0ull;      // leaf mode: where Y begins
+    if (lane == 0) start_copy(qY, LEAVES ? srcY : tile_src(qY & kQTile), 0);
 
     uint32_t trouble = 0;              // sticky: the image does not fit
-    while (is_tile(qX & qV & qW & qY)) {
-        const bool hotY = is_tile(qY);
-        if (hotY) {
-            wait_for_copy<!ENT>(&tc->mbar, phase, g.wait_ns, ws.ctrl);
-            phase ^= 1u;
-            // leaf mode: a tile that was copied from the 16-byte boundary below it starts that many
-            // bytes into the stage: whole words from a quarter of that on, each put together from two
-            // neighbours when the remainder is no multiple of four
-            const uint32_t off = LEAVES ? (qY >> kQOffShift) & 15u : 0u;
-            const uint32_t sh = (off & 3u) * 8u;
-            const uint32_t* const p = my_words + (off >> 2);
-            if (LEAVES && sh) {
-#pragma unroll
-                for (int i = 0; i < 16; i++) d[i] = __funnelshift_r(p[i * 32], p[i * 32 + 1], sh);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 16; i++) d[i] = p[i * 32];
-            }
-        }
-        team_bar(team);                   // stage free; what the leader left at the end of the last step is visible
+    uint32_t d[kWordsPerLane];
+    while (is_tile(qX & qW & qY)) {
+        enc_team_bar(team);            // W's widths and digests are complete; what was handed over in the last step is visible
+        const uint32_t par = step & 1u;
+        const uint32_t slX = (step - 2u) & 3u, slW = (step - 1u) & 3u, slY = step & 3u;
         const uint32_t qN = tc->next[par ^ 1u];
         const unsigned long long exclX = tc->excl[par ^ 1u];
-        // The tile measured in the last step (W now): its 32 widths are complete behind the barrier.
-        // One warp that has no other single-lane chore adds them up and publishes the tile's length
-        // (half a step later than the last-arriving warp could have, which the three steps of slack
-        // before the tile is packed absorb; but no warp waits for a counter in the measuring step
-        // and the sum is off the path of whichever warp was slowest there).
-        if (warp == 6u && is_tile(qW)) {
-            const uint32_t slW = (sl + 2u) & 7u;
-            const uint32_t wt = tc->wtab[slW][lane];
-            const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u);
-            // entropy option: the ENT form is taken when it is shorter than the planes and than raw
-            uint32_t ent_words = 0;
-            if (ENT) ent_words = __reduce_add_sync(0xFFFFFFFFu, lane < 8u ? tc->etab[slW][lane] >> 8 : 0u);
-            const uint32_t plane_len = total <= 253u ? 8256u + 32u * total : kTile;
-            const bool ent_tile = ENT && ent_tile_bytes(ent_words) < plane_len;
-            // unused memory (every warp's first entry carries the mark): no payload
-            // (one value throughout: every warp's first entry carries the mark and they are all alike;
-            // a tile of zeros has no payload, any other value 32 bytes)
-            const uint32_t wt0 = __shfl_sync(0xFFFFFFFFu, wt, 0);
-            const bool const_tile = ZEROS && __all_sync(0xFFFFFFFFu, (lane & 3u) != 0u || ((wt & kWarpConst) != 0u && wt == wt0));
-            const bool zero_tile = const_tile && (wt0 & kWarpAllZero) != 0u;
-            if (lane == 0) {
-                tc->ssum[slW] = zero_tile ? kSumZeroTile : const_tile ? kSumConstTile : ent_tile ? kSumEnt | ent_words : total;
-                publish_len(slW, qW & kQTile, zero_tile ? 0u : const_tile ? 32u : ent_tile ? ent_tile_bytes(ent_words) : plane_len);
-            }
-        }
-        // The team's single-lane chores are spread over its warps, because the team waits for
-        // whichever warp has the most to do.  Warp 2 starts the copy of the next tile (it has the
-        // whole step to arrive).  Two round trips to L2 are started now and used at the end of the
-        // step: the ticket of the tile to measure two steps on (warp 0, the leader) and the offset
-        // of the tile to pack in the next step (warp 3).  Warp 1 notes what is left about X.
-        uint32_t pv = 0, tk = 0xFFFFFFFFu;
-        unsigned long long pA = 0;
-        if (tt == 64u) start_copy(qN, LEAVES ? tc->nptr[par ^ 1u] : tile_src(qN & kQTile));
-        if (tt == 96u && is_tile(qV)) pv = ld_relaxed_u32(ws.lbk + place_of((sl + 1u) & 7u, qV & kQTile));
-        uint32_t plA = 0;
-        if (leader) {
-            if (claiming) tk = next_ticket(ws.ctrl);
-            if (LEAVES && is_tile(qA)) pA = tile_src(qA & kQTile);
-            if (kLateList && haveA) plA = __ldg(ws.plist + chunk_of(g, kA));
-        }
+        const unsigned long long srcN = LEAVES ? tc->nptr[par ^ 1u] : 0ull;
 
-        // ---- Y: digest, exponent ranges, length out, words parked
-        const uint32_t slY = (sl + 3u) & 7u;
-        if (hotY) {
-            const uint32_t v = tile_digest_block(S, d, (qY & kQFirst) != 0, warp, lane);
-            // From here on the words are kept rotated left by one bit: each half then reads
-            // [E | mantissa | a sign bit], E in its high byte (the two sign bits of a word
-            // land in each other's half; the packing step puts them right).
-#pragma unroll
-            for (int i = 0; i < 16; i++) d[i] = __funnelshift_l(d[i], d[i], 1);
-            uint32_t gw[4];               // per group: base | width << 8
-            uint32_t ent_w = 0;           // entropy option: anchor | words << 8 of this warp's share
-            if (ENT) {
-                // the share's anchor (rounded mean of its 1024 exponents: bytes 1 and 3 of a rotated
-                // word), every strand's length in bits and the words the share's stream needs
-                uint32_t acc = 0;
-#pragma unroll
-                for (int i = 0; i < 16; i++) acc = __dp4a(d[i], 0x01000100u, acc);       // bytes 1 and 3
-                const uint32_t anchor = (__reduce_add_sync(0xFFFFFFFFu, acc) + 512u) >> 10;
-                uint32_t bits = 0;
-                const uint32_t lb = lenE_s - anchor;
-#pragma unroll
-                for (int i = 0; i < 16; i++)
-                    bits += lds_tab_u8(lb + __byte_perm(d[i], 0u, 0x4441)) + lds_tab_u8(lb + (d[i] >> 24));
-                // (a strand the length byte cannot hold, above 319 bits, keeps the tile out of the form:
-                // the count is then so large that the form is never the shortest)
-                const uint32_t share_bits = __reduce_add_sync(0xFFFFFFFFu, bits);
-                const bool too_long = __any_sync(0xFFFFFFFFu, bits > 319u);
-                tc->sbits[step & 3u][32u * warp + lane] = (unsigned char)(bits - 64u);
-                ent_w = anchor | ((too_long ? 0xFFFFu : (share_bits + 31u) >> 5) << 8);
-            }
-            {
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint32_t a0 = d[4 * j], a1 = d[4 * j + 1], a2 = d[4 * j + 2], a3 = d[4 * j + 3];
-                uint32_t mn = min_u16x2(min_u16x2(a0, a1), min_u16x2(a2, a3));
-                uint32_t mx = max_u16x2(max_u16x2(a0, a1), max_u16x2(a2, a3));
-                // both halves get the smaller (larger) of the two, so that the word as a whole
-                // orders like its halves and one warp reduction per bound does
-                mn = min_u16x2(mn, __byte_perm(mn, mn, 0x1032));
-                mx = max_u16x2(mx, __byte_perm(mx, mx, 0x1032));
-                const uint32_t emin = __reduce_min_sync(0xFFFFFFFFu, mn) >> 24;
-                const uint32_t emax = __reduce_max_sync(0xFFFFFFFFu, mx) >> 24;
-                gw[j] = emin | ((32u - __clz(emax - emin)) << 8);
-            }
-            }
-            // Option ZEROS.  Unused memory: when all four groups have exponent 0 throughout (rare in live data)
-            // look at the words themselves; a warp whose 2 KiB are all zero marks its first entry.
-            // The same for any one value (a mask fill, say): all four groups have one exponent and width
-            // 0; then every word must equal the warp's first, and that word's two halves each other.
-            if (ZEROS && gw[0] < 256u && gw[1] == gw[0] && gw[2] == gw[0] && gw[3] == gw[0]) {
-                const uint32_t first = __shfl_sync(0xFFFFFFFFu, d[0], 0);
-                uint32_t diff = (first >> 16) ^ (first & 0xFFFFu);
-#pragma unroll
-                for (int i = 0; i < 16; i++) diff |= d[i] ^ first;
-                if (!__any_sync(0xFFFFFFFFu, diff != 0u))
-                    gw[0] |= kWarpConst | ((first & 0xFFu) << 16) | (first == 0u ? kWarpAllZero : 0u);
-            }
-            // one lane leaves the warp's results; the tile's length is added up and published right
-            // after the next barrier, when all eight warps' widths are there (see the top of the step)
-            if (lane == 0) {
-                tc->wdig[slY][warp] = v;
-                *reinterpret_cast<uint4*>(&tc->wtab[slY][4 * warp]) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
-                if (ENT) tc->etab[slY][warp] = ent_w;
-            }
-            tmem_store16(tmem_warp + 16u * (step & 3u), d);
+        // ---- W: warp 1 puts its digest together
+        if (warp == 1u && is_tile(qW)) {
+            const uint32_t v = place_team4_digests(S, tc_s + (uint32_t)offsetof(EncTeamCtl, wdig) + 16u * slW, lane);
+            if (lane == 0) ws.dig[qW & kQTile] = v;
         }
+        // Round trips to L2 are under way during a step whose answers are taken at its end: W's offset (asked
+        // for by warp 2 in front of Y's second share) and the ticket of the tile to measure two steps on
+        // (the leader).  Tickets are claimed as late as that allows: the time from a claim to the tile's
+        // length, times how unevenly the teams run, is what an offset waits for.  With a mask or leaves a
+        // ticket is looked up once more (its chunk's number, its address): it is claimed at the start of
+        // the step and looked up where the others are claimed.
+        uint32_t pv = 0, tk = 0xFFFFFFFFu, qC = kQNone, plA = 0;
+        unsigned long long pA = 0;
+        if ((MASKED || LEAVES) && leader && claiming) tk = next_ticket(ws.ctrl);
+        auto ask = [&]() {
+            if (tt == 64u && is_tile(qW)) pv = ld_relaxed_u32(ws.lbk + place_of(step - 1u, qW));
+            if (leader && claiming) {
+                if (!MASKED && !LEAVES) {
+                    tk = next_ticket(ws.ctrl);
+                } else if (tk < n_hot) {
+                    if (LEAVES) { qC = describe_tile<MASKED>(g, ws.plist, n_hot, tk); pA = tile_src(qC & kQTile); }
+                    else plA = __ldg(ws.plist + chunk_of(g, tk));
+                }
+            }
+        };
 
         // ---- X: its words back from tensor memory, packed straight into the wire image
-        const uint32_t tXn = qX & kQTile;
         if (is_tile(qX)) {
-            tmem_load16(tmem_warp + 16u * ((step + 1u) & 3u), d);
-            const uint32_t Smark = tc->ssum[sl];
+            const uint32_t Smark = tc->ssum[slX];
             const bool ent_form = ENT && (Smark & kSumEnt) != 0u;
             const uint32_t Ssum = ent_form ? Smark & 0xFFFFu : Smark;       // words of the streams, or the sum of the widths
             const bool packs = !ent_form && Ssum <= 253u;
@@ -700,13 +595,14 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                                          : packs ? 8256u + 32u * Ssum : (ZEROS && Ssum == kSumZeroTile) ? 0u
                                          : (ZEROS && Ssum == kSumConstTile) ? 32u : kTile;
             unsigned char* const dst = payload + exclX;
+            tmem_wait_stores();
             if (exclX + enc_len > room) {
                 trouble |= 1u;
             } else if (ent_form) {
                 // header: anchors, word counts, 40 zero bytes; zero fill behind the last stream
-                if (warp == 5) {
+                if (warp == 2u) {
                     if (lane < 8u) {
-                        const uint32_t wt = tc->etab[sl][lane];
+                        const uint32_t wt = tc->etab[slX][lane];
                         stg_u8(dst + lane, wt & 0xFFu);
                         stg_u16(dst + 8u + 2u * lane, wt >> 8);
                     } else if (lane < 18u) {
@@ -714,110 +610,115 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                     }
                     if (4u * lane < enc_len - 8512u - 4u * Ssum) st_stream_u32(dst + 8512u + 4u * Ssum + 4u * lane, 0u);
                 }
-                unsigned char* const sm_dst = dst + sm_off;
+#pragma unroll 1
+                for (uint32_t part = 0; part < 2u; part++) {
+                    const uint32_t share = 2u * warp + part;
+                    tmem_load16(tmem_warp + 32u * par + 16u * part, d);
+                    unsigned char* const sm_dst = dst + 64u + 1024u * share + 8u * lane;
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint32_t sa = __byte_perm(d[4 * j], d[4 * j + 1], 0x6420), sb = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x6420);
-                    const uint32_t ya = __byte_perm(sa, sa, 0x2301), yb = __byte_perm(sb, sb, 0x2301);
-                    stg_v2(sm_dst + 256 * j, (sa & 0xFEFEFEFEu) | (ya & 0x01010101u), (sb & 0xFEFEFEFEu) | (yb & 0x01010101u));
-                }
-                // This share's stream starts behind the streams of the warps before it; inside it the
-                // strands follow one another bit by bit, so lane l starts where the lengths of the
-                // lanes before it (measured three steps ago) add up to.
-                const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? tc->etab[sl][lane] >> 8 : 0u);
-                const uint32_t anchor = tc->etab[sl][warp] & 0xFFu;
-                const uint32_t nb8 = tc->sbits[(step + 1u) & 3u][32u * warp + lane];
-                stg_u8(dst + 8256u + 32u * warp + lane, nb8);
-                uint32_t incl = 64u + nb8;
-#pragma unroll
-                for (int k = 1; k < 32; k <<= 1) {
-                    const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, k);
-                    if (lane >= (uint32_t)k) incl += o;
-                }
-                const uint32_t start = incl - 64u - nb8;
-                unsigned char* const w_dst = dst + 8512u + 4u * before;
-                // acc: the stream's bits from the last word boundary on, n of them valid (the first n
-                // of the lane's first word belong to the lane before it).  Two codewords are joined
-                // first (32 bits at most) and go in together; both shifts are multiplications by a
-                // power of two from the table or from n (one multiply-add each, on the pipe that has
-                // little else to do here, where the shifts and ORs would queue up with everything
-                // else).  Words go out as they fill up, except the lane's first one, which is held
-                // back until the lane before has handed over the bits it left in it.
-                unsigned long long acc = 0;
-                uint32_t n = start & 31u, wp = start >> 5, w_first = 0;
-                bool have_first = false;
-                const uint32_t lb = lenE_s - anchor, cb = cwE_s - 2u * anchor;
-#pragma unroll
-                for (int i = 0; i < 16; i++) {
-                    const uint32_t E0 = __byte_perm(d[i], 0u, 0x4441), E1 = d[i] >> 24;
-                    const uint32_t len0 = lds_tab_u8(lb + E0), len1 = lds_tab_u8(lb + E1);
-                    // (the table's escape entry is 0xFFFF: the AND lets the exponent through there only)
-                    const uint32_t c0 = lds_tab_u16(cb + 2u * E0) & __byte_perm(E0, 0xFFu, 0x4404);
-                    const uint32_t c1 = lds_tab_u16(cb + 2u * E1) & __byte_perm(E1, 0xFFu, 0x4404);
-                    const uint32_t pair = c1 * (1u << len0) + c0;
-                    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(pair), "r"(1u << n));
-                    n += len0 + len1;
-                    if (n >= 32u) {                        // (two codewords are 32 bits at most: one word per pair)
-                        const uint32_t word = (uint32_t)acc;
-                        if (have_first) st_stream_u32(w_dst + 4u * wp, word); else w_first = word;
-                        have_first = true;
-                        acc >>= 32;
-                        n -= 32u;
-                        wp++;
+                    for (int j = 0; j < 4; j++) {
+                        const uint32_t sa = __byte_perm(d[4 * j], d[4 * j + 1], 0x6420), sb = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x6420);
+                        const uint32_t ya = __byte_perm(sa, sa, 0x2301), yb = __byte_perm(sb, sb, 0x2301);
+                        stg_v2(sm_dst + 256 * j, (sa & 0xFEFEFEFEu) | (ya & 0x01010101u), (sb & 0xFEFEFEFEu) | (yb & 0x01010101u));
                     }
+                    // This share's stream starts behind the streams of the shares before it; inside it the
+                    // strands follow one another bit by bit, so lane l starts where the lengths of the
+                    // lanes before it (measured two steps ago) add up to.
+                    const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < share ? tc->etab[slX][lane] >> 8 : 0u);
+                    const uint32_t anchor = tc->etab[slX][share] & 0xFFu;
+                    const uint32_t nb8 = tc->sbits[par][32u * share + lane];
+                    stg_u8(dst + 8256u + 32u * share + lane, nb8);
+                    uint32_t incl = 64u + nb8;
+#pragma unroll
+                    for (int k = 1; k < 32; k <<= 1) {
+                        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, k);
+                        if (lane >= (uint32_t)k) incl += o;
+                    }
+                    const uint32_t start = incl - 64u - nb8;
+                    unsigned char* const w_dst = dst + 8512u + 4u * before;
+                    // acc: the stream's bits from the last word boundary on, n of them valid (the first n
+                    // of the lane's first word belong to the lane before it).  Two codewords are joined
+                    // first (32 bits at most) and go in together; both shifts are multiplications by a
+                    // power of two from the table or from n (one multiply-add each, on the pipe that has
+                    // little else to do here, where the shifts and ORs would queue up with everything
+                    // else).  Words go out as they fill up, except the lane's first one, which is held
+                    // back until the lane before has handed over the bits it left in it.
+                    unsigned long long acc = 0;
+                    uint32_t n = start & 31u, wp = start >> 5, w_first = 0;
+                    bool have_first = false;
+                    const uint32_t lb = lenE_s - anchor, cb = cwE_s - 2u * anchor;
+#pragma unroll
+                    for (int i = 0; i < 16; i++) {
+                        const uint32_t E0 = __byte_perm(d[i], 0u, 0x4441), E1 = d[i] >> 24;
+                        const uint32_t len0 = lds_tab_u8(lb + E0), len1 = lds_tab_u8(lb + E1);
+                        // (the table's escape entry is 0xFFFF: the AND lets the exponent through there only)
+                        const uint32_t c0 = lds_tab_u16(cb + 2u * E0) & __byte_perm(E0, 0xFFu, 0x4404);
+                        const uint32_t c1 = lds_tab_u16(cb + 2u * E1) & __byte_perm(E1, 0xFFu, 0x4404);
+                        const uint32_t pair = c1 * (1u << len0) + c0;
+                        asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(pair), "r"(1u << n));
+                        n += len0 + len1;
+                        if (n >= 32u) {                        // (two codewords are 32 bits at most: one word per pair)
+                            const uint32_t word = (uint32_t)acc;
+                            if (have_first) st_stream_u32(w_dst + 4u * wp, word); else w_first = word;
+                            have_first = true;
+                            acc >>= 32;
+                            n -= 32u;
+                            wp++;
+                        }
+                    }
+                    // (a strand is 64 bits at least, so every lane has crossed a word boundary by now)
+                    const uint32_t tail = (uint32_t)acc;                   // n bits of the next word, 0 when n == 0
+                    const uint32_t from_below = __shfl_up_sync(0xFFFFFFFFu, tail, 1);
+                    st_stream_u32(w_dst + 4u * (start >> 5), w_first | (lane ? from_below : 0u));
+                    if (lane == 31u && n) st_stream_u32(w_dst + 4u * wp, tail);
                 }
-                // (a strand is 64 bits at least, so every lane has crossed a word boundary by now)
-                const uint32_t tail = (uint32_t)acc;                   // n bits of the next word, 0 when n == 0
-                const uint32_t from_below = __shfl_up_sync(0xFFFFFFFFu, tail, 1);
-                st_stream_u32(w_dst + 4u * (start >> 5), w_first | (lane ? from_below : 0u));
-                if (lane == 31u && n) st_stream_u32(w_dst + 4u * wp, tail);
             } else if (packs) {
-                if (warp == 5) {           // (any one warp: not one that has a single-lane chore)
-                    const uint32_t wt = tc->wtab[sl][lane];
+                if (warp == 2u) {
+                    const uint32_t wt = tc->wtab[slX][lane];
                     stg_u16(dst + 2 * lane, desc_of(wt & 0xFFu, (wt >> 8) & 15u));
                 }
-                unsigned char* const sm_dst = dst + sm_off;
-                unsigned char* const pl_dst = dst + 8256;
                 // widths of all 32 groups (one per lane): 32-byte units before this warp's first group
-                const uint32_t wall = (tc->wtab[sl][lane] >> 8) & 15u;
-                uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < 4u * warp ? wall : 0u);
-                const uint4 g4 = *reinterpret_cast<const uint4*>(&tc->wtab[sl][4 * warp]);
-                const uint32_t gq[4] = {g4.x, g4.y, g4.z, g4.w};
+                const uint32_t wall = (tc->wtab[slX][lane] >> 8) & 15u;
+                unsigned char* rec = dst + 8256u + 32u * __reduce_add_sync(0xFFFFFFFFu, lane < 8u * warp ? wall : 0u);
+                unsigned char* sm_dst = dst + 64u + 2048u * warp + 8u * lane;      // this lane's place in a group's sign-mantissa run
+#pragma unroll 1
+                for (uint32_t part = 0; part < 2u; part++) {
+                    tmem_load16(tmem_warp + 32u * par + 16u * part, d);
+                    const uint4 g4 = *reinterpret_cast<const uint4*>(&tc->wtab[slX][8u * warp + 4u * part]);
+                    const uint32_t gq[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint32_t wtg = gq[j];
-                    const uint32_t base = wtg & 0xFFu, wd = (wtg >> 8) & 15u;
-                    // bytes 0 and 2 of a rotated word: mantissa << 1 | the other element's sign;
-                    // bytes 1 and 3: the exponents.  Gather, then swap bit 0 inside byte pairs.
-                    const uint32_t sa = __byte_perm(d[4 * j], d[4 * j + 1], 0x6420), sb = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x6420);
-                    const uint32_t ya = __byte_perm(sa, sa, 0x2301), yb = __byte_perm(sb, sb, 0x2301);
-                    stg_v2(sm_dst + 256 * j, (sa & 0xFEFEFEFEu) | (ya & 0x01010101u), (sb & 0xFEFEFEFEu) | (yb & 0x01010101u));
-                    const uint32_t e4a = __byte_perm(d[4 * j], d[4 * j + 1], 0x7531), e4b = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x7531);
-                    unsigned char* rec = pl_dst + 32u * before;
-                    before += wd;
-                    pack_group(wd, e4a, e4b, base, rec, lane);
+                    for (int j = 0; j < 4; j++) {
+                        const uint32_t wtg = gq[j];
+                        const uint32_t base = wtg & 0xFFu, wd = (wtg >> 8) & 15u;
+                        // bytes 0 and 2 of a rotated word: mantissa << 1 | the other element's sign;
+                        // bytes 1 and 3: the exponents.  Gather, then swap bit 0 inside byte pairs.
+                        const uint32_t sa = __byte_perm(d[4 * j], d[4 * j + 1], 0x6420), sb = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x6420);
+                        const uint32_t ya = __byte_perm(sa, sa, 0x2301), yb = __byte_perm(sb, sb, 0x2301);
+                        stg_v2(sm_dst + 256 * j, (sa & 0xFEFEFEFEu) | (ya & 0x01010101u), (sb & 0xFEFEFEFEu) | (yb & 0x01010101u));
+                        const uint32_t e4a = __byte_perm(d[4 * j], d[4 * j + 1], 0x7531), e4b = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x7531);
+                        pack_group(wd, e4a, e4b, base, rec, lane);
+                        rec += 32u * wd;
+                    }
+                    sm_dst += 1024;
                 }
             } else if (ZEROS && Ssum == kSumConstTile) {
                 // the value (any word's low half, rotated back), then 30 zero bytes
-                if (warp == 5 && lane < 8u) st_stream_u32(dst + 4u * lane, lane == 0u ? __funnelshift_r(d[0], d[0], 1) & 0xFFFFu : 0u);
+                tmem_load16(tmem_warp + 32u * par, d);
+                if (warp == 2u && lane < 8u) st_stream_u32(dst + 4u * lane, lane == 0u ? __funnelshift_r(d[0], d[0], 1) & 0xFFFFu : 0u);
             } else if (enc_len) {
-                unsigned char* q = dst + warp * 2048u + lane * 4u;
+#pragma unroll 1
+                for (uint32_t part = 0; part < 2u; part++) {
+                    tmem_load16(tmem_warp + 32u * par + 16u * part, d);
+                    unsigned char* q = dst + (2u * warp + part) * kShare + lane * 4u;
 #pragma unroll
-                for (int i = 0; i < 16; i++) st_stream_u32(q + i * 128, __funnelshift_r(d[i], d[i], 1));
+                    for (int i = 0; i < 16; i++) st_stream_u32(q + i * 128, __funnelshift_r(d[i], d[i], 1));
+                }
             }
         }
-
-        // What is left to note about X is done by two other warps' first lanes (the leader's
-        // warp is the one the team waits for): the digest by warp 1; the table entry, where its
-        // chunk starts and the total by warp 7 (not warp 4: warps w and w + 4 issue through the same
-        // scheduler, and warp 4 would share the end of the step with the leader's hand-over).
-        if (warp == 1u && is_tile(qX)) {
-            const uint32_t v = place_warp_digests(S, (uint32_t)__cvta_generic_to_shared(tc->wdig[sl]), lane);
-            if (lane == 0) ws.dig[tXn] = v;
-        }
-        if (tt == 224u && is_tile(qX)) {
+        // What is left to note about X: the table entry, where its chunk starts, the total.
+        if (tt == 32u && is_tile(qX)) {
+            const uint32_t tXn = qX & kQTile, Ssum = tc->ssum[slX];
             uint32_t entry, enc_len;
-            const uint32_t Ssum = tc->ssum[sl];
             if (ENT && (Ssum & kSumEnt)) {
                 enc_len = ent_tile_bytes(Ssum & 0xFFFFu);
                 entry = 0x8000u | (enc_len / 32u);
@@ -825,45 +726,160 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 entry = Ssum <= 253u ? 258u + Ssum : (ZEROS && Ssum == kSumZeroTile) ? 1u : (ZEROS && Ssum == kSumConstTile) ? 2u : 512u;
                 enc_len = (ZEROS && entry <= 2u) ? 32u * (entry - 1u) : 32u * entry;
             }
-            tile_tab[tXn] = (uint16_t)entry;
-            if (qX & kQFirst) *reinterpret_cast<unsigned long long*>(dir + 16ull * chunk_of(g, tXn)) = exclX;
-            if (place_of(sl, tXn) + 1 == n_tickets) ws.ctrl->payload_total = exclX + enc_len;
+            reinterpret_cast<uint16_t*>(wire + 64 + 16ull * g.n_chunks)[tXn] = (uint16_t)entry;
+            if (qX & kQFirst) *reinterpret_cast<unsigned long long*>(wire + 64 + 16ull * chunk_of(g, tXn)) = exclX;
+            if (place_of(step - 2u, qX) + 1 == n_tickets) ws.ctrl->payload_total = exclX + enc_len;
         }
-        if (leader && kLateList) {     // hand over the ticket whose chunk number arrived during this step
+        // ---- Y: digest, exponent ranges, words parked, a share at a time
+        if (is_tile(qY)) {
+            uint32_t st = ((qY & kQFirst) && tt == 0u) ? 0xFFFFFFFFu : 0u;      // (the all-ones start value complements the chunk's first word)
+#pragma unroll 1
+            for (uint32_t part = 0; part < 2u; part++) {
+                const uint32_t share = 2u * warp + part;
+                wait_for_copy_at<!ENT>(bar_s, phase, g.wait_ns, ws.ctrl);
+                phase ^= 1u;
+                // leaf mode: a tile that was copied from the 16-byte boundary below it starts that many
+                // bytes into the stage: whole words from a quarter of that on, each put together from two
+                // neighbours when the remainder is no multiple of four
+                const uint32_t off = LEAVES ? (qY >> kQOffShift) & 15u : 0u;
+                const uint32_t sh = (off & 3u) * 8u;
+                if (LEAVES && sh) {
+                    const uint32_t* const p = reinterpret_cast<const uint32_t*>(stages + wc * kStage + (off & 12u)) + lane;
+#pragma unroll
+                    for (int i = 0; i < 16; i++) d[i] = __funnelshift_r(p[i * 32], p[i * 32 + 1], sh);
+                } else {
+                    read_staged_words_at(stage_s + (off & 12u), 0u, lane, d);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    if (part == 0u) start_copy(qY, LEAVES ? srcY : tile_src(qY & kQTile), 1u);
+                    else start_copy(qN, LEAVES ? srcN : tile_src(qN & kQTile), 0u);
+                }
+                if (part) {
+                    ask();
+                    st = chain_step(S, st);
+                }
+#pragma unroll
+                for (int i = 0; i < 15; i++) st = chain_step(S, st ^ d[i]);
+                st ^= d[15];
+                // From here on the words are kept rotated left by one bit: each half then reads
+                // [E | mantissa | a sign bit], E in its high byte (the two sign bits of a word
+                // land in each other's half; the packing step puts them right).
+#pragma unroll
+                for (int i = 0; i < 16; i++) d[i] = __funnelshift_l(d[i], d[i], 1);
+                uint32_t gw[4];               // per group: base | width << 8
+                uint32_t ent_w = 0;           // entropy option: anchor | words << 8 of this share
+                if (ENT) {
+                    // the share's anchor (rounded mean of its 1024 exponents: bytes 1 and 3 of a rotated
+                    // word), every strand's length in bits and the words the share's stream needs
+                    uint32_t acc = 0;
+#pragma unroll
+                    for (int i = 0; i < 16; i++) acc = __dp4a(d[i], 0x01000100u, acc);       // bytes 1 and 3
+                    const uint32_t anchor = (__reduce_add_sync(0xFFFFFFFFu, acc) + 512u) >> 10;
+                    uint32_t bits = 0;
+                    const uint32_t lb = lenE_s - anchor;
+#pragma unroll
+                    for (int i = 0; i < 16; i++)
+                        bits += lds_tab_u8(lb + __byte_perm(d[i], 0u, 0x4441)) + lds_tab_u8(lb + (d[i] >> 24));
+                    // (a strand the length byte cannot hold, above 319 bits, keeps the tile out of the form:
+                    // the count is then so large that the form is never the shortest)
+                    const uint32_t share_bits = __reduce_add_sync(0xFFFFFFFFu, bits);
+                    const bool too_long = __any_sync(0xFFFFFFFFu, bits > 319u);
+                    tc->sbits[par][32u * share + lane] = (unsigned char)(bits - 64u);
+                    ent_w = anchor | ((too_long ? 0xFFFFu : (share_bits + 31u) >> 5) << 8);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const uint32_t a0 = d[4 * j], a1 = d[4 * j + 1], a2 = d[4 * j + 2], a3 = d[4 * j + 3];
+                    uint32_t mn = min_u16x2(min_u16x2(a0, a1), min_u16x2(a2, a3));
+                    uint32_t mx = max_u16x2(max_u16x2(a0, a1), max_u16x2(a2, a3));
+                    // both halves get the smaller (larger) of the two, so that the word as a whole
+                    // orders like its halves and one warp reduction per bound does
+                    mn = min_u16x2(mn, __byte_perm(mn, mn, 0x1032));
+                    mx = max_u16x2(mx, __byte_perm(mx, mx, 0x1032));
+                    const uint32_t emin = __reduce_min_sync(0xFFFFFFFFu, mn) >> 24;
+                    const uint32_t emax = __reduce_max_sync(0xFFFFFFFFu, mx) >> 24;
+                    gw[j] = emin | ((32u - __clz(emax - emin)) << 8);
+                }
+                // Option ZEROS.  Unused memory: when all four groups have exponent 0 throughout (rare in live data)
+                // look at the words themselves; a share whose 2 KiB are all zero marks its first entry.
+                // The same for any one value (a mask fill, say): all four groups have one exponent and width
+                // 0; then every word must equal the share's first, and that word's two halves each other.
+                if (ZEROS && gw[0] < 256u && gw[1] == gw[0] && gw[2] == gw[0] && gw[3] == gw[0]) {
+                    const uint32_t first = __shfl_sync(0xFFFFFFFFu, d[0], 0);
+                    uint32_t diff = (first >> 16) ^ (first & 0xFFFFu);
+#pragma unroll
+                    for (int i = 0; i < 16; i++) diff |= d[i] ^ first;
+                    if (!__any_sync(0xFFFFFFFFu, diff != 0u))
+                        gw[0] |= kWarpConst | ((first & 0xFFu) << 16) | (first == 0u ? kWarpAllZero : 0u);
+                }
+                if (lane == 0) {
+                    *reinterpret_cast<uint4*>(&tc->wtab[slY][4u * share]) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
+                    if (ENT) tc->etab[slY][share] = ent_w;
+                }
+                tmem_store16(tmem_warp + 32u * par + 16u * part, d);
+            }
+            const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, st));
+            if (lane == 0) {
+                tc->wdig[slY][warp] = v;
+                mbar_arrive_at(tc_s + (uint32_t)offsetof(EncTeamCtl, measured));
+            }
+            // Warp 3 adds up the 32 widths and publishes the tile's length as soon as all four warps have
+            // measured, not behind the next team barrier: that one waits for W's offset, and an offset that
+            // comes late must not hold back a length that other teams' offsets are waiting for.
+            if (warp == 3u) {
+                wait_for_copy_at<true>(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase, g.wait_ns, ws.ctrl);
+                measured_phase ^= 1u;
+                const uint32_t wt = tc->wtab[slY][lane];
+                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u);
+                // entropy option: the ENT form is taken when it is shorter than the planes and than raw
+                uint32_t ent_words = 0;
+                if (ENT) ent_words = __reduce_add_sync(0xFFFFFFFFu, lane < 8u ? tc->etab[slY][lane] >> 8 : 0u);
+                const uint32_t plane_len = total <= 253u ? 8256u + 32u * total : kTile;
+                const bool ent_tile = ENT && ent_tile_bytes(ent_words) < plane_len;
+                // unused memory (every share's first entry carries the mark): no payload
+                // (one value throughout: every share's first entry carries the mark and they are all alike;
+                // a tile of zeros has no payload, any other value 32 bytes)
+                const uint32_t wt0 = __shfl_sync(0xFFFFFFFFu, wt, 0);
+                const bool const_tile = ZEROS && __all_sync(0xFFFFFFFFu, (lane & 3u) != 0u || ((wt & kWarpConst) != 0u && wt == wt0));
+                const bool zero_tile = const_tile && (wt0 & kWarpAllZero) != 0u;
+                if (lane == 0) {
+                    tc->ssum[slY] = zero_tile ? kSumZeroTile : const_tile ? kSumConstTile : ent_tile ? kSumEnt | ent_words : total;
+                    const uint32_t len = zero_tile ? 0u : const_tile ? 32u : ent_tile ? ent_tile_bytes(ent_words) : plane_len;
+                    st_relaxed_u32(ws.lbk + place_of(step, qY), kFlagA | (len / kUnit));
+                }
+            }
+        } else {
+            if (lane == 0) start_copy(qN, LEAVES ? srcN : tile_src(qN & kQTile), 0u);
+            ask();
+        }
+
+        // ---- hand over: the tile to measure two steps on, and W's offset
+        if (leader) {
             uint32_t qn = kQNone;
-            if (haveA) {
-                const uint32_t j = chunk_of(g, kA);
-                qn = (plA * g.tiles_per_chunk + (kA - j * g.tiles_per_chunk)) | (first_in_chunk(g, kA) ? kQFirst : 0u);
+            if (tk < n_hot) {
+                if (LEAVES) {
+                    qn = with_mark(qC, pA);
+                    tc->nptr[par] = pA;
+                } else if (MASKED) {
+                    const uint32_t j = chunk_of(g, tk);
+                    qn = (plA * g.tiles_per_chunk + (tk - j * g.tiles_per_chunk)) | (first_in_chunk(g, tk) ? kQFirst : 0u);
+                } else {
+                    qn = describe_tile<false>(g, ws.plist, n_hot, tk);
+                }
             }
+            claiming = claiming && is_tile(qn);
             tc->next[par] = qn;
-            tc->kring[(sl + 5u) & 7u] = kA;
-            haveA = claiming && tk < n_hot;
-            claiming = haveA;
-            kA = tk;
-        } else if (leader) {
-            uint32_t qn2 = kQNone;
-            if (claiming) { qn2 = describe_tile<MASKED>(g, ws.plist, n_hot, tk); claiming = is_tile(qn2); }
-            // (the tile handed over now is measured two steps on, in ring slot sl + 5)
-            if (LEAVES) {              // hand over the tile whose address arrived during this step
-                tc->next[par] = with_mark(qA, pA);
-                tc->nptr[par] = pA;
-                if (MASKED) tc->kring[(sl + 5u) & 7u] = kA;
-                qA = qn2;
-                kA = tk;
-            } else {
-                tc->next[par] = qn2;
-                if (MASKED) tc->kring[(sl + 5u) & 7u] = tk;
-            }
+            if (MASKED) tc->kring[(step + 2u) & 7u] = tk;
         }
-        if (tt == 96u) {
+        if (tt == 64u) {
             unsigned long long e = 0;
-            if (is_tile(qV))
-                e = (pv >> 30) == 2u ? (unsigned long long)(pv & kValMask) * kUnit : wait_prefix(ws.lbk, place_of((sl + 1u) & 7u, qV & kQTile), ws.ctrl, g.wait_ns);
+            if (is_tile(qW))
+                e = (pv >> 30) == 2u ? (unsigned long long)(pv & kValMask) * kUnit : wait_prefix(ws.lbk, place_of(step - 1u, qW), ws.ctrl, g.wait_ns);
             tc->excl[par] = e;
         }
-        qX = qV; qV = qW; qW = qY; qY = qN;
-        sl = (sl + 1u) & 7u;
-        par ^= 1u;
+        qX = qW; qW = qY; qY = qN;
+        srcY = srcN;
         step++;
     }
     if ((trouble & 1u) && lane == 0) atomicOr(&ws.ctrl->err, 1u);

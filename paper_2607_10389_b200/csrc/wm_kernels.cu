@@ -41,7 +41,6 @@ namespace wm {
 
 // ------------------------------------------------------------------ host side
 
-constexpr int kTeams = 4;        // encode: teams per block (plus the scanner warp)
 constexpr int kTeamsPlain = 4;   // checksum / decode: teams per block
 constexpr uint32_t kStreamTiles = 112;   // checksum: tiles per SM from which a warp takes a tile of its own
 
@@ -88,14 +87,14 @@ static const DeviceState* device_state()
     if (cudaDeviceGetAttribute(&s.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
     const int big = kDynSmem;
     {
-        const void* enc[] = {(const void*)k_encode<kTeams, false, false, false>, (const void*)k_encode<kTeams, true, false, false>,
-                             (const void*)k_encode<kTeams, false, true, false>,  (const void*)k_encode<kTeams, true, true, false>,
-                             (const void*)k_encode<kTeams, false, false, true>,  (const void*)k_encode<kTeams, true, false, true>,
-                             (const void*)k_encode<kTeams, false, true, true>,   (const void*)k_encode<kTeams, true, true, true>,
-                             (const void*)k_encode<kTeams, false, false, false, true>, (const void*)k_encode<kTeams, true, false, false, true>,
-                             (const void*)k_encode<kTeams, false, true, false, true>,  (const void*)k_encode<kTeams, true, true, false, true>,
-                             (const void*)k_encode<kTeams, false, false, true, true>,  (const void*)k_encode<kTeams, true, false, true, true>,
-                             (const void*)k_encode<kTeams, false, true, true, true>,   (const void*)k_encode<kTeams, true, true, true, true>};
+        const void* enc[] = {(const void*)k_encode<false, false, false>, (const void*)k_encode<true, false, false>,
+                             (const void*)k_encode<false, true, false>,  (const void*)k_encode<true, true, false>,
+                             (const void*)k_encode<false, false, true>,  (const void*)k_encode<true, false, true>,
+                             (const void*)k_encode<false, true, true>,   (const void*)k_encode<true, true, true>,
+                             (const void*)k_encode<false, false, false, true>, (const void*)k_encode<true, false, false, true>,
+                             (const void*)k_encode<false, true, false, true>,  (const void*)k_encode<true, true, false, true>,
+                             (const void*)k_encode<false, false, true, true>,  (const void*)k_encode<true, false, true, true>,
+                             (const void*)k_encode<false, true, true, true>,   (const void*)k_encode<true, true, true, true>};
         for (const void* f : enc)
             if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     }
@@ -437,30 +436,31 @@ static wm_status encode_any(const void* cache, const wm_leaf* leaves, uint32_t n
     // one block per SM: one of them scans, the others encode
     // (tiles are claimed by ticket, so any number of blocks gives the same image; a caller that
     // shares the GPU with other work caps it)
-    const uint32_t need = (g.n_tiles + kTeams - 1) / kTeams + 1;
+    // (with few tiles a block runs fewer of its teams, see the kernel's prologue)
+    const uint32_t need = g.n_tiles + 1;
     uint32_t grid = need < (uint32_t)ds->sm_count ? need : (uint32_t)ds->sm_count;
     if (block_cap && grid > block_cap) grid = block_cap;
     {
         MainKernelTimer timer(ds, 2, s);
         const int variant = (dirty ? 1 : 0) | (leaves ? 2 : 0) | (opt_zero ? 4 : 0) | (opt_ent ? 8 : 0);
-        auto go = [&](auto kernel) { launch_after(kernel, grid, kTeams * 256, kDynSmem, s, c, g, dirty, w, wire_cap, ws, ds->tables); };
+        auto go = [&](auto kernel) { launch_after(kernel, grid, kEncTeams * kEncTeamThreads, kDynSmem, s, c, g, dirty, w, wire_cap, ws, ds->tables); };
         switch (variant) {
-            case 0: go(k_encode<kTeams, false, false, false>); break;
-            case 1: go(k_encode<kTeams, true, false, false>); break;
-            case 2: go(k_encode<kTeams, false, true, false>); break;
-            case 3: go(k_encode<kTeams, true, true, false>); break;
-            case 4: go(k_encode<kTeams, false, false, true>); break;
-            case 5: go(k_encode<kTeams, true, false, true>); break;
-            case 6: go(k_encode<kTeams, false, true, true>); break;
-            case 7: go(k_encode<kTeams, true, true, true>); break;
-            case 8: go(k_encode<kTeams, false, false, false, true>); break;
-            case 9: go(k_encode<kTeams, true, false, false, true>); break;
-            case 10: go(k_encode<kTeams, false, true, false, true>); break;
-            case 11: go(k_encode<kTeams, true, true, false, true>); break;
-            case 12: go(k_encode<kTeams, false, false, true, true>); break;
-            case 13: go(k_encode<kTeams, true, false, true, true>); break;
-            case 14: go(k_encode<kTeams, false, true, true, true>); break;
-            default: go(k_encode<kTeams, true, true, true, true>); break;
+            case 0: go(k_encode<false, false, false>); break;
+            case 1: go(k_encode<true, false, false>); break;
+            case 2: go(k_encode<false, true, false>); break;
+            case 3: go(k_encode<true, true, false>); break;
+            case 4: go(k_encode<false, false, true>); break;
+            case 5: go(k_encode<true, false, true>); break;
+            case 6: go(k_encode<false, true, true>); break;
+            case 7: go(k_encode<true, true, true>); break;
+            case 8: go(k_encode<false, false, false, true>); break;
+            case 9: go(k_encode<true, false, false, true>); break;
+            case 10: go(k_encode<false, true, false, true>); break;
+            case 11: go(k_encode<true, true, false, true>); break;
+            case 12: go(k_encode<false, false, true, true>); break;
+            case 13: go(k_encode<true, false, true, true>); break;
+            case 14: go(k_encode<false, true, true, true>); break;
+            default: go(k_encode<true, true, true, true>); break;
         }
     }
     launch_after(k_encode_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, dirty, crc_inout, w, ws, ds->tables,

@@ -145,11 +145,6 @@ __device__ __forceinline__ bool x_wait(uint32_t bar, uint32_t parity, uint32_t b
     if (!ok) *fail = 1u;
     return ok;
 }
-__device__ __forceinline__ void x_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
 // One step of a chain: s' = rotl(s, 31) * P1 + x.  Written out in 32-bit halves: behind the rotation
 // (two funnel shifts) stand one wide product with x as its addend and, beside it, the two products
 // that only reach the high half; one add joins them.  23 cycles a step, where the plain formula
@@ -229,7 +224,7 @@ k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t
             for (uint32_t i = 0; i < kUnits; i++)
                 asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a + 256u * i), "l"(u[i] * kXP2), "l"(v[i] * kXP2) : "memory");
             __syncwarp();
-            if (lane == 0) x_arrive(full + 8u * (s % kXSlots));
+            if (lane == 0) mbar_arrive_at(full + 8u * (s % kXSlots));
         };
         uint32_t done = 0;
         for (uint32_t s = 0; s < n_seg; s++) {
@@ -307,7 +302,7 @@ k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t
         if (g != odd_seg) steps(x1);
         if ((stripes + kXSeg - 1u) / kXSeg == g + 1u) at_end = s;
         __syncwarp();
-        if (lane == 0) x_arrive(empty + 8u * slot);
+        if (lane == 0) mbar_arrive_at(empty + 8u * slot);
         slot = n_slot; parity = n_parity; a = n_a;
     }
     if (stripes) v = x_step(at_end, 0ull);

@@ -140,3 +140,22 @@ def test_sparse_and_degenerate_masks(chunk_tiles, options, kw):
                 assert np.array_equal(got[lo:hi], host.numpy()[lo:hi]), (name, c)
             else:
                 assert (got[lo:hi] == 0x3C).all(), (name, c)
+
+
+@pytest.mark.parametrize("tiles", [1, 2, 7, 8, 147, 148, 8 * 147, 8 * 147 + 1, 2 * 8 * 148, 2 * 8 * 148 + 1])
+@pytest.mark.parametrize("masked", [False, True])
+def test_encode_around_the_numbers_of_teams(tiles, masked):
+    """A block runs fewer of its eight teams when there are fewer tiles than teams; every team takes one tile first
+    up to two tiles per team, two from there on."""
+    n, chunk = tiles * 16384, 2 * 16384
+    g = torch.Generator("cuda").manual_seed(tiles)
+    cur = torch.randn(n // 2, generator=g, device="cuda").to(torch.bfloat16).view(torch.uint8)
+    nc = wm.num_chunks(n, chunk)
+    mask = np.array([c % 4 != 2 for c in range(nc)], np.uint8) if masked else None
+    want_wire, want_crc, want = oracle.encode(cur.cpu().numpy(), chunk, dirty=mask, crc_in=np.zeros(nc, np.uint32))
+    ws, res, crc = wm.new_workspace(n, chunk), wm.new_result(), torch.zeros(nc, dtype=torch.int32, device="cuda")
+    wire = torch.zeros(wm.wire_bound(n, chunk), dtype=torch.uint8, device="cuda")
+    wm.wm_encode(cur, chunk, None if mask is None else torch.from_numpy(mask).cuda(), crc, wire, ws, res)
+    r = wm.read_result(res)
+    assert r.ok and r.wire_len == want.wire_len and np.array_equal(wire[: r.wire_len].cpu().numpy(), want_wire)
+    assert np.array_equal(crc.cpu().numpy().view(np.uint32), want_crc)
