@@ -18,10 +18,10 @@
  *     small or not 16-byte aligned, wire_cap below the metadata size), WM_ERR_CUDA for
  *     a launch failure, else WM_OK.
  *   - Calls that share a workspace must be ordered on one stream (or by events).
- *   - A call enqueues a short chain of kernels; all but the first are launched with
- *     programmatic stream serialization (they may start while their predecessor drains and
- *     wait inside before touching its results).  Work enqueued by the caller before or after
- *     a call keeps ordinary stream order.
+ *   - A call enqueues a short chain of kernels, launched with programmatic stream
+ *     serialization (a kernel may start while its predecessor on the stream drains and
+ *     waits inside for its end before touching anything).  Work enqueued by the caller before
+ *     or after a call keeps ordinary stream order.
  *   - All integers in the wire image are little-endian.  Tile = 16384 bytes, group = 256
  *     bf16 elements; n_chunks = ceil(nbytes / chunk_bytes), n_tiles = ceil(nbytes / 16384).
  */

@@ -17,12 +17,13 @@ namespace wm {
 // The cleared control block: the error word in it is the call's outcome (wm_workspace_status).
 __global__ void k_checksum_init(Ctrl* ctrl)
 {
+    grid_dep_wait();
     grid_dep_launch();
     if (threadIdx.x < sizeof(Ctrl) / 4) reinterpret_cast<uint32_t*>(ctrl)[threadIdx.x] = 0u;
 }
 
 // Small caches.  A block takes one chunk of at most TEAMS tiles, a tile per team, straight into
-// registers (asked for before the tables are in place), and thread 0 folds the chunk.  Nothing in
+// registers, and thread 0 folds the chunk.  Nothing in
 // here waits for a copy, so there is no outcome to report but success.
 template <int TEAMS>
 __global__ void __launch_bounds__(TEAMS * 256, 1)
@@ -35,6 +36,13 @@ k_chunk_crcs(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables
     const uint32_t c = blockIdx.x, t0 = c * g.tiles_per_chunk, t = t0 + team;
     const uint32_t ntc = min(g.tiles_per_chunk, g.n_tiles - t0);
     const bool full = team < ntc && t < g.n_full_tiles;
+    const uint32_t ht = (&tab->HT[0][0])[threadIdx.x];
+    Smem S = setup_smem(smem, tab);
+    unsigned char* const slot = S.take(kTile);
+    uint32_t* const sHT = reinterpret_cast<uint32_t*>(S.take(4096));        // (complete behind the block's barrier)
+    sHT[threadIdx.x] = ht;
+    grid_dep_wait();
+    grid_dep_launch();
     if (c == 0 && threadIdx.x == 0) ws.ctrl->err = 0;
     uint32_t d[kWordsPerLane];
     if (full) {
@@ -42,11 +50,6 @@ k_chunk_crcs(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables
 #pragma unroll
         for (int i = 0; i < 16; i++) d[i] = __ldcs(p + 32 * i);
     }
-    const uint32_t ht = (&tab->HT[0][0])[threadIdx.x];
-    Smem S = setup_smem(smem, tab);
-    unsigned char* const slot = S.take(kTile);
-    uint32_t* const sHT = reinterpret_cast<uint32_t*>(S.take(4096));        // (complete behind the block's barrier)
-    sHT[threadIdx.x] = ht;
     if (full) {
         const uint32_t v = tile_digest_part(S, d, team == 0u, warp, lane);
         if (lane == 0) s_wdig[team][warp] = v;
@@ -198,6 +201,7 @@ k_checksum_finish(const unsigned char* __restrict__ cache, Geo g, Ws ws, const T
     __shared__ FinishStage stage;
     load_ht_t0(sHT, sT0, tab);
     grid_dep_wait();
+    grid_dep_launch();
     const uint32_t c0 = blockIdx.x * g.finish_cb;
     stage_chunk_digests(g, stage, ws.dig, c0);
     const uint32_t c = c0 + threadIdx.x;

@@ -9,6 +9,7 @@ namespace wm {
 
 __global__ void k_decode_init(Ws ws)
 {
+    grid_dep_wait();
     grid_dep_launch();
     if (blockIdx.x == 0 && threadIdx.x < sizeof(Ctrl) / 4) {
         uint32_t v = 0;
@@ -815,6 +816,7 @@ k_decode_finish(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g
     __shared__ int s_status;
     load_ht_t0(sHT, sT0, tab);
     grid_dep_wait();
+    grid_dep_launch();
     if (ld_volatile_u32(&ws.ctrl->gate)) return;
     const uint32_t c0 = blockIdx.x * g.finish_cb;
     stage_chunk_digests(g, stage, ws.dig, c0);

@@ -137,8 +137,9 @@ __device__ __forceinline__ void sts_now(uint32_t addr, uint32_t v)
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// Programmatic dependent launch.  Every call enqueues a short chain of kernels; each kernel but
-// the first is launched with permission to start before its predecessor has finished.  It then
+// Programmatic dependent launch.  Every call enqueues a short chain of kernels; each is launched with
+// permission to start before its predecessor on the stream has finished (the first one too: its
+// predecessor is the caller's or the previous call's last kernel).  It then
 // sets up what does not depend on the predecessor (tables into shared memory, allocations) and
 // waits here; the wait returns once the predecessor has completed and its writes are visible.
 // Every block of such a kernel must pass the wait before it exits or reads anything the chain

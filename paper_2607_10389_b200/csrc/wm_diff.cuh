@@ -8,6 +8,7 @@ namespace wm {
 
 __global__ void k_diff_init(Ws ws)
 {
+    grid_dep_wait();
     grid_dep_launch();
     if (threadIdx.x == 0 && blockIdx.x == 0) { ws.ctrl->ticket = 0; ws.ctrl->n_present = 0; ws.ctrl->err = 0; }
 }
@@ -81,6 +82,7 @@ k_diff_compact(Geo g, const uint8_t* __restrict__ dirty, uint32_t* __restrict__ 
 {
     __shared__ uint32_t s_part[33];
     grid_dep_wait();
+    grid_dep_launch();
     const uint32_t per = (g.n_chunks + 1023u) / 1024u;
     const uint32_t c0 = min(threadIdx.x * per, g.n_chunks), c1 = min(c0 + per, g.n_chunks);
     uint32_t mine = 0;

@@ -15,6 +15,7 @@ namespace wm {
 __global__ void __launch_bounds__(1024)
 k_encode_init(Geo g, Ws ws, unsigned char* wire, const uint8_t* __restrict__ dirty)
 {
+    grid_dep_wait();
     grid_dep_launch();
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;

@@ -213,19 +213,20 @@ static wm_status checksum_any(const unsigned char* c, const Geo& g, const Ws& ws
 {
     // A chunk per block and a tile per team, when they all fit at once: one launch instead of three.
     // Measured (us a call, this and the three): 2 MiB in 16 KiB chunks 5.2 and 8.0, 2 and 8 MiB in 64 KiB
-    // chunks 7.8 and 8.2, 8.3 and 8.8; with more chunks per block (16 MiB) 12.7 and 10.8.
+    // chunks 7.3 and 8.2, 7.7 and 8.8; with more chunks per block (16 MiB) 12.7 and 10.8.
     // (The test hook for waits that run out needs a kernel that waits.)
     if (g.n_chunks <= n_sm && g.tiles_per_chunk <= (uint32_t)kTeamsPlain && !g.inject) {
+        auto go = [&]() { launch_after(k_chunk_crcs<kTeamsPlain>, g.n_chunks, kTeamsPlain * 256, kDynSmem, s, c, g, ws, tab, crc_out); };
         if (timed) {
             MainKernelTimer timer(timed, 0, s);
-            k_chunk_crcs<kTeamsPlain><<<g.n_chunks, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, tab, crc_out);
+            go();
         } else {
-            k_chunk_crcs<kTeamsPlain><<<g.n_chunks, kTeamsPlain * 256, kDynSmem, s>>>(c, g, ws, tab, crc_out);
+            go();
         }
         g_launches = 1;
         return launch_status();
     }
-    k_checksum_init<<<1, 64, 0, s>>>(ws.ctrl);
+    launch_after(k_checksum_init, 1, 64, 0, s, ws.ctrl);
     auto digests = [&]() {
         // A warp per tile needs enough tiles for even shares.  Measured (us a call, a team and a warp per
         // tile): 77 MB 21 and 24, 155 MB 34 and 36, 310 MB 59 and 58, 620 MB 112 and 105, 1.67 GB 275 and 257.
@@ -387,7 +388,7 @@ wm_status wm_dirty_diff(const void* cache, const void* prev, uint64_t nbytes, ui
     if (!ds) return WM_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Ws ws = ws_carve(workspace, g);
-    k_diff_init<<<1, 32, 0, s>>>(ws);
+    launch_after(k_diff_init, 1, 32, 0, s, ws);
     const uint32_t want = (uint32_t)ds->sm_count * 4;
     const uint32_t grid = g.n_chunks < want ? g.n_chunks : want;
     {
@@ -427,7 +428,7 @@ static wm_status encode_any(const void* cache, const wm_leaf* leaves, uint32_t n
     const unsigned char* c = static_cast<const unsigned char*>(cache);
     unsigned char* w = static_cast<unsigned char*>(wire);
     const uint32_t init_blocks = (g.n_tiles + 1023) / 1024 < 1024 ? (g.n_tiles + 1023) / 1024 : 1024;
-    k_encode_init<<<init_blocks ? init_blocks : 1, 1024, 0, s>>>(g, ws, w, dirty);
+    launch_after(k_encode_init, init_blocks ? init_blocks : 1, 1024, 0, s, g, ws, w, dirty);
     if (leaves) {
         const uint32_t map_blocks = (g.n_tiles + 1023) / 1024 < 148 ? (g.n_tiles + 1023) / 1024 : 148;      // a tile per thread
         launch_after(k_leaf_map, map_blocks ? map_blocks : 1, 1024, 0, s, leaves, n_leaves, g, ws, result, 0);
@@ -508,7 +509,7 @@ static wm_status decode_any(const void* wire, uint64_t wire_len, void* dst, cons
     Ws ws = ws_carve(workspace, g);
     const unsigned char* w = static_cast<const unsigned char*>(wire);
     unsigned char* d = static_cast<unsigned char*>(dst);
-    k_decode_init<<<1, 64, 0, s>>>(ws);
+    launch_after(k_decode_init, 1, 64, 0, s, ws);
     if (leaves) {
         const uint32_t map_blocks = (g.n_tiles + 1023) / 1024 < 148 ? (g.n_tiles + 1023) / 1024 : 148;      // a tile per thread
         launch_after(k_leaf_map, map_blocks ? map_blocks : 1, 1024, 0, s, leaves, n_leaves, g, ws, result, 1);

@@ -79,6 +79,7 @@ k_meta_crc(unsigned char* wire, Geo g, Ws ws, const Tables* __restrict__ tab, wm
     s_wdig += 8 * team;
     sHT[threadIdx.x] = (&tab->HT[0][0])[threadIdx.x];
     grid_dep_wait();
+    grid_dep_launch();
     const uint64_t pad = (uint64_t)g.n_meta_slices * kTile - g.meta_end;    // multiple of 4
     const uint32_t s = blockIdx.x * 4 + team;
     if (s < g.n_meta_slices) {
