@@ -891,6 +891,58 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     if (threadIdx.x < 32) tmem_free_all(s_tmem);
 }
 
+// Chunk c's directory entry and CRC (the calling thread's chunk: c0 + i).  Returns its term of the
+// whole-cache CRC; `present` says whether the image carries it.
+__device__ __forceinline__ uint32_t close_chunk(const unsigned char* __restrict__ cache, const Geo& g, const uint8_t* __restrict__ dirty,
+                                                uint32_t* __restrict__ crc_inout, unsigned char* wire, const Ws& ws, const uint32_t* sHT,
+                                                const uint32_t* sT0, const FinishStage& stage, const ChunkPowers& cp, unsigned long long total,
+                                                uint32_t c, uint32_t i, uint32_t& present)
+{
+    unsigned char* dir = wire + 64;
+    present = (!dirty || dirty[c]) ? 1u : 0u;
+    // Where the chunk's payload starts: a present chunk's offset was written by the team that
+    // placed its first tile; an absent chunk (the main kernel never saw it) starts where the next
+    // present chunk does, or at the end of the payload.
+    const uint32_t n_list = dirty ? ld_volatile_u32(&ws.ctrl->n_list) : 0u;
+    auto starts_at = [&](uint32_t cc) -> unsigned long long {
+        if (cc >= g.n_chunks) return total;
+        if (!dirty || dirty[cc]) return *reinterpret_cast<const unsigned long long*>(dir + 16ull * cc);
+        uint32_t lo = 0, hi = n_list;              // the first listed chunk above cc
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) / 2;
+            if (ws.plist[mid] < cc) lo = mid + 1; else hi = mid;
+        }
+        return lo < n_list ? *reinterpret_cast<const unsigned long long*>(dir + 16ull * ws.plist[lo]) : total;
+    };
+    const unsigned long long po = starts_at(c), nx = starts_at(c + 1);
+    uint32_t crc;
+    if (present) {
+        crc = chunk_crc_staged(g, sHT, sT0, stage, ws.dig, chunk_first_byte(g, ws, cache, c), c, i);
+        crc_inout[c] = crc;
+    } else {
+        crc = crc_inout[c];
+        *reinterpret_cast<unsigned long long*>(dir + 16ull * c) = po;
+    }
+    *reinterpret_cast<uint32_t*>(dir + 16ull * c + 8) = (uint32_t)(nx - po);
+    *reinterpret_cast<uint32_t*>(dir + 16ull * c + 12) = crc;
+    return cache_crc_term(g, cp, crc, c);
+}
+
+// The header (one thread; meta_crc left zero).
+__device__ __forceinline__ void write_header(const Geo& g, unsigned char* wire, bool masked, uint32_t option_flags, uint32_t n_present,
+                                             unsigned long long total, uint32_t cache_crc)
+{
+    uint32_t* h = reinterpret_cast<uint32_t*>(wire);
+    h[0] = 0x31564D57u;                                  // "WMV1"
+    h[1] = 1u | ((masked ? 1u : 0u) << 16) | (option_flags << 16);      // version, flags (bit 1 zero tiles, bit 2 ENT tiles)
+    h[2] = (uint32_t)g.nbytes; h[3] = (uint32_t)(g.nbytes >> 32);
+    h[4] = g.chunk_bytes; h[5] = kTile; h[6] = g.n_chunks; h[7] = n_present;
+    h[8] = (uint32_t)total; h[9] = (uint32_t)(total >> 32);
+    const unsigned long long wl = g.meta_end + total;
+    h[10] = (uint32_t)wl; h[11] = (uint32_t)(wl >> 32);
+    h[12] = cache_crc; h[13] = 0u; h[14] = 0u; h[15] = 0u;
+}
+
 // Directory (enc_len, crc), chunk CRCs, present count; the last block to finish combines the
 // chunk CRCs into the cache CRC and writes the header (meta_crc left zero).
 __global__ void __launch_bounds__(1024)
@@ -908,42 +960,14 @@ k_encode_finish(const unsigned char* __restrict__ cache, Geo g, const uint8_t* _
     grid_dep_launch();
     const uint32_t c0 = blockIdx.x * g.finish_cb;
     stage_chunk_digests(g, stage, ws.dig, c0);
-    unsigned char* dir = wire + 64;
     const unsigned long long total = ws.ctrl->payload_total;
     // only finish_cb threads of a block fold chunks (the lookups of a full block would queue up
     // on one SM's shared memory)
     const uint32_t c = c0 + threadIdx.x;
     uint32_t present = 0, term = 0;
     const bool dead = (ld_volatile_u32(&ws.ctrl->err) & 8u) != 0;      // leaf mode: the table was rejected
-    if (!dead && threadIdx.x < g.finish_cb && c < g.n_chunks) {
-        present = (!dirty || dirty[c]) ? 1u : 0u;
-        uint32_t crc;
-        if (present) {
-            crc = chunk_crc_staged(g, sHT, sT0, stage, ws.dig, chunk_first_byte(g, ws, cache, c), c, threadIdx.x);
-            crc_inout[c] = crc;
-        } else {
-            crc = crc_inout[c];
-        }
-        // Where the chunk's payload starts: a present chunk's offset was written by the team that
-        // placed its first tile; an absent chunk (the main kernel never saw it) starts where the next
-        // present chunk does, or at the end of the payload.
-        const uint32_t n_list = dirty ? ld_volatile_u32(&ws.ctrl->n_list) : 0u;
-        auto starts_at = [&](uint32_t cc) -> unsigned long long {
-            if (cc >= g.n_chunks) return total;
-            if (!dirty || dirty[cc]) return *reinterpret_cast<const unsigned long long*>(dir + 16ull * cc);
-            uint32_t lo = 0, hi = n_list;              // the first listed chunk above cc
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) / 2;
-                if (ws.plist[mid] < cc) lo = mid + 1; else hi = mid;
-            }
-            return lo < n_list ? *reinterpret_cast<const unsigned long long*>(dir + 16ull * ws.plist[lo]) : total;
-        };
-        const unsigned long long po = starts_at(c), nx = starts_at(c + 1);
-        if (!present) *reinterpret_cast<unsigned long long*>(dir + 16ull * c) = po;
-        *reinterpret_cast<uint32_t*>(dir + 16ull * c + 8) = (uint32_t)(nx - po);
-        *reinterpret_cast<uint32_t*>(dir + 16ull * c + 12) = crc;
-        term = cache_crc_term(g, cp, crc, c);
-    }
+    if (!dead && threadIdx.x < g.finish_cb && c < g.n_chunks)
+        term = close_chunk(cache, g, dirty, crc_inout, wire, ws, sHT, sT0, stage, cp, total, c, threadIdx.x, present);
     accumulate_cache_crc(ws.ctrl, term, &s_acc);
     const uint32_t cnt = __syncthreads_count(present);
     if (threadIdx.x == 0) {
@@ -956,15 +980,7 @@ k_encode_finish(const unsigned char* __restrict__ cache, Geo g, const uint8_t* _
     __threadfence();
     const uint32_t cache_crc = ld_volatile_u32(&ws.ctrl->cache_acc);
     const uint32_t n_present = ld_volatile_u32(&ws.ctrl->n_present);
-    uint32_t* h = reinterpret_cast<uint32_t*>(wire);
-    h[0] = 0x31564D57u;                                  // "WMV1"
-    h[1] = 1u | ((dirty ? 1u : 0u) << 16) | (option_flags << 16);      // version, flags (bit 1 zero tiles, bit 2 ENT tiles)
-    h[2] = (uint32_t)g.nbytes; h[3] = (uint32_t)(g.nbytes >> 32);
-    h[4] = g.chunk_bytes; h[5] = kTile; h[6] = g.n_chunks; h[7] = n_present;
-    h[8] = (uint32_t)total; h[9] = (uint32_t)(total >> 32);
-    const unsigned long long wl = g.meta_end + total;
-    h[10] = (uint32_t)wl; h[11] = (uint32_t)(wl >> 32);
-    h[12] = cache_crc; h[13] = 0u; h[14] = 0u; h[15] = 0u;
+    write_header(g, wire, dirty != nullptr, option_flags, n_present, total, cache_crc);
     ws.ctrl->hdr_cache_crc = cache_crc;
     ws.ctrl->hdr_n_present = n_present;
     ws.ctrl->payload_total = total;

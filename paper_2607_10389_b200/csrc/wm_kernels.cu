@@ -113,7 +113,8 @@ static const DeviceState* device_state()
     }
     for (const void* f : {(const void*)k_tile_digests<kTeamsPlain>, (const void*)k_tile_digests_stream, (const void*)k_chunk_crcs<kTeamsPlain>})
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
-    if (cudaFuncSetAttribute(k_meta_crc, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
+    for (const void* f : {(const void*)k_meta_crc, (const void*)k_encode_close})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     if (cudaFuncSetAttribute(k_xxh64_paced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXSmem) != cudaSuccess) return nullptr;
     for (int k = 0; k < 4; k++)
         for (int j = 0; j < 2; j++)
@@ -464,10 +465,16 @@ static wm_status encode_any(const void* cache, const wm_leaf* leaves, uint32_t n
             default: go(k_encode<true, true, true, true>); break;
         }
     }
-    launch_after(k_encode_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, dirty, crc_inout, w, ws, ds->tables,
-                 chunk_powers(g), (opt_ent ? 4u : 0u) | (opt_zero ? 2u : 0u));
-    launch_after(k_meta_crc, (g.n_meta_slices + 3) / 4, 1024, kDynSmem, s, w, g, ws, ds->tables, result);
-    g_launches = leaves ? 6 : 4;
+    const uint32_t flags = (opt_ent ? 4u : 0u) | (opt_zero ? 2u : 0u);
+    const bool close = g.n_chunks <= g.finish_cb && g.n_meta_slices <= 4u;       // one block can do both
+    if (close) {
+        launch_after(k_encode_close, 1, 1024, kDynSmem, s, c, g, dirty, crc_inout, w, ws, ds->tables, chunk_powers(g), flags, result);
+    } else {
+        launch_after(k_encode_finish, (g.n_chunks + g.finish_cb - 1) / g.finish_cb, 1024, 0, s, c, g, dirty, crc_inout, w, ws, ds->tables,
+                     chunk_powers(g), flags);
+        launch_after(k_meta_crc, (g.n_meta_slices + 3) / 4, 1024, kDynSmem, s, w, g, ws, ds->tables, result);
+    }
+    g_launches = (leaves ? 6 : 4) - (close ? 1 : 0);
     return launch_status();
 }
 
