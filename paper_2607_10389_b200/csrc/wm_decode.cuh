@@ -7,11 +7,10 @@ namespace wm {
 
 // ------------------------------------------------------------------ wm_decode_verify
 
-__global__ void k_decode_init(Ws ws)
+// The control block's words at the start of a decode call.
+__device__ __forceinline__ void decode_init_ctrl(const Ws& ws)
 {
-    grid_dep_wait();
-    grid_dep_launch();
-    if (blockIdx.x == 0 && threadIdx.x < sizeof(Ctrl) / 4) {
+    if (threadIdx.x < sizeof(Ctrl) / 4) {
         uint32_t v = 0;
         const uint32_t i = threadIdx.x;
         if (i == offsetof(Ctrl, bad3_first) / 4 || i == offsetof(Ctrl, bad4_first) / 4 ||
@@ -20,6 +19,12 @@ __global__ void k_decode_init(Ws ws)
             v = 0xFFFFFFFFu;
         reinterpret_cast<uint32_t*>(ws.ctrl)[i] = v;
     }
+}
+__global__ void k_decode_init(Ws ws)
+{
+    grid_dep_wait();
+    grid_dep_launch();
+    decode_init_ctrl(ws);
 }
 
 __device__ __forceinline__ void fill_result(wm_result* result, const Ctrl* ctrl, uint64_t wire_len, int status,
@@ -55,6 +60,10 @@ __host__ __device__ __forceinline__ uint32_t check_chunks_per_warp(uint32_t tile
     return tiles_per_chunk <= 16u ? 32u / tiles_per_chunk : 1u;
 }
 
+// SINGLE: the call's metadata is so little that the warps of one block are enough for both parts (the
+// first eight per slice digest, the others check chunks); that block then also does what k_decode_init
+// does for the other calls, and a small cache's chain has one kernel less.
+template <bool SINGLE>
 __global__ void __launch_bounds__(1024)
 k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g, Ws ws,
                const Tables* __restrict__ tab, wm_result* result, uint32_t meta_blocks, uint32_t expect_ent)
@@ -70,8 +79,12 @@ k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g,
     const uint32_t lane = threadIdx.x % 32, wblk = threadIdx.x / 32;
     if (blockIdx.x < meta_blocks) load_small_chain_tables(sG, tab);       // (the structure blocks need no tables)
     grid_dep_wait();
+    if (SINGLE) {
+        decode_init_ctrl(ws);
+        __syncthreads();
+    }
     grid_dep_launch();
-    if (ld_volatile_u32(&ws.ctrl->gate)) return;        // leaf mode: the destination table was rejected
+    if (!SINGLE && ld_volatile_u32(&ws.ctrl->gate)) return;        // leaf mode: the destination table was rejected
     if (threadIdx.x == 0) s_format_bad = header_matches(wire, wire_len, g, expect_ent) ? 0 : 1;
     __syncthreads();
     if (s_format_bad) {
@@ -86,12 +99,15 @@ k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g,
     }
     const unsigned char* dir = wire + 64;
     const bool zero_ok = ((reinterpret_cast<const uint32_t*>(wire)[1] >> 17) & 1u) != 0u;   // the image declares the option
-    if (blockIdx.x < meta_blocks) {
-        const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
+    const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
+    const uint32_t meta_warps = SINGLE ? 8u * g.n_meta_slices : 0u;
+    if (SINGLE ? wblk < meta_warps : blockIdx.x < meta_blocks) {
         const uint32_t s = blockIdx.x * 4 + team;
         if (s < g.n_meta_slices) meta_slice_parts(wire, g, s, sG, tab, s_wdig[team], tt / 32, lane);
-        __syncthreads();
-        if (tt == 0 && s < g.n_meta_slices) ws.mdig[s] = xor8(s_wdig[team]);
+        if (!SINGLE) {
+            __syncthreads();
+            if (tt == 0 && s < g.n_meta_slices) ws.mdig[s] = xor8(s_wdig[team]);
+        }
     } else {
         const uint16_t* tab16 = reinterpret_cast<const uint16_t*>(wire + 64 + 16ull * g.n_chunks);
         // one tile entry: its payload length and what it says about its chunk
@@ -119,7 +135,7 @@ k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g,
             return po == (pr.x | ((unsigned long long)pr.y << 32)) + pr.z;
         };
         const uint32_t tpc = g.tiles_per_chunk, cpw = check_chunks_per_warp(tpc);
-        const uint32_t cw = ((blockIdx.x - meta_blocks) * 32u + wblk) * cpw;        // the warp's first chunk
+        const uint32_t cw = (SINGLE ? wblk - meta_warps : (blockIdx.x - meta_blocks) * 32u + wblk) * cpw;        // the warp's first chunk
         bool present = false, bad = false;            // the verdict on chunk c, held by the lane that reports it
         uint32_t c = cw;
         if (cpw == 1u) {
@@ -196,20 +212,33 @@ k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g,
         if (present) ws.plist[slot0 + __popc(pres & ((1u << lane) - 1u))] = c;
         if (bad) { atomicMin(&ws.ctrl->bad3_first, c); atomicAdd(&ws.ctrl->bad3_count, 1u); }
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        s_first = 0xFFFFFFFFu; s_count = 0;
+    uint32_t crc = 0;
+    if (SINGLE) {
+        sHT[threadIdx.x] = (&tab->HT[0][0])[threadIdx.x];
+        if (threadIdx.x == 0) { s_first = 0xFFFFFFFFu; s_count = 0; }
         __threadfence();
-        s_last = atomicAdd(&ws.ctrl->done_b, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t st = 0;
+            for (uint32_t i = 0; i < g.n_meta_slices; i++) st = advance_tile(sHT, st) ^ xor8(s_wdig[i]);
+            crc = ~st;
+        }
+    } else {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_first = 0xFFFFFFFFu; s_count = 0;
+            __threadfence();
+            s_last = atomicAdd(&ws.ctrl->done_b, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        sHT[threadIdx.x] = (&tab->HT[0][0])[threadIdx.x];
+        crc = fold_meta_digests(g, ws, sHT, s_dig);
     }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
 
     // ---- the last block: metadata CRC first
-    sHT[threadIdx.x] = (&tab->HT[0][0])[threadIdx.x];
-    const uint32_t crc = fold_meta_digests(g, ws, sHT, s_dig);
     if (threadIdx.x == 0) {
         const uint32_t* h = reinterpret_cast<const uint32_t*>(wire);
         ws.ctrl->hdr_n_present = h[7];
@@ -458,12 +487,16 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     // at once.
     const bool masked = ((reinterpret_cast<const uint32_t*>(wire)[1] >> 16) & 1u) != 0u;
     const uint32_t n_tickets = masked ? ld_volatile_u32(&ws.ctrl->n_present) * g.tiles_per_chunk : 0u;
+    auto tile_of = [&](uint32_t k) -> uint32_t {
+        if (!masked) return k;
+        const uint32_t j = chunk_of(g, k);
+        return ws.plist[j] * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
+    };
     auto claim = [&]() -> uint32_t {
         uint32_t k = atomicAdd(&ws.ctrl->ticket, 1u);
         if (!masked) return k;
         while (k < n_tickets) {
-            const uint32_t j = chunk_of(g, k);
-            const uint32_t t = ws.plist[j] * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
+            const uint32_t t = tile_of(k);
             if (t < g.n_full_tiles) return t;
             k = atomicAdd(&ws.ctrl->ticket, 1u);
         }
@@ -472,16 +505,16 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage);
     const uint32_t sm_s = stage_s + 64u + 1024u * warp + 8u * lane;     // this lane's sign-mantissa bytes, group 4 warp
 
-    // a tile's entry word and payload offset (blocking: prologue only)
-    auto lookup = [&](uint32_t t, DecSlot* sl) {
-        if (LEAVES && t < g.n_full_tiles) tc->dstp[sl - tc->slot] = ws.tptr[t];
-        sl->t = t;
-        sl->entry = 0; sl->src = 0;
-        if (t < g.n_full_tiles) {
-            const uint32_t e = tab16_of()[t];
-            sl->entry = e | (first_in_chunk(g, t) ? 0x10000u : 0u);
-            if (e) sl->src = *reinterpret_cast<const unsigned long long*>(dir_of() + 16ull * chunk_of(g, t)) + ws.rel[t];
-        }
+    // two tiles' entry words and payload offsets (blocking: prologue only; all loads under way together)
+    auto lookup2 = [&](uint32_t ta, uint32_t tb) {
+        const bool a = ta < g.n_full_tiles, b = tb < g.n_full_tiles;
+        const uint32_t ea = a ? tab16_of()[ta] : 0u, eb = b ? tab16_of()[tb] : 0u;
+        const unsigned long long pa = a ? *reinterpret_cast<const unsigned long long*>(dir_of() + 16ull * chunk_of(g, ta)) + ws.rel[ta] : 0ull;
+        const unsigned long long pb = b ? *reinterpret_cast<const unsigned long long*>(dir_of() + 16ull * chunk_of(g, tb)) + ws.rel[tb] : 0ull;
+        const unsigned long long da = LEAVES && a ? ws.tptr[ta] : 0ull, db = LEAVES && b ? ws.tptr[tb] : 0ull;
+        if (LEAVES) { tc->dstp[0] = da; tc->dstp[1] = db; }
+        tc->slot[0] = {ta, a ? ea | (first_in_chunk(g, ta) ? 0x10000u : 0u) : 0u, ea ? pa : 0ull};
+        tc->slot[1] = {tb, b ? eb | (first_in_chunk(g, tb) ? 0x10000u : 0u) : 0u, eb ? pb : 0ull};
     };
     // staged tiles: full RAW and PACK tiles (everything except absent tiles and zero / constant ones)
     // (images with the entropy option hold ENT tiles too: entry 0x8000 | length / 32)
@@ -508,9 +541,22 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     }
     if (leader) {
         mbar_init(&tc->mbar, 1);
-        lookup(claim(), &tc->slot[0]);
-        lookup(claim(), &tc->slot[1]);
-        tc->slot[2].t = claim();      // its look-ups happen in the first step
+        uint32_t ta, tb, tn;               // the tiles of the first three steps
+        const uint32_t n_claim = masked ? n_tickets : g.n_full_tiles, teams = gridDim.x * TEAMS;
+        if (n_claim <= teams) {
+            // a tile per team at most: dealt out evenly over the blocks, nobody draws a second one
+            const uint32_t k = blockIdx.x + gridDim.x * team;
+            ta = k < n_claim ? tile_of(k) : kNone;
+            tb = tn = kNone;
+        } else if (!masked) {
+            ta = atomicAdd(&ws.ctrl->ticket, 3u);
+            tb = ta + 1u;
+            tn = ta + 2u;
+        } else {
+            ta = claim(); tb = claim(); tn = claim();
+        }
+        lookup2(ta, tb);
+        tc->slot[2].t = tn;                // its look-ups happen in the first step
         start_copy(tc->slot[0]);
     }
     team_bar(team);

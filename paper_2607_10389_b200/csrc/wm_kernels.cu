@@ -516,17 +516,22 @@ static wm_status decode_any(const void* wire, uint64_t wire_len, void* dst, cons
     Ws ws = ws_carve(workspace, g);
     const unsigned char* w = static_cast<const unsigned char*>(wire);
     unsigned char* d = static_cast<unsigned char*>(dst);
-    launch_after(k_decode_init, 1, 64, 0, s, ws);
+    const uint32_t per_warp = check_chunks_per_warp(g.tiles_per_chunk);
+    const uint32_t meta_blocks = (g.n_meta_slices + 3) / 4;
+    const bool ent = (options & WM_OPT_ENTROPY) != 0;      // the option says which kind of image the call expects
+    const bool single = !leaves && 8ull * g.n_meta_slices + (g.n_chunks + per_warp - 1u) / per_warp <= 32u;      // one block checks, and clears
+    if (!single) launch_after(k_decode_init, 1, 64, 0, s, ws);
     if (leaves) {
         const uint32_t map_blocks = (g.n_tiles + 1023) / 1024 < 148 ? (g.n_tiles + 1023) / 1024 : 148;      // a tile per thread
         launch_after(k_leaf_map, map_blocks ? map_blocks : 1, 1024, 0, s, leaves, n_leaves, g, ws, result, 1);
     }
     // a wire shorter than the metadata is rejected by the header check before anything else is read
-    const uint32_t meta_blocks = (g.n_meta_slices + 3) / 4;
-    const uint32_t chunks_per_block = 32u * check_chunks_per_warp(g.tiles_per_chunk);
-    const bool ent = (options & WM_OPT_ENTROPY) != 0;      // the option says which kind of image the call expects
-    launch_after(k_decode_check, meta_blocks + (g.n_chunks + chunks_per_block - 1) / chunks_per_block, 1024, 0, s, w, wire_len, g, ws, ds->tables, result, meta_blocks,
-                 ent ? 1u : 0u);
+    const uint32_t chunks_per_block = 32u * per_warp;
+    if (single)
+        launch_after(k_decode_check<true>, 1, 1024, 0, s, w, wire_len, g, ws, ds->tables, result, 1u, ent ? 1u : 0u);
+    else
+        launch_after(k_decode_check<false>, meta_blocks + (g.n_chunks + chunks_per_block - 1) / chunks_per_block, 1024, 0, s, w, wire_len, g, ws,
+                     ds->tables, result, meta_blocks, ent ? 1u : 0u);
     const uint32_t need = (g.n_tiles + kTeamsPlain - 1) / kTeamsPlain;
     uint32_t grid = need < (uint32_t)ds->sm_count ? need : (uint32_t)ds->sm_count;
     if (block_cap && grid > block_cap) grid = block_cap;
@@ -554,7 +559,7 @@ static wm_status decode_any(const void* wire, uint64_t wire_len, void* dst, cons
         else pass(k_decode<kTeamsPlain, false, 2>, k_decode<kTeamsPlain, true, 2>);
         if (leaves) launch_after(k_leaf_scatter, 1024, 256, 0, s, leaves, n_leaves, g, ws);
     }
-    g_launches = (leaves ? 6 : 4) + (strict ? 1 : 0) + (ent ? (strict ? 2 : 1) : 0);
+    g_launches = (leaves ? 6 : single ? 3 : 4) + (strict ? 1 : 0) + (ent ? (strict ? 2 : 1) : 0);
     return launch_status();
 }
 

@@ -122,3 +122,41 @@ def test_many_small_chunks_round_trip_and_mask(tpc, nc):
     rd = wm.read_result(res)
     assert rd.ok and rd.n_present == int(mask.sum())
     assert torch.equal(old, cur) and np.array_equal(dcrc.cpu().numpy().view(np.uint32), want_crc)
+
+
+@pytest.mark.parametrize("tiles,chunk_tiles", [(128, 1), (129, 1), (4 * 192, 4), (4 * 193, 4), (24 * 40, 40), (25 * 40, 40), (591, 4), (592, 4), (593, 4)])
+@pytest.mark.parametrize("masked", [False, True])
+def test_calls_around_the_one_block_kernels(tiles, chunk_tiles, masked):
+    """One block closes an encode (up to 128 chunks) and checks a decode (as long as its 32 warps are enough); up to
+    a tile per team the decode kernel deals tiles out without tickets.  Damaged metadata gets the oracle's verdict."""
+    import torch
+    from paper_2607_10389_b200 import binding as wm
+    n, chunk = tiles * 16384 - 777, chunk_tiles * 16384
+    g = torch.Generator("cuda").manual_seed(tiles)
+    cur = torch.randn((n + 1) // 2, generator=g, device="cuda").to(torch.bfloat16).view(torch.uint8)[:n].contiguous()
+    nc = wm.num_chunks(n, chunk)
+    mask = np.array([c % 3 != 1 for c in range(nc)], np.uint8) if masked else None
+    old = oracle.checksum(cur.cpu().numpy(), chunk)
+    want_wire, want_crc, want = oracle.encode(cur.cpu().numpy(), chunk, dirty=mask, crc_in=old)
+    ws, res = wm.new_workspace(n, chunk), wm.new_result()
+    crc = torch.from_numpy(old.view(np.int32).copy()).cuda()
+    wire = torch.zeros(wm.wire_bound(n, chunk), dtype=torch.uint8, device="cuda")
+    wm.wm_encode(cur, chunk, None if mask is None else torch.from_numpy(mask).cuda(), crc, wire, ws, res)
+    r = wm.read_result(res)
+    assert r.ok and (r.wire_len, r.cache_crc, r.n_present) == (want.wire_len, want.cache_crc, want.n_present)
+    assert np.array_equal(wire[: r.wire_len].cpu().numpy(), want_wire) and np.array_equal(crc.cpu().numpy().view(np.uint32), want_crc)
+    dst = cur.clone()
+    for c in range(nc):
+        if mask is None or mask[c]:
+            dst[c * chunk: min((c + 1) * chunk, n)] = 0x11
+    dst0 = dst.clone()
+    wm.wm_decode_verify(wire, r.wire_len, dst, chunk, crc, ws, res)
+    assert wm.read_result(res).ok and torch.equal(dst, cur)
+    meta = wm.meta_bytes(n, chunk)
+    for at, bit in ((20, 1), (60, 0), (64 + 8, 2), (64 + 16 * (nc - 1) + 3, 5), (64 + 16 * nc + 2 * (tiles // 2), 3), (meta - 40, 1)):
+        bad = wire.clone()
+        bad[at] ^= 1 << bit
+        wm.wm_decode_verify(bad, r.wire_len, dst0.clone(), chunk, crc, ws, res)
+        got = wm.read_result(res)
+        _, _, o = oracle.decode_verify(bad[: r.wire_len].cpu().numpy(), n, chunk, dst=dst0.cpu().numpy(), dst_crc=crc.cpu().numpy().view(np.uint32))
+        assert (got.status, got.first_bad_chunk, got.n_bad_chunks) == (o.status, o.first_bad_chunk, o.n_bad_chunks), (at, bit)
