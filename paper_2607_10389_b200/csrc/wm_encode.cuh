@@ -650,11 +650,11 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                     const uint32_t lb = lenE_s - anchor, cb = cwE_s - 2u * anchor;
 #pragma unroll
                     for (int i = 0; i < 16; i++) {
-                        const uint32_t E0 = __byte_perm(d[i], 0u, 0x4441), E1 = d[i] >> 24;
-                        const uint32_t len0 = lds_tab_u8(lb + E0), len1 = lds_tab_u8(lb + E1);
-                        // (the table's escape entry is 0xFFFF: the AND lets the exponent through there only)
-                        const uint32_t c0 = lds_tab_u16(cb + 2u * E0) & __byte_perm(E0, 0xFFu, 0x4404);
-                        const uint32_t c1 = lds_tab_u16(cb + 2u * E1) & __byte_perm(E1, 0xFFu, 0x4404);
+                        const uint32_t len0 = lds_tab_u8(__dp4a(d[i], 0x00000100u, lb)), len1 = lds_tab_u8(__dp4a(d[i], 0x01000000u, lb));
+                        // (the table's escape entry is 0xFFFF: the AND lets the exponent, which is in the
+                        // second byte of the word or of its high half, through there only)
+                        const uint32_t c0 = lds_tab_u16(__dp4a(d[i], 0x00000200u, cb)) & (d[i] | 0xFFFF00FFu);
+                        const uint32_t c1 = lds_tab_u16(__dp4a(d[i], 0x02000000u, cb)) & ((d[i] >> 16) | 0xFFFF00FFu);
                         const uint32_t pair = c1 * (1u << len0) + c0;
                         asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(pair), "r"(1u << n));
                         n += len0 + len1;
@@ -777,11 +777,13 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
 #pragma unroll
                     for (int i = 0; i < 16; i++) acc = __dp4a(d[i], 0x01000100u, acc);       // bytes 1 and 3
                     const uint32_t anchor = (__reduce_add_sync(0xFFFFFFFFu, acc) + 512u) >> 10;
+                    // (the exponents are bytes 1 and 3 of a rotated word: the dot product that picks one
+                    // and adds the table's address is the look-up's whole address arithmetic)
                     uint32_t bits = 0;
                     const uint32_t lb = lenE_s - anchor;
 #pragma unroll
                     for (int i = 0; i < 16; i++)
-                        bits += lds_tab_u8(lb + __byte_perm(d[i], 0u, 0x4441)) + lds_tab_u8(lb + (d[i] >> 24));
+                        bits += lds_tab_u8(__dp4a(d[i], 0x00000100u, lb)) + lds_tab_u8(__dp4a(d[i], 0x01000000u, lb));
                     // (a strand the length byte cannot hold, above 319 bits, keeps the tile out of the form:
                     // the count is then so large that the form is never the shortest)
                     const uint32_t share_bits = __reduce_add_sync(0xFFFFFFFFu, bits);
