@@ -58,7 +58,7 @@ constexpr uint32_t kUnit = 32;              // placement words count in units of
 //
 // lbk[t] starts at 0.  The team that encodes tile t publishes kFlagA | len(t)/32 as soon as the
 // length is known.  One scanner warp (alone in the block that wins a lock at kernel start, so
-// that it has an SM's issue slots to itself) walks the array in order, 512 entries per poll,
+// that it has an SM's issue slots to itself) walks the array in order, 256 entries per poll,
 // turns every leading run of published lengths into kFlagP | (exclusive prefix)/32, and moves
 // on.  The owner of tile t then reads its offset back from lbk[t].  Every encoded length that
 // another tile has to add is a multiple of 32 (only the cache's last tile can be ragged, and
@@ -101,72 +101,86 @@ __device__ __forceinline__ unsigned long long wait_prefix(const uint32_t* lbk, u
     return 0;
 }
 
-// Scanner side (one full warp).  A poll copies 512 consecutive entries into shared memory with
-// coalesced asynchronous 16-byte copies (one round trip to L2, no registers held meanwhile);
-// lane l then owns entries 16 l .. 16 l + 15 of the window.
-constexpr int kScanPerLane = 16;
-__device__ void scan_tile_lengths(uint32_t* lbk, uint32_t n_tiles, uint32_t lane, Ctrl* ctrl, uint32_t* win,
-                                  uint32_t budget_ns)
+// Scanner side (one full warp).  A poll fetches 256 consecutive entries, lane l four of either half in
+// one 16-byte load (one round trip to L2), and turns the leading run of published ones into offsets.
+// The time of a poll is what every owner's offset waits for, so nothing in it is spread out: a half's
+// entries lie across the lanes as they lie in memory, both ways one coalesced access, and the two
+// halves' prefix sums run side by side.  (512 entries through shared memory, sixteen consecutive ones
+// per lane with a store each, took 1.5 us a poll, this takes 1.0.)
+__device__ __forceinline__ uint4 ld_now_v4(const uint32_t* p)
 {
-    uint64_t f = 0;                 // first unresolved entry
-    uint64_t base = 0;              // units before f
+    uint4 v;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ void scan_tile_lengths(uint32_t* lbk, uint32_t n_tiles, uint32_t lane, Ctrl* ctrl, uint32_t budget_ns)
+{
+    uint32_t f = 0;                 // first unresolved entry
+    uint32_t base = 0;              // units before f
     uint32_t spins = 0;             // polls in a row that resolved nothing
     uint32_t t0 = 0;                // the clock when that run of empty polls began
     while (f < n_tiles) {
-        const uint64_t w0 = f & ~3ull;                    // 16-byte aligned window start
-        const uint32_t skip = (uint32_t)(f - w0);         // entries before f (already resolved)
+        const uint32_t w0 = f & ~3u;                      // 16-byte aligned window start
+        uint32_t v[2][4], cnt[2], sum[2], incl[2], lead[2];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const uint32_t slot = 4u * (lane + 32u * q);
-            if (w0 + slot < n_tiles) {                    // n_tiles entries are padded to a multiple of 4
-                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(win + slot);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(lbk + w0 + slot) : "memory");
-            } else {
-                *reinterpret_cast<uint4*>(win + slot) = make_uint4(0, 0, 0, 0);
+        for (int h = 0; h < 2; h++) {
+            const uint32_t at = w0 + 128u * h + 4u * lane;                   // (the entries are padded to a multiple of 4)
+            const uint4 x = at < n_tiles ? ld_now_v4(lbk + at) : make_uint4(0u, 0u, 0u, 0u);
+            v[h][0] = x.x; v[h][1] = x.y; v[h][2] = x.z; v[h][3] = x.w;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            // the lane's leading published entries (those before f are done: they count, with value 0)
+            const uint32_t at = w0 + 128u * h + 4u * lane;
+            cnt[h] = 0; sum[h] = 0;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const bool done = at + j < f;
+                if (cnt[h] == (uint32_t)j && at + j < n_tiles && (done || (v[h][j] >> 30) == 1u)) {
+                    cnt[h]++;
+                    sum[h] += done ? 0u : v[h][j] & kValMask;
+                }
             }
+            const uint32_t fm = __ballot_sync(0xFFFFFFFFu, cnt[h] == 4u);
+            lead[h] = fm == 0xFFFFFFFFu ? 32u : (uint32_t)(__ffs(~fm) - 1);      // leading full lanes
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncwarp();
-        uint32_t v[kScanPerLane];
+        if (lead[0] < 32u) lead[1] = 0xFFFFFFFFu;          // the run ends in the first half: nothing of the second counts
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const uint4 x = *reinterpret_cast<const uint4*>(win + kScanPerLane * lane + 4 * q);
-            v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+        for (int h = 0; h < 2; h++) {
+            if (lead[h] == 0xFFFFFFFFu || lane > lead[h]) { cnt[h] = 0; sum[h] = 0; }
+            incl[h] = sum[h];
         }
-        __syncwarp();
-        // leading published entries of this lane (entries before f count as published, value 0)
-        uint32_t r = 0, sum = 0;
-#pragma unroll
-        for (int j = 0; j < kScanPerLane; j++) {
-            const uint32_t rel = kScanPerLane * lane + j;
-            const bool old = rel < skip;
-            const bool in = w0 + rel < n_tiles;
-            if (r == (uint32_t)j && in && (old || (v[j] >> 30) == 1u)) { r++; if (!old) sum += v[j] & kValMask; }
-        }
-        const uint32_t fm = __ballot_sync(0xFFFFFFFFu, r == (uint32_t)kScanPerLane);
-        const uint32_t lead = (fm == 0xFFFFFFFFu) ? 32u : (uint32_t)(__ffs(~fm) - 1);   // leading full lanes
-        const uint32_t contrib = lane <= lead ? sum : 0u;
-        uint32_t incl = contrib;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-            if (lane >= (uint32_t)d) incl += o;
-        }
-        const uint32_t cnt = lane < lead ? (uint32_t)kScanPerLane : (lane == lead ? r : 0u);
-        uint64_t run = base + (incl - contrib);
 #pragma unroll
-        for (int j = 0; j < kScanPerLane; j++) {
-            const uint32_t rel = kScanPerLane * lane + j;
-            if ((uint32_t)j < cnt && rel >= skip) {
-                st_relaxed_u32(lbk + w0 + rel, kFlagP | (uint32_t)run);
-                run += v[j] & kValMask;
+            for (int h = 0; h < 2; h++) {
+                const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl[h], d);
+                if (lane >= (uint32_t)d) incl[h] += o;
             }
         }
-        const uint32_t r_lead = __shfl_sync(0xFFFFFFFFu, r, lead & 31u);
-        const uint32_t k_all = (uint32_t)kScanPerLane * lead + (lead < 32u ? r_lead : 0u);   // includes `skip`
-        const uint32_t k = k_all > skip ? k_all - skip : 0u;
-        base += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        const uint32_t all0 = __shfl_sync(0xFFFFFFFFu, incl[0], 31), all1 = __shfl_sync(0xFFFFFFFFu, incl[1], 31);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const uint32_t at = w0 + 128u * h + 4u * lane;
+            const uint32_t r0 = base + (h ? all0 : 0u) + incl[h] - sum[h];       // units before the lane's first new entry
+            if (cnt[h] == 4u && at >= f) {
+                const uint32_t r1 = r0 + (v[h][0] & kValMask), r2 = r1 + (v[h][1] & kValMask), r3 = r2 + (v[h][2] & kValMask);
+                asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(lbk + at), "r"(kFlagP | r0), "r"(kFlagP | r1), "r"(kFlagP | r2),
+                             "r"(kFlagP | r3) : "memory");
+            } else {
+                uint32_t run = r0;
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    if ((uint32_t)j < cnt[h] && at + j >= f) {
+                        st_relaxed_u32(lbk + at + j, kFlagP | run);
+                        run += v[h][j] & kValMask;
+                    }
+                }
+            }
+        }
+        const uint32_t k_all = __reduce_add_sync(0xFFFFFFFFu, cnt[0] + cnt[1]);  // entries from w0 on that are resolved now
+        const uint32_t k = w0 + k_all - f;
+        base += all0 + all1;
         f += k;
         if (k == 0) {
             // nothing new: the owners are behind.  Every 64 such polls in a row the scanner looks at the
@@ -440,12 +454,11 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     const bool ragged = g.tail_len != 0u && (!MASKED || dirty[g.n_chunks - 1u] != 0);
     const uint32_t n_hot = ragged ? n_tickets - 1u : n_tickets;
     if (s_scanner) {
-        uint32_t* win = reinterpret_cast<uint32_t*>(S.take(2048));      // 512 entries
         unsigned char* slot = S.take(kTile);
         uint32_t* wdig = reinterpret_cast<uint32_t*>(S.take(32));
         if (!S.ok) { if (threadIdx.x == 0) atomicOr(&ws.ctrl->err, 4u); return; }
         // (test hook: with the scanner left out no offset is ever handed out, and the owners' waits run out)
-        if (threadIdx.x < 32 && !(g.inject & kInjectNoScanner)) scan_tile_lengths(ws.lbk, n_tickets, threadIdx.x, ws.ctrl, win, g.wait_ns);
+        if (threadIdx.x < 32 && !(g.inject & kInjectNoScanner)) scan_tile_lengths(ws.lbk, n_tickets, threadIdx.x, ws.ctrl, g.wait_ns);
         if (ragged && threadIdx.x / kTeamThreads == 1u)
             encode_ragged_tile(S, g, LEAVES ? reinterpret_cast<const unsigned char*>(ws.tptr[g.n_full_tiles]) : cache + (uint64_t)g.n_full_tiles * kTile,
                                wire, wire_cap, ws, n_tickets - 1u, slot, wdig);
