@@ -407,6 +407,14 @@ __device__ __forceinline__ void unpack_group(const PlaneWords& pw, uint32_t base
     }
 }
 
+// A share whose four groups have width 4 and bases that no delta carries past 255.
+__device__ __forceinline__ bool all_of_width_4(uint2 dd)
+{
+    const uint32_t w = ((dd.x ^ 0x04000400u) | (dd.y ^ 0x04000400u)) & 0x0F000F00u;
+    const uint32_t over = (((dd.x & 0x00FF00FFu) + 0x000F000Fu) | ((dd.y & 0x00FF00FFu) + 0x000F000Fu)) & 0x01000100u;
+    return (w | over) == 0u;
+}
+
 // Unpack + checksum of the decoded bytes.  Tiles are claimed by ticket.  The team owns one
 // 16 KiB stage in shared memory; the encoded tile arrives there by one bulk copy (TMA) that is
 // started a tile ahead, each lane takes what it needs (descriptors, its 8 sign-mantissa bytes
@@ -447,7 +455,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     if (ld_volatile_u32(&ws.ctrl->gate)) return;
     if (ENT != 0 && (ENT == 1) == (ld_volatile_u32(&ws.ctrl->has_pack) != 0u)) return;      // the other kernel's image
     const uint32_t team = threadIdx.x / kTeamThreads, tt = threadIdx.x % kTeamThreads;
-    const uint32_t warp = tt / 32, lane = tt % 32;
+    const uint32_t warp = warp_uniform(tt / 32), lane = tt % 32;
     unsigned char* stage = nullptr;
     for (int i = 0; i < TEAMS; i++) {          // every thread carves the same blocks in the same order
         unsigned char* p = S.take(kTile);
@@ -704,6 +712,11 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                 const uint32_t w01 = min_u16x2((dd.x >> 8) & 0x000F000Fu, 0x00080008u), w23 = min_u16x2((dd.y >> 8) & 0x000F000Fu, 0x00080008u);
                 dd.x = (dd.x & 0x00FF00FFu) | (w01 << 8);
                 dd.y = (dd.y & 0x00FF00FFu) | (w23 << 8);
+                if (all_of_width_4(dd)) {            // (what most shares are: the planes' places are fixed)
+                    const uint32_t rec = stage_s + 8256u + 32u * min(off, 237u) + 4u * lane;
+                    sm[0] = lds_now_v2<0>(sm_s); sm[1] = lds_now_v2<256>(sm_s); sm[2] = lds_now_v2<512>(sm_s); sm[3] = lds_now_v2<768>(sm_s);
+                    pw[0].a = lds_now<0>(rec); pw[1].a = lds_now<128>(rec); pw[2].a = lds_now<256>(rec); pw[3].a = lds_now<384>(rec);
+                } else
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     const uint32_t wg = j == 0 ? w01 & 15u : j == 1 ? w01 >> 16 : j == 2 ? w23 & 15u : w23 >> 16;
@@ -786,13 +799,17 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                 // table look-ups overlap the next group's arithmetic.
                 const uint32_t fold_mask = (fold && warp == 0u && lane == 0u) ? 0xFFFFFFFFu : 0u;
                 uint32_t st = 0, last = 0;
+                auto groups = [&](auto all4) {
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     const uint32_t dw = j < 2 ? dd.x : dd.y;
                     const uint32_t base = (j & 1) ? (dw >> 16) & 0xFFu : dw & 0xFFu, wd = (j & 1) ? dw >> 24 : (dw >> 8) & 15u;
                     uint32_t ea, eb;
                     if (ENT == 1 || (ENT == 2 && is_ent)) { ea = pw[j].a; eb = pw[j].b; }     // the exponent bytes are already there
-                    else unpack_group(pw[j], base, wd, ea, eb);
+                    else if (decltype(all4)::value) {
+                        unpack_nibbles(pw[j].a, ea, eb);
+                        ea += base * 0x01010101u; eb += base * 0x01010101u;
+                    } else unpack_group(pw[j], base, wd, ea, eb);
                     // A word rotated left by one bit reads [E | m << 1 | sign of the other half] in
                     // each half: swap bit 0 inside the byte pairs of the sign-mantissa words, put
                     // the exponent bytes beside them, rotate back.
@@ -810,6 +827,9 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                         if (j < 3) st = chain_step(S, st ^ w3); else last = st ^ w3;
                     }
                 }
+                };
+                if (ENT != 1 && HOW != 2u && all_of_width_4(dd)) groups(std::true_type());      // (byte stores: rare)
+                else groups(std::false_type());
                 if (MODE != 2) {
                     const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, last));
                     if (lane == 0) sts_now(tc_s + (uint32_t)offsetof(DecTeamCtl, wdig) + 32u * p + 4u * warp, v);

@@ -81,6 +81,11 @@ __device__ __forceinline__ Smem setup_smem(unsigned char* smem, const Tables* __
     return s;
 }
 
+// A value that is the same in every lane, told to the compiler: a warp reduction's result lives in a
+// uniform register, arithmetic on it leaves the lanes' pipe alone and branches on it need no
+// reconvergence bookkeeping.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __reduce_min_sync(0xFFFFFFFFu, v); }
+
 template <int OFF>
 __device__ __forceinline__ uint32_t lds_off(uint32_t addr)
 {

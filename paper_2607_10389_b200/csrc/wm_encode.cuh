@@ -700,6 +700,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                     tmem_load16(tmem_warp + 32u * par + 16u * part, d);
                     const uint4 g4 = *reinterpret_cast<const uint4*>(&tc->wtab[slX][8u * warp + 4u * part]);
                     const uint32_t gq[4] = {g4.x, g4.y, g4.z, g4.w};
+                    auto groups = [&](auto all4) {
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
                         const uint32_t wtg = gq[j];
@@ -710,8 +711,21 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                         const uint32_t ya = __byte_perm(sa, sa, 0x2301), yb = __byte_perm(sb, sb, 0x2301);
                         stg_v2(sm_dst + 256 * j, (sa & 0xFEFEFEFEu) | (ya & 0x01010101u), (sb & 0xFEFEFEFEu) | (yb & 0x01010101u));
                         const uint32_t e4a = __byte_perm(d[4 * j], d[4 * j + 1], 0x7531), e4b = __byte_perm(d[4 * j + 2], d[4 * j + 3], 0x7531);
-                        pack_group(wd, e4a, e4b, base, rec, lane);
-                        rec += 32u * wd;
+                        if (decltype(all4)::value) {
+                            const uint32_t b4 = base * 0x01010101u;
+                            pack_nibbles(e4a - b4, e4b - b4, rec + 128 * j, lane);
+                        } else {
+                            pack_group(wd, e4a, e4b, base, rec, lane);
+                            rec += 32u * wd;
+                        }
+                    }
+                    };
+                    // (four groups of width 4, what most shares are: the planes' places are fixed)
+                    if ((((g4.x ^ 0x400u) | (g4.y ^ 0x400u) | (g4.z ^ 0x400u) | (g4.w ^ 0x400u)) & 0xF00u) == 0u) {
+                        groups(std::true_type());
+                        rec += 512;
+                    } else {
+                        groups(std::false_type());
                     }
                     sm_dst += 1024;
                 }

@@ -480,3 +480,34 @@ def test_checksum_around_the_warp_per_tile_kernel(G, tiles, tail):
     assert res.status == 0 and np.array_equal(got, crc)
     for lo, hi in ((0, 3), (g.nc // 2, g.nc // 2 + 2), (g.nc - 3, g.nc)):
         assert np.array_equal(got[lo:hi], oracle.checksum(src[lo * chunk: min(hi * chunk, n)].cpu().numpy(), chunk))
+
+
+@pytest.mark.parametrize("bases", [(100, 100, 100, 100), (240, 0, 239, 240), (241, 7, 7, 7), (7, 7, 7, 247)])
+@pytest.mark.parametrize("widths", [(4, 4, 4, 4), (4, 4, 4, 3), (5, 4, 4, 4), (4, 0, 4, 4)])
+def test_shares_of_four_groups_of_width_four(G, bases, widths):
+    """The straight path for a share whose four groups have width 4, next to shares that just miss it; then
+    every plane nibble all ones, so that a delta carries a base above 240 past 255."""
+    from gpu_util import same_result, to_dev
+    rng = np.random.default_rng(sum(bases) + 7 * sum(widths))
+    E = np.zeros(3 * 8192, dtype=np.uint32)
+    for g in range(E.size // 256):
+        b, w = bases[g % 4], widths[(g // 4 + g) % 4] if (g // 4) % 3 == 2 else 4      # two shares of three are all fours
+        hi = min(1 << w, 256 - b)
+        d = rng.integers(0, hi, 256)
+        d[0], d[1] = 0, hi - 1
+        E[g * 256:(g + 1) * 256] = b + d
+    SM = rng.integers(0, 256, E.size).astype(np.uint32)
+    a = (((SM & 1) << 15) | (E << 7) | (SM >> 1)).astype("<u2").view(np.uint8)
+    n, chunk = a.size, 2 * TILE
+    g = G(n, chunk)
+    want_wire, want_crc, want = oracle.encode(a, chunk)
+    wire, crc, res, wire_dev = g.encode(to_dev(a))
+    assert same_result(res, want) and np.array_equal(wire[: res.wire_len], want_wire)
+    out, _, r = g.decode(wire_dev, res.wire_len)
+    assert r.status == 0 and np.array_equal(out, a)
+    meta = wire.size - n                                   # (wire_bound is the metadata and n)
+    bad = want_wire.copy()
+    bad[meta + 64 + 8192: meta + 64 + 8192 + 2048] = 0xFF  # the first tile's planes
+    out, _, r = g.decode(to_dev(bad), bad.size)
+    want_out, _, want_r = oracle.decode_verify(bad, n, chunk)
+    assert same_result(r, want_r) and r.status_name == "ERR_CHUNK_CRC"
