@@ -760,11 +760,41 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         }
         // ---- Y: digest, exponent ranges, words parked, a share at a time
         if (is_tile(qY)) {
+            // Warp 3 adds up the 32 widths and publishes the tile's length: in the middle of its second share's
+            // digest when the other warps' widths are there by then, else at the end of its own measuring,
+            // not behind the next team barrier: that one waits for W's offset, and an offset that comes late
+            // must not hold back a length that other teams' offsets are waiting for.
+            bool published = false;
+            auto publish = [&]() {
+                measured_phase ^= 1u;
+                published = true;
+                const uint32_t wt = tc->wtab[slY][lane];
+                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u);
+                // entropy option: the ENT form is taken when it is shorter than the planes and than raw
+                uint32_t ent_words = 0;
+                if (ENT) ent_words = __reduce_add_sync(0xFFFFFFFFu, lane < 8u ? tc->etab[slY][lane] >> 8 : 0u);
+                const uint32_t plane_len = total <= 253u ? 8256u + 32u * total : kTile;
+                const bool ent_tile = ENT && ent_tile_bytes(ent_words) < plane_len;
+                // unused memory (every share's first entry carries the mark): no payload
+                // (one value throughout: every share's first entry carries the mark and they are all alike;
+                // a tile of zeros has no payload, any other value 32 bytes)
+                const uint32_t wt0 = __shfl_sync(0xFFFFFFFFu, wt, 0);
+                const bool const_tile = ZEROS && __all_sync(0xFFFFFFFFu, (lane & 3u) != 0u || ((wt & kWarpConst) != 0u && wt == wt0));
+                const bool zero_tile = const_tile && (wt0 & kWarpAllZero) != 0u;
+                if (lane == 0) {
+                    tc->ssum[slY] = zero_tile ? kSumZeroTile : const_tile ? kSumConstTile : ent_tile ? kSumEnt | ent_words : total;
+                    const uint32_t len = zero_tile ? 0u : const_tile ? 32u : ent_tile ? ent_tile_bytes(ent_words) : plane_len;
+                    st_relaxed_u32(ws.lbk + place_of(step, qY), kFlagA | (len / kUnit));
+                }
+            };
             uint32_t st = ((qY & kQFirst) && tt == 0u) ? 0xFFFFFFFFu : 0u;      // (the all-ones start value complements the chunk's first word)
-#pragma unroll 1
+            // (both shares written out: the second one's wait, loads and first look-ups come up beside the first
+            // one's measuring; 518 -> 510 us, masked 399 -> 394, leaf mode 549 -> 541.  The packing loop above is
+            // better left a loop: 513 when it is unrolled too.)
+#pragma unroll
             for (uint32_t part = 0; part < 2u; part++) {
                 const uint32_t share = 2u * warp + part;
-                wait_for_copy_at<!ENT>(bar_s, phase, g.wait_ns, ws.ctrl);
+                wait_for_copy_at<ENT>(bar_s, phase, g.wait_ns, ws.ctrl);
                 phase ^= 1u;
                 // leaf mode: a tile that was copied from the 16-byte boundary below it starts that many
                 // bytes into the stage: whole words from a quarter of that on, each put together from two
@@ -783,18 +813,36 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                     if (part == 0u) start_copy(qY, LEAVES ? srcY : tile_src(qY & kQTile), 1u);
                     else start_copy(qN, LEAVES ? srcN : tile_src(qN & kQTile), 0u);
                 }
+                auto chain = [&](int from, int to) {
+#pragma unroll
+                    for (int i = from; i < to; i++) st = i < 15 ? chain_step(S, st ^ d[i]) : st ^ d[i];
+                };
+                // The words are kept rotated left by one bit: each half then reads [E | mantissa | a sign bit],
+                // E in its high byte (the two sign bits of a word land in each other's half; the packing
+                // step puts them right).
+                auto rotate = [&]() {
+#pragma unroll
+                    for (int i = 0; i < 16; i++) d[i] = __funnelshift_l(d[i], d[i], 1);
+                };
+                // The second share's widths come before its digest, off the words with their signs cleared
+                // (one instruction a word more): the sooner a length is out, the less an offset is waited
+                // for.  With incompressible data, where a step is short, that wait was 30 % of a step and
+                // the engine cache's size took 640 us; now 533 to 547.  An 8 MB cache's call: 20.5 -> 17.4 us.
+                // (The last of the four warps publishing at once, found by a counter: 538 us, but 520 instead
+                // of 508 on the engine cache, as the slowest warp then has the most to do; the first share's
+                // widths moved forward as well: 528.  With the entropy option the measuring needs the
+                // rotated words all the same and a step is long: digest first.)
+                const bool early = !ENT && part != 0u;
                 if (part) {
-                    ask();
+                    if (ENT) ask();
                     st = chain_step(S, st);
                 }
-#pragma unroll
-                for (int i = 0; i < 15; i++) st = chain_step(S, st ^ d[i]);
-                st ^= d[15];
-                // From here on the words are kept rotated left by one bit: each half then reads
-                // [E | mantissa | a sign bit], E in its high byte (the two sign bits of a word
-                // land in each other's half; the packing step puts them right).
-#pragma unroll
-                for (int i = 0; i < 16; i++) d[i] = __funnelshift_l(d[i], d[i], 1);
+                if (!early) {
+                    chain(0, 16);
+                    rotate();
+                }
+                auto word = [&](int i) { return early ? d[i] & 0x7FFF7FFFu : d[i]; };
+                const uint32_t exp_shift = early ? 23u : 24u;
                 uint32_t gw[4];               // per group: base | width << 8
                 uint32_t ent_w = 0;           // entropy option: anchor | words << 8 of this share
                 if (ENT) {
@@ -820,15 +868,15 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 }
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    const uint32_t a0 = d[4 * j], a1 = d[4 * j + 1], a2 = d[4 * j + 2], a3 = d[4 * j + 3];
+                    const uint32_t a0 = word(4 * j), a1 = word(4 * j + 1), a2 = word(4 * j + 2), a3 = word(4 * j + 3);
                     uint32_t mn = min_u16x2(min_u16x2(a0, a1), min_u16x2(a2, a3));
                     uint32_t mx = max_u16x2(max_u16x2(a0, a1), max_u16x2(a2, a3));
                     // both halves get the smaller (larger) of the two, so that the word as a whole
                     // orders like its halves and one warp reduction per bound does
                     mn = min_u16x2(mn, __byte_perm(mn, mn, 0x1032));
                     mx = max_u16x2(mx, __byte_perm(mx, mx, 0x1032));
-                    const uint32_t emin = __reduce_min_sync(0xFFFFFFFFu, mn) >> 24;
-                    const uint32_t emax = __reduce_max_sync(0xFFFFFFFFu, mx) >> 24;
+                    const uint32_t emin = __reduce_min_sync(0xFFFFFFFFu, mn) >> exp_shift;
+                    const uint32_t emax = __reduce_max_sync(0xFFFFFFFFu, mx) >> exp_shift;
                     gw[j] = emin | ((32u - __clz(emax - emin)) << 8);
                 }
                 // Option ZEROS.  Unused memory: when all four groups have exponent 0 throughout (rare in live data)
@@ -841,43 +889,27 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
 #pragma unroll
                     for (int i = 0; i < 16; i++) diff |= d[i] ^ first;
                     if (!__any_sync(0xFFFFFFFFu, diff != 0u))
-                        gw[0] |= kWarpConst | ((first & 0xFFu) << 16) | (first == 0u ? kWarpAllZero : 0u);
+                        gw[0] |= kWarpConst | (((early ? first << 1 | first >> 31 : first) & 0xFFu) << 16) | (first == 0u ? kWarpAllZero : 0u);
                 }
                 if (lane == 0) {
                     *reinterpret_cast<uint4*>(&tc->wtab[slY][4u * share]) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
                     if (ENT) tc->etab[slY][share] = ent_w;
                 }
+                if (part && lane == 0) mbar_arrive_at(tc_s + (uint32_t)offsetof(EncTeamCtl, measured));
+                if (early) {
+                    ask();                       // (here, not in front of the widths: 586 -> 550 us with incompressible data)
+                    chain(0, 8);
+                    if (warp == 3u && __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase))) publish();
+                    chain(8, 16);
+                    rotate();
+                }
                 tmem_store16(tmem_warp + 32u * par + 16u * part, d);
             }
             const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, st));
-            if (lane == 0) {
-                tc->wdig[slY][warp] = v;
-                mbar_arrive_at(tc_s + (uint32_t)offsetof(EncTeamCtl, measured));
-            }
-            // Warp 3 adds up the 32 widths and publishes the tile's length as soon as all four warps have
-            // measured, not behind the next team barrier: that one waits for W's offset, and an offset that
-            // comes late must not hold back a length that other teams' offsets are waiting for.
-            if (warp == 3u) {
+            if (lane == 0) tc->wdig[slY][warp] = v;
+            if (warp == 3u && !published) {
                 wait_for_copy_at<true>(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase, g.wait_ns, ws.ctrl);
-                measured_phase ^= 1u;
-                const uint32_t wt = tc->wtab[slY][lane];
-                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u);
-                // entropy option: the ENT form is taken when it is shorter than the planes and than raw
-                uint32_t ent_words = 0;
-                if (ENT) ent_words = __reduce_add_sync(0xFFFFFFFFu, lane < 8u ? tc->etab[slY][lane] >> 8 : 0u);
-                const uint32_t plane_len = total <= 253u ? 8256u + 32u * total : kTile;
-                const bool ent_tile = ENT && ent_tile_bytes(ent_words) < plane_len;
-                // unused memory (every share's first entry carries the mark): no payload
-                // (one value throughout: every share's first entry carries the mark and they are all alike;
-                // a tile of zeros has no payload, any other value 32 bytes)
-                const uint32_t wt0 = __shfl_sync(0xFFFFFFFFu, wt, 0);
-                const bool const_tile = ZEROS && __all_sync(0xFFFFFFFFu, (lane & 3u) != 0u || ((wt & kWarpConst) != 0u && wt == wt0));
-                const bool zero_tile = const_tile && (wt0 & kWarpAllZero) != 0u;
-                if (lane == 0) {
-                    tc->ssum[slY] = zero_tile ? kSumZeroTile : const_tile ? kSumConstTile : ent_tile ? kSumEnt | ent_words : total;
-                    const uint32_t len = zero_tile ? 0u : const_tile ? 32u : ent_tile ? ent_tile_bytes(ent_words) : plane_len;
-                    st_relaxed_u32(ws.lbk + place_of(step, qY), kFlagA | (len / kUnit));
-                }
+                publish();
             }
         } else {
             if (lane == 0) start_copy(qN, LEAVES ? srcN : tile_src(qN & kQTile), 0u);
