@@ -511,3 +511,23 @@ def test_shares_of_four_groups_of_width_four(G, bases, widths):
     out, _, r = g.decode(to_dev(bad), bad.size)
     want_out, _, want_r = oracle.decode_verify(bad, n, chunk)
     assert same_result(r, want_r) and r.status_name == "ERR_CHUNK_CRC"
+
+
+@pytest.mark.parametrize("share", [0, 1, 6, 7])
+@pytest.mark.parametrize("outlier", [0x0000, 0x8000, 0x007F, 0x7F80, 0xFFFF])
+def test_exponent_range_of_a_share_with_either_sign(G, share, outlier):
+    """One element of the smallest or largest exponent, with either sign, in a share of either parity (the
+    first and the second share of a warp are measured differently): the widths take no sign for exponent."""
+    from gpu_util import same_result, to_dev
+    rng = np.random.default_rng(share + outlier)
+    h = rng.integers(0x3F00, 0x4080, 4 * 8192).astype(np.uint32) | (rng.integers(0, 2, 4 * 8192).astype(np.uint32) << 15)
+    for t in range(4):
+        h[t * 8192 + share * 1024 + 250 * t + 17] = outlier
+    h[3 * 8192: 4 * 8192] = rng.integers(0, 65536, 8192)             # a tile that is stored raw
+    a = h.astype("<u2").view(np.uint8)
+    g = G(a.size, 2 * TILE)
+    want_wire, want_crc, want = oracle.encode(a, 2 * TILE)
+    wire, crc, res, wire_dev = g.encode(to_dev(a))
+    assert same_result(res, want) and np.array_equal(wire[: res.wire_len], want_wire)
+    out, _, r = g.decode(wire_dev, res.wire_len)
+    assert r.status == 0 and np.array_equal(out, a)
