@@ -123,11 +123,11 @@ k_tile_digests(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tabl
     for (; t < g.n_full_tiles; t += stride) {
         const bool first = first_in_chunk(g, (uint32_t)t);
         uint32_t d[kWordsPerLane];
-        wait_for_copy<false>(&tc->mbar, phase, g.wait_ns, ws.ctrl, (g.inject & kInjectNoCopy) != 0u);
+        wait_for_copy_at<false>((uint32_t)__cvta_generic_to_shared(&tc->mbar), phase, g.wait_ns, ws.ctrl, (g.inject & kInjectNoCopy) != 0u);
         phase ^= 1u;
         read_staged_words(stage, warp, lane, d);
         team_bar(team);                          // stage free; the previous tile's digest parts complete
-        if (tt == 64u) start_copy(t + stride);
+        if (tt == 64u && phase < kStuck) start_copy(t + stride);
         if (tt == 32u && t_done != ~0ull) ws.dig[t_done] = xor8(tc->wdig[par ^ 1u]);
         const uint32_t v = tile_digest_part(S, d, first, warp, lane);
         if (lane == 0) tc->wdig[par][warp] = v;
@@ -181,7 +181,7 @@ k_tile_digests_stream(const unsigned char* __restrict__ cache, Geo g, Ws ws, con
             uint32_t w[kWordsPerLane];
             read_staged_words_at(stage_s, 0u, lane, w);
             __syncwarp();
-            if (lane == 0) start_copy(part < 7u ? t : t + stride, (part + 1u) & 7u);
+            if (lane == 0 && phase < kStuck) start_copy(part < 7u ? t : t + stride, (part + 1u) & 7u);
             if (part) s = chain_step(S, s);
 #pragma unroll
             for (int i = 0; i < 15; i++) s = chain_step(S, s ^ w[i]);

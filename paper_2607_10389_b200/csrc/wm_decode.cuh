@@ -752,7 +752,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         // ahead and the ticket of the tile three ahead (answers taken at the end of the step).
         uint32_t l_tk = kNone;
         // (spread over three warps: the team waits for whichever warp has the most to do)
-        if (tt == 64u) start_copy(TC()->slot[(it + 1u) & 3u]);
+        if (tt == 64u && phase < kStuck) start_copy(TC()->slot[(it + 1u) & 3u]);
         store_digest(t_done, p ^ 1u);
         uint32_t t_look = kNone;           // warps 0 and 3: the tile claimed a step ago (two tiles ahead)
         if (leader) {                      // its table entry and offsets

@@ -368,7 +368,7 @@ __device__ __forceinline__ uint32_t now_ns()
 // Wait for the phase with the given parity to complete, for at most `budget_ns`.  Returns false
 // when the time ran out.  try_wait suspends the thread in hardware until the phase completes or
 // the time hint runs out, so a waiting warp does not burn issue slots that the other teams on
-// the SM need.  (The waiting loop itself, wait_for_copy, follows the control block's definition.)
+// the SM need.  (The waiting loop itself, wait_for_copy_at, follows the control block's definition.)
 __device__ __forceinline__ uint32_t mbar_try(uint32_t bar_s, uint32_t parity)
 {
     uint32_t done;

@@ -503,7 +503,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     const uint32_t tc_s = (uint32_t)__cvta_generic_to_shared(tc);
     const uint32_t bar_s = tc_s + (uint32_t)offsetof(EncTeamCtl, mbar) + 8u * warp;
     const bool leader = (tt == 0);
-    uint32_t phase = 0;                // parity of the stage's next completion
+    uint32_t stuck = 0;                // kStuck when a copy into the stage has not come
     uint32_t measured_phase = 0;       // warp 3: of the measures'
 
     auto is_tile = [](uint32_t q) { return (int32_t)q >= 0; };
@@ -513,11 +513,11 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     auto tile_src = [&](uint32_t t) -> unsigned long long {
         return LEAVES ? ws.tptr[t] : reinterpret_cast<unsigned long long>(cache + (uint64_t)t * kTile);
     };
-    // Lane 0 of a warp, when the warp's stage is free: the copy of one of its two shares.  Leaf mode: a
+    // Lane 0 of a warp, when the warp's stage is free (never again once it is stuck): the copy of one of its two shares.  Leaf mode: a
     // tile may start off a 16-byte boundary; the copy then starts at the boundary below and takes 16
     // bytes more (k_leaf_map saw to it that they belong to the leaf); the readers shift by the remainder.
     auto start_copy = [&](uint32_t q, unsigned long long src, uint32_t part) {
-        if (!is_tile(q)) return;
+        if (!is_tile(q | stuck)) return;
         const unsigned long long a = (LEAVES ? src & ~15ull : src) + kShare * (2u * warp + part);
         bulk_load_at(stage_s, reinterpret_cast<const void*>(a), (LEAVES && (src & 15ull)) ? kShare + 16u : kShare, bar_s, pol_once);
     };
@@ -794,8 +794,9 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
 #pragma unroll
             for (uint32_t part = 0; part < 2u; part++) {
                 const uint32_t share = 2u * warp + part;
-                wait_for_copy_at<ENT>(bar_s, phase, g.wait_ns, ws.ctrl);
-                phase ^= 1u;
+                uint32_t phase = part | stuck;        // (two copies a tile: the first one's phase is even)
+                wait_for_copy_at<true>(bar_s, phase, g.wait_ns, ws.ctrl);
+                stuck = phase & kStuck;
                 // leaf mode: a tile that was copied from the 16-byte boundary below it starts that many
                 // bytes into the stage: whole words from a quarter of that on, each put together from two
                 // neighbours when the remainder is no multiple of four
@@ -899,7 +900,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 if (early) {
                     ask();                       // (here, not in front of the widths: 586 -> 550 us with incompressible data)
                     chain(0, 8);
-                    if (warp == 3u && __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase))) publish();
+                    if (warp == 3u && __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase & 1u))) publish();
                     chain(8, 16);
                     rotate();
                 }

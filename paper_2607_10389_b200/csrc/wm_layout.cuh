@@ -78,48 +78,49 @@ __device__ __forceinline__ void give_up(Ctrl* ctrl)
     atomicMax(&ctrl->ticket, 0x7FFF0000u);
 }
 
-// Wait for a bulk copy into a stage: the phase of `bar` with the given parity, for at most
-// `budget_ns`.  A copy is started a whole step before it is needed, so the first try nearly
-// always succeeds, and everything else happens only after a try has come back empty: the clock is
-// read, and when the budget has passed the thread gives up for the whole call, then gives the
-// copy one more budget to land (so that the block, and with it the stage, does not go away under
-// a copy still in flight) and returns false.  A thread that comes here after the call has been
-// given up makes its one try and no more.  `no_second`: test hook, no copy is in flight.
-// What follows a first try that came back empty.
-__device__ __forceinline__ bool wait_for_copy_rest(uint32_t b, uint32_t parity, uint32_t budget_ns, Ctrl* ctrl, bool no_second)
+// Wait for a bulk copy into a stage: the phase of barrier `b` (its shared-window address) with the
+// parity in `phase`'s low bit, for at most `budget_ns`.  A copy is started a whole step before it is
+// needed, so the first try nearly always succeeds, and everything else happens only after a try has
+// come back empty: the clock is read, and when the budget has passed the thread gives up for the
+// whole call, then gives the copy one more budget to land (so that the block, and with it the stage,
+// does not go away under a copy still in flight).  A thread that comes here after another has given
+// up the call still waits for its own copy, which as a rule is on its way, for one budget.
+// When the copy has not come, `phase` gets kStuck, for good: the barrier may be in the midst of a
+// phase, so NO further copy is started on it (a second arrival in one phase is an error that ends
+// the context), and later waits do not wait.  `no_second`: no copy is in flight (the test hook, or
+// a barrier that other warps arrive on).
+constexpr uint32_t kStuck = 1u << 31;
+// What follows a first try that came back empty: the new phase word.
+__device__ __forceinline__ uint32_t wait_for_copy_rest(uint32_t b, uint32_t phase, uint32_t budget_ns, Ctrl* ctrl, bool no_second)
 {
-    if (*reinterpret_cast<volatile uint32_t*>(&ctrl->err) & 2u) return false;
+    if (phase & kStuck) return phase;
+    const bool given_up = (*reinterpret_cast<volatile uint32_t*>(&ctrl->err) & 2u) != 0u;
+    if (given_up && no_second) return phase | kStuck;
     uint32_t t0 = now_ns();
     do {
-        if (mbar_try(b, parity)) return true;
+        if (mbar_try(b, phase)) return phase;
     } while (now_ns() - t0 <= budget_ns);
+    if (given_up) return phase | kStuck;
     give_up(ctrl);
-    if (no_second) return false;
+    if (no_second) return phase | kStuck;
     t0 = now_ns();
     do {
-        if (mbar_try(b, parity)) break;
+        if (mbar_try(b, phase)) break;
     } while (now_ns() - t0 <= budget_ns);
-    return false;
+    return phase | kStuck;
 }
-__device__ __noinline__ bool wait_for_copy_rest_call(uint32_t b, uint32_t parity, uint32_t budget_ns, Ctrl* ctrl, bool no_second)
+__device__ __noinline__ uint32_t wait_for_copy_rest_call(uint32_t b, uint32_t phase, uint32_t budget_ns, Ctrl* ctrl, bool no_second)
 {
-    return wait_for_copy_rest(b, parity, budget_ns, ctrl, no_second);
+    return wait_for_copy_rest(b, phase, budget_ns, ctrl, no_second);
 }
 // OUT_OF_LINE: the rest is a call.  Which form is faster differs from kernel to kernel (it decides
 // how the compiler lays out the hot loop around it); each kernel takes the one measured better.
 template <bool OUT_OF_LINE>
-__device__ __forceinline__ bool wait_for_copy_at(uint32_t b, uint32_t parity, uint32_t budget_ns, Ctrl* ctrl,
-                                                 bool no_second = false)        // b: the barrier's shared-window address
+__device__ __forceinline__ void wait_for_copy_at(uint32_t b, uint32_t& phase, uint32_t budget_ns, Ctrl* ctrl, bool no_second = false)
 {
-    if (mbar_try(b, parity)) return true;
-    return OUT_OF_LINE ? wait_for_copy_rest_call(b, parity, budget_ns, ctrl, no_second)
-                       : wait_for_copy_rest(b, parity, budget_ns, ctrl, no_second);
-}
-template <bool OUT_OF_LINE>
-__device__ __forceinline__ bool wait_for_copy(unsigned long long* bar, uint32_t parity, uint32_t budget_ns, Ctrl* ctrl,
-                                              bool no_second = false)
-{
-    return wait_for_copy_at<OUT_OF_LINE>((uint32_t)__cvta_generic_to_shared(bar), parity, budget_ns, ctrl, no_second);
+    if (mbar_try(b, phase & 1u)) return;
+    phase = OUT_OF_LINE ? wait_for_copy_rest_call(b, phase, budget_ns, ctrl, no_second)
+                        : wait_for_copy_rest(b, phase, budget_ns, ctrl, no_second);
 }
 
 struct Ws {

@@ -69,6 +69,36 @@ def test_encode_gives_up_when_no_offset_ever_comes(stalled):
     assert np.array_equal(crc.cpu().numpy().view(np.uint32), want_crc)
 
 
+@pytest.mark.parametrize("options", [0, wm.OPT_ENTROPY])
+@pytest.mark.parametrize("masked", [False, True])
+def test_encode_gives_up_with_several_tiles_per_team(stalled, options, masked):
+    """When one team gives up for the call, the others have copies on their way into their stages: a team has to wait
+    for its own before it starts another on the same barrier, and before its block ends."""
+    n, chunk = 4000 * 16384 + 7777, 8 * 16384
+    cur = torch.randn((n + 1) // 2, generator=torch.Generator("cuda").manual_seed(3), device="cuda").to(torch.bfloat16).view(torch.uint8)[:n].contiguous()
+    nc, cap = wm.num_chunks(n, chunk), wm.wire_bound(n, chunk)
+    mask = (torch.arange(nc, device="cuda") % 8 != 3).to(torch.uint8) if masked else None
+    ws, res = wm.new_workspace(n, chunk), wm.new_result()
+    wire = torch.full((cap + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    crc = torch.zeros(nc, dtype=torch.int32, device="cuda")
+
+    def encode():
+        wm.wm_encode_opt(cur, chunk, mask, crc, wire[:cap], ws, res, options)
+        return wm.read_result(res)
+    r = encode()
+    want, want_crc = wire[: r.wire_len].clone(), crc.clone()
+    assert r.ok
+    for _ in range(3):
+        t0 = time.time()
+        with stalled():
+            bad = encode()
+        assert bad.status_name == "ERR_TIMEOUT" and time.time() - t0 < 20
+        assert bool((wire[cap:] == 0xA5).all()), "wrote past wire_cap"
+        crc.zero_()
+        r = encode()
+        assert r.ok and torch.equal(wire[: r.wire_len], want) and torch.equal(crc, want_crc)
+
+
 @pytest.mark.parametrize("options", [0, wm.OPT_ENTROPY, wm.OPT_STRICT])
 def test_decode_gives_up_when_the_copies_never_arrive(stalled, options):
     host, cur, chunk = _cache()
