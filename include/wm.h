@@ -106,10 +106,12 @@ wm_status wm_workspace_status(const void* workspace, void* stream);
  * wm_inject_stall - test hook for the give-up paths (the paper has no counterpart).
  * While on, calls issued by this process leave out what their bounded waits wait for: the encode
  * kernel's scanner returns at once (no tile ever gets its offset), the checksum and decode kernels
- * do not start their bulk copies.  Every wait then runs out after wm_wait_budget_ms and the call
- * ends in WM_ERR_TIMEOUT without a fault or a hang, which is what tests need to see the timeout
- * handling run (set a budget of a few tens of milliseconds first).  Off by default; never turn
- * it on in production.
+ * do not start their bulk copies.  With on == 2 it is instead the warp of the encode kernel that
+ * publishes a tile's length which never hears that the tile's widths are all there (the other calls
+ * run normally).  Every wait then runs out after wm_wait_budget_ms and the call ends in
+ * WM_ERR_TIMEOUT without a fault or a hang, which is what tests need to see the timeout handling
+ * run (set a budget of a few tens of milliseconds first).  Off by default; never turn it on in
+ * production.
  */
 void wm_inject_stall(int on);
 

@@ -173,10 +173,11 @@ def wait_budget_ms(ms: int) -> None:
     lib().wm_wait_budget_ms(int(ms))
 
 
-def inject_stall(on: bool) -> None:
+def inject_stall(on) -> None:
     """Test hook: calls issued while it is on leave out what their bounded waits wait for, so the
-    waits run out after the budget and the calls end in ERR_TIMEOUT."""
-    lib().wm_inject_stall(1 if on else 0)
+    waits run out after the budget and the calls end in ERR_TIMEOUT.  2: the encode kernel's wait
+    for a tile's widths instead of its scanner and the other calls' copies."""
+    lib().wm_inject_stall(2 if on == 2 else 1 if on else 0)
 
 
 def workspace_status(workspace, stream=None) -> int:

@@ -387,6 +387,7 @@ constexpr uint32_t kQOffShift = 22;
 // kWarpConst: all 1024 elements of the share's rows hold one value (its sign-mantissa byte rides in
 // bits 16-23 of the entry, the exponent is the base); kSumConstTile: the tile holds one value.
 constexpr uint32_t kWarpAllZero = 0x8000u, kWarpConst = 0x4000u, kSumZeroTile = 0xFFFFu, kSumConstTile = 0xFFFEu;
+constexpr uint32_t kSumRaw = 256u;          // as the sum of the widths: stored raw (any sum above 253 is)
 // The tile is stored in ENT form (shorter than its bit planes and than raw); low half: words of its streams.
 constexpr uint32_t kSumEnt = 0x10000u;
 
@@ -504,7 +505,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     const uint32_t bar_s = tc_s + (uint32_t)offsetof(EncTeamCtl, mbar) + 8u * warp;
     const bool leader = (tt == 0);
     uint32_t stuck = 0;                // kStuck when a copy into the stage has not come
-    uint32_t measured_phase = 0;       // warp 3: of the measures'
+    uint32_t no_measures = 0;          // warp 3: kStuck when a wait for the team's measures has run out
 
     auto is_tile = [](uint32_t q) { return (int32_t)q >= 0; };
     // (the placement words are indexed by ticket: with a mask that is the tile's entry in kring, else the tile number)
@@ -556,7 +557,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         }
     }
     if (lane == 0) mbar_init(&tc->mbar[warp], 1);
-    if (tt == 96u) mbar_init(&tc->measured, 4);
+    if (tt == 96u) mbar_init(&tc->measured, (g.inject & kInjectNoMeasures) ? 5 : 4);      // (test hook: the fifth never comes)
     enc_team_bar(team);
     qY = tc->next[0];
     unsigned long long srcY = LEAVES ? tc->nptr[0] : 0ull;      // leaf mode: where Y begins
@@ -764,22 +765,25 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             // digest when the other warps' widths are there by then, else at the end of its own measuring,
             // not behind the next team barrier: that one waits for W's offset, and an offset that comes late
             // must not hold back a length that other teams' offsets are waiting for.
+            // When the wait for the widths runs out (the call has failed then) nothing in the tables can be
+            // trusted, now or in any later step: the tile and all that follow it are published as raw, whose
+            // length is the same whatever the widths turn out to be, so that the packing step, which checks
+            // the published length against the room in the wire buffer, never writes more than that.
             bool published = false;
-            auto publish = [&]() {
-                measured_phase ^= 1u;
+            auto publish = [&](bool complete) {
                 published = true;
                 const uint32_t wt = tc->wtab[slY][lane];
-                const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u);
+                const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u), total = complete ? sum : kSumRaw;
                 // entropy option: the ENT form is taken when it is shorter than the planes and than raw
                 uint32_t ent_words = 0;
                 if (ENT) ent_words = __reduce_add_sync(0xFFFFFFFFu, lane < 8u ? tc->etab[slY][lane] >> 8 : 0u);
                 const uint32_t plane_len = total <= 253u ? 8256u + 32u * total : kTile;
-                const bool ent_tile = ENT && ent_tile_bytes(ent_words) < plane_len;
+                const bool ent_tile = ENT && complete && ent_tile_bytes(ent_words) < plane_len;
                 // unused memory (every share's first entry carries the mark): no payload
                 // (one value throughout: every share's first entry carries the mark and they are all alike;
                 // a tile of zeros has no payload, any other value 32 bytes)
                 const uint32_t wt0 = __shfl_sync(0xFFFFFFFFu, wt, 0);
-                const bool const_tile = ZEROS && __all_sync(0xFFFFFFFFu, (lane & 3u) != 0u || ((wt & kWarpConst) != 0u && wt == wt0));
+                const bool const_tile = ZEROS && complete && __all_sync(0xFFFFFFFFu, (lane & 3u) != 0u || ((wt & kWarpConst) != 0u && wt == wt0));
                 const bool zero_tile = const_tile && (wt0 & kWarpAllZero) != 0u;
                 if (lane == 0) {
                     tc->ssum[slY] = zero_tile ? kSumZeroTile : const_tile ? kSumConstTile : ent_tile ? kSumEnt | ent_words : total;
@@ -900,7 +904,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 if (early) {
                     ask();                       // (here, not in front of the widths: 586 -> 550 us with incompressible data)
                     chain(0, 8);
-                    if (warp == 3u && __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase & 1u))) publish();
+                    if (warp == 3u && !no_measures && __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), par))) publish(true);
                     chain(8, 16);
                     rotate();
                 }
@@ -909,8 +913,10 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, st));
             if (lane == 0) tc->wdig[slY][warp] = v;
             if (warp == 3u && !published) {
-                wait_for_copy_at<true>(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase, g.wait_ns, ws.ctrl);
-                publish();
+                uint32_t phase = par | no_measures;       // (one phase a step)
+                wait_for_copy_at<true>(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), phase, g.wait_ns, ws.ctrl, true);
+                no_measures = __any_sync(0xFFFFFFFFu, (phase & kStuck) != 0u) ? kStuck : 0u;
+                publish(no_measures == 0u);
             }
         } else {
             if (lane == 0) start_copy(qN, LEAVES ? srcN : tile_src(qN & kQTile), 0u);

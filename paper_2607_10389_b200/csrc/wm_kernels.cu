@@ -183,7 +183,7 @@ void wm_zero_tiles_enable(int on) { g_zero_tiles = on != 0; }
 void wm_entropy_enable(int on) { g_entropy = on != 0; }
 
 void wm_wait_budget_ms(uint32_t ms) { g_wait_ns = (ms == 0u ? 1u : ms > 4000u ? 4000u : ms) * 1000000u; }
-void wm_inject_stall(int on) { g_inject = on ? (kInjectNoScanner | kInjectNoCopy) : 0u; }
+void wm_inject_stall(int on) { g_inject = on == 2 ? kInjectNoMeasures : on ? (kInjectNoScanner | kInjectNoCopy) : 0u; }
 
 wm_status wm_workspace_status(const void* workspace, void* stream)
 {

@@ -29,8 +29,9 @@ struct Geo {
 };
 // Geo::inject.  What a bounded wait waits for is left out, so that the wait runs out and the
 // give-up path can be tested without a fault: the scanner warp returns at once (encode), the bulk
-// copies into the stages are not issued (checksum, decode).
-constexpr uint32_t kInjectNoScanner = 1u, kInjectNoCopy = 2u;
+// copies into the stages are not issued (checksum, decode), a tile's measures never count as
+// complete (encode).
+constexpr uint32_t kInjectNoScanner = 1u, kInjectNoCopy = 2u, kInjectNoMeasures = 4u;
 
 // Powers of k_chunk = x^(8 chunk_bytes), by 7-bit digit of the exponent: k_chunk^e is the product
 // of d0[e & 127], d1[(e >> 7) & 127], d2[(e >> 14) & 127] and, beyond 2^21 chunks, of the

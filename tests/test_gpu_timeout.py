@@ -25,9 +25,12 @@ BUDGET_MS = 40
 def stalled():
     """Calls issued inside the `with stalled():` block time out; outside it they run normally."""
     class Ctx:
+        def __init__(self, what=True):
+            self.what = what
+
         def __enter__(self):
             wm.wait_budget_ms(BUDGET_MS)
-            wm.inject_stall(True)
+            wm.inject_stall(self.what)
 
         def __exit__(self, *a):
             torch.cuda.synchronize()
@@ -97,6 +100,38 @@ def test_encode_gives_up_with_several_tiles_per_team(stalled, options, masked):
         crc.zero_()
         r = encode()
         assert r.ok and torch.equal(wire[: r.wire_len], want) and torch.equal(crc, want_crc)
+
+
+@pytest.mark.parametrize("options", [0, wm.OPT_ENTROPY, wm.OPT_ZERO_TILES])
+@pytest.mark.parametrize("tiles", [1, 3000])
+def test_encode_publishes_raw_lengths_when_the_widths_never_count_as_complete(stalled, options, tiles):
+    """A length that is published without its tile's widths must hold whatever they turn out to be, or the packing
+    step writes more than was checked against the room in the wire buffer: the tile has to be published as raw."""
+    n, chunk = tiles * 16384, 8 * 16384
+    g = torch.Generator("cuda").manual_seed(tiles + options)
+    cur = torch.randn(n // 2, generator=g, device="cuda").to(torch.bfloat16).view(torch.uint8)
+    cur[n // 2:].random_(0, 256, generator=g)                        # half of it incompressible
+    nc, meta = wm.num_chunks(n, chunk), wm.meta_bytes(n, chunk)
+    ws, res = wm.new_workspace(n, chunk), wm.new_result()
+    crc = torch.zeros(nc, dtype=torch.int32, device="cuda")
+    wire = torch.full((wm.wire_bound(n, chunk) + 65536,), 0xA5, dtype=torch.uint8, device="cuda")
+    wm.wm_encode_opt(cur, chunk, None, crc, wire, ws, res, options)
+    good = wm.read_result(res)
+    image, want_crc = wire[: good.wire_len].clone(), crc.clone()
+    assert good.ok and good.wire_len < meta + n
+    cap = good.wire_len                                              # (the tiles do not fit into it raw)
+    wire.fill_(0xA5)
+    t0 = time.time()
+    with stalled(2):
+        wm.wm_encode_opt(cur, chunk, None, crc, wire[:cap], ws, res, options)
+        r = wm.read_result(res)
+    assert r.status_name == "ERR_TIMEOUT" and wm.workspace_status(ws) == -10 and time.time() - t0 < 20
+    assert bool((wire[cap:] == 0xA5).all()), "wrote past wire_cap"
+    if tiles == 1:                                                   # the one tile is placed at the payload's start, raw
+        assert r.wire_len == meta + 16384 and int(wire[64 + 16 * nc: 66 + 16 * nc].view(torch.int16)) == 512
+    wm.wm_encode_opt(cur, chunk, None, crc, wire, ws, res, options)
+    r = wm.read_result(res)
+    assert r.ok and r.wire_len == good.wire_len and torch.equal(wire[: r.wire_len], image) and torch.equal(crc, want_crc)
 
 
 @pytest.mark.parametrize("options", [0, wm.OPT_ENTROPY, wm.OPT_STRICT])
