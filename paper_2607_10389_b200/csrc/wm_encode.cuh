@@ -505,7 +505,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
     const uint32_t bar_s = tc_s + (uint32_t)offsetof(EncTeamCtl, mbar) + 8u * warp;
     const bool leader = (tt == 0);
     uint32_t stuck = 0;                // kStuck when a copy into the stage has not come
-    uint32_t no_measures = 0;          // warp 3: kStuck when a wait for the team's measures has run out
+    uint32_t measured_phase = 0;       // warp 3: parity of the measures', kStuck when a wait for them has run out
 
     auto is_tile = [](uint32_t q) { return (int32_t)q >= 0; };
     // (the placement words are indexed by ticket: with a mask that is the tile's entry in kring, else the tile number)
@@ -771,6 +771,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             // the published length against the room in the wire buffer, never writes more than that.
             bool published = false;
             auto publish = [&](bool complete) {
+                measured_phase ^= 1u;
                 published = true;
                 const uint32_t wt = tc->wtab[slY][lane];
                 const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, (wt >> 8) & 15u), total = complete ? sum : kSumRaw;
@@ -904,7 +905,9 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                 if (early) {
                     ask();                       // (here, not in front of the widths: 586 -> 550 us with incompressible data)
                     chain(0, 8);
-                    if (warp == 3u && !no_measures && __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), par))) publish(true);
+                    if (warp == 3u && measured_phase < kStuck &&
+                        __all_sync(0xFFFFFFFFu, mbar_test(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase)))
+                        publish(true);
                     chain(8, 16);
                     rotate();
                 }
@@ -913,10 +916,9 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
             const uint32_t v = __reduce_xor_sync(0xFFFFFFFFu, lane_finish(S, st));
             if (lane == 0) tc->wdig[slY][warp] = v;
             if (warp == 3u && !published) {
-                uint32_t phase = par | no_measures;       // (one phase a step)
-                wait_for_copy_at<true>(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), phase, g.wait_ns, ws.ctrl, true);
-                no_measures = __any_sync(0xFFFFFFFFu, (phase & kStuck) != 0u) ? kStuck : 0u;
-                publish(no_measures == 0u);
+                wait_for_copy_at<true>(tc_s + (uint32_t)offsetof(EncTeamCtl, measured), measured_phase, g.wait_ns, ws.ctrl, true);
+                if (__any_sync(0xFFFFFFFFu, measured_phase >= kStuck)) measured_phase |= kStuck;
+                publish(measured_phase < kStuck);
             }
         } else {
             if (lane == 0) start_copy(qN, LEAVES ? srcN : tile_src(qN & kQTile), 0u);
