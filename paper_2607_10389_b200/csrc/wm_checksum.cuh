@@ -27,7 +27,7 @@ __global__ void k_checksum_init(Ctrl* ctrl)
 // here waits for a copy, so there is no outcome to report but success.
 template <int TEAMS>
 __global__ void __launch_bounds__(TEAMS * 256, 1)
-k_chunk_crcs(const unsigned char* __restrict__ cache, Geo g, Ws ws, const Tables* __restrict__ tab, uint32_t* __restrict__ crc_out)
+k_chunk_crcs(const unsigned char* cache, Geo g, Ws ws, const Tables* __restrict__ tab, uint32_t* __restrict__ crc_out)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_wdig[TEAMS][8], s_rdig[8], s_dig[TEAMS];

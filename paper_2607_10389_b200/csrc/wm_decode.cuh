@@ -65,7 +65,7 @@ __host__ __device__ __forceinline__ uint32_t check_chunks_per_warp(uint32_t tile
 // does for the other calls, and a small cache's chain has one kernel less.
 template <bool SINGLE>
 __global__ void __launch_bounds__(1024)
-k_decode_check(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g, Ws ws,
+k_decode_check(const unsigned char* wire, uint64_t wire_len, Geo g, Ws ws,
                const Tables* __restrict__ tab, wm_result* result, uint32_t meta_blocks, uint32_t expect_ent)
 {
     __shared__ uint32_t sG[1024];
@@ -871,7 +871,7 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
 // the last block to finish decides the status and, on success only, updates dst_crc_inout.
 __global__ void __launch_bounds__(1024)
 k_decode_finish(const unsigned char* __restrict__ wire, uint64_t wire_len, Geo g,
-                const unsigned char* __restrict__ dst, uint32_t* __restrict__ dst_crc, Ws ws,
+                const unsigned char* dst, uint32_t* __restrict__ dst_crc, Ws ws,
                 const Tables* __restrict__ tab, wm_result* result, const __grid_constant__ ChunkPowers cp, uint32_t strict)
 {
     __shared__ uint32_t sHT[1024];

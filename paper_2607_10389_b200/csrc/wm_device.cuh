@@ -150,6 +150,12 @@ __device__ __forceinline__ void sts_now(uint32_t addr, uint32_t v)
 // Every block of such a kernel must pass the wait before it exits or reads anything the chain
 // produced.  A kernel tells the scheduler that its successor may be brought in with
 // grid_dep_launch (the successor's blocks take SM resources as they become free).
+// Such a kernel's life begins before its predecessor has written all that it reads, and the read-only
+// data path wants memory that does not change in a kernel's whole life.  So whatever a predecessor may
+// still be writing (for a call's first kernel: everything the caller hands in; behind it, what the chain
+// itself writes) is read through plain pointers or __ldcg, never through `const __restrict__`
+// parameters or __ldg.  A chain's first kernel waits before it lets the second in, so the second and all
+// behind it find the caller's data complete when they start.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -490,7 +496,7 @@ __device__ __forceinline__ void stage_ragged_tile(unsigned char* stage, const un
     }
     if (off && tt == kTeamThreads - 1u) {              // the last word: its last bytes are not a whole word of the tile
         const uint32_t at = len & ~3u;
-        for (uint32_t j = 0; j < off; j++) v[15] |= (uint32_t)tile[at + j] << (8u * (4u - off + j));
+        for (uint32_t j = 0; j < off; j++) v[15] |= (uint32_t)__ldcg(tile + at + j) << (8u * (4u - off + j));
     }
 #pragma unroll
     for (int i = 0; i < 16; i++) {
@@ -518,14 +524,14 @@ __device__ __forceinline__ void copy_ragged_tile(unsigned char* __restrict__ dst
     for (int i = 0; i < 4; i++)
         if (16u * (tt + kTeamThreads * i) + 16u <= len) reinterpret_cast<uint4*>(dst)[tt + kTeamThreads * i] = v[i];
     const uint32_t at = (len & ~15u) + tt;
-    if (at < len) dst[at] = src[at];
+    if (at < len) dst[at] = __ldcg(src + at);
 }
 
 // CRC32C of a short run computed byte by byte (chunks shorter than four bytes).
 __device__ __forceinline__ uint32_t crc_bytewise(const uint32_t* T0, const unsigned char* p, uint32_t n)
 {
     uint32_t crc = 0xFFFFFFFFu;
-    for (uint32_t i = 0; i < n; i++) crc = T0[(crc ^ p[i]) & 0xFF] ^ (crc >> 8);
+    for (uint32_t i = 0; i < n; i++) crc = T0[(crc ^ __ldcg(p + i)) & 0xFF] ^ (crc >> 8);
     return ~crc;
 }
 

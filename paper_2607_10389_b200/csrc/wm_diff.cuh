@@ -78,7 +78,7 @@ k_diff(const unsigned char* __restrict__ cache, const unsigned char* __restrict_
 // Ascending index list of dirty chunks and their count: one block, every thread a run of
 // consecutive chunks, one prefix over the threads' counts.
 __global__ void __launch_bounds__(1024)
-k_diff_compact(Geo g, const uint8_t* __restrict__ dirty, uint32_t* __restrict__ idx_out, uint32_t* __restrict__ n_out)
+k_diff_compact(Geo g, const uint8_t* dirty, uint32_t* __restrict__ idx_out, uint32_t* __restrict__ n_out)
 {
     __shared__ uint32_t s_part[33];
     grid_dep_wait();

@@ -13,7 +13,7 @@ namespace wm {
 // chunks in ascending order (ws.plist; every thread a run of consecutive chunks, one prefix over
 // the threads' counts) and leaves the number of tiles to claim in the control block.
 __global__ void __launch_bounds__(1024)
-k_encode_init(Geo g, Ws ws, unsigned char* wire, const uint8_t* __restrict__ dirty)
+k_encode_init(Geo g, Ws ws, unsigned char* wire, const uint8_t* dirty)
 {
     grid_dep_wait();
     grid_dep_launch();
@@ -396,14 +396,14 @@ constexpr uint32_t kSumEnt = 0x10000u;
 // present chunk (plist, ascending, written by k_encode_init), so placement runs over tickets and a
 // sparse mask costs nothing for what it leaves out.  n_hot: tickets of full tiles.
 template <bool MASKED>
-__device__ __forceinline__ uint32_t describe_tile(const Geo& g, const uint32_t* __restrict__ plist, uint32_t n_hot, uint32_t k)
+__device__ __forceinline__ uint32_t describe_tile(const Geo& g, const uint32_t* plist, uint32_t n_hot, uint32_t k)
 {
     if (k >= n_hot) return kQNone;
     uint32_t t = k;
     bool first = first_in_chunk(g, k);
     if (MASKED) {
         const uint32_t j = chunk_of(g, k);
-        t = plist[j] * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
+        t = __ldcg(plist + j) * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
     }
     return t | (first ? kQFirst : 0u);
 }
@@ -594,7 +594,7 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
                     tk = next_ticket(ws.ctrl);
                 } else if (tk < n_hot) {
                     if (LEAVES) { qC = describe_tile<MASKED>(g, ws.plist, n_hot, tk); pA = tile_src(qC & kQTile); }
-                    else plA = __ldg(ws.plist + chunk_of(g, tk));
+                    else plA = __ldcg(ws.plist + chunk_of(g, tk));
                 }
             }
         };

@@ -189,8 +189,8 @@ __device__ __forceinline__ void copy_run(unsigned char* __restrict__ dst, const 
         if (i < words) q[i] = v[k];
     }
     const uint32_t rest = n - head - 4u * words;                       // at most 7
-    if (threadIdx.x < head) dst[threadIdx.x] = src[threadIdx.x];
-    if (threadIdx.x < rest) dst[n - rest + threadIdx.x] = src[n - rest + threadIdx.x];
+    if (threadIdx.x < head) dst[threadIdx.x] = __ldcg(src + threadIdx.x);
+    if (threadIdx.x < rest) dst[n - rest + threadIdx.x] = __ldcg(src + n - rest + threadIdx.x);
 }
 
 // Encode: every walked tile copied from the leaves into its slot (one block per tile at a time).
