@@ -153,8 +153,8 @@ wm_status wm_checksum_poly(const void* cache, uint64_t nbytes, uint32_t chunk_by
  *   hash_out  [dev] u64[n_chunks]; hash_out[c] = XXH64(cache[c*chunk_bytes, min((c+1)*chunk_bytes, nbytes)), seed)
  * No workspace.  Unlike a CRC, hashes of pieces cannot be combined, so there is no whole-cache
  * value and wm_encode / wm_decode_verify do not use this hash.  WM_ERR_ARG on a bad geometry.
- * Should one of the kernel's bounded waits ever run out (see wm_wait_budget_ms), the entries of the
- * chunks concerned are 0.
+ * The call cannot fail on the device: should a wait inside the kernel ever run out (see
+ * wm_wait_budget_ms), the chunks concerned are hashed again by a slower path that waits for nothing.
  */
 wm_status wm_checksum_xxh64(const void* cache, uint64_t nbytes, uint32_t chunk_bytes, uint64_t seed,
                             uint64_t* hash_out, void* stream);

@@ -316,7 +316,7 @@ wm_status wm_checksum_xxh64(const void* cache, uint64_t nbytes, uint32_t chunk_b
     // (427 blocks: 311 against 289).
     const uint32_t octets = (g.n_chunks + kXRows - 1u) / kXRows, n_sm = (uint32_t)ds->sm_count;
     if (octets <= 2u * n_sm)
-        k_xxh64_paced<<<octets, kXThreads, kXSmem, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, n_sm, g.wait_ns);
+        k_xxh64_paced<<<octets, kXThreads, kXSmem, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, n_sm, g.wait_ns, g.inject);
     else
         k_xxh64<<<(4u * g.n_chunks + 31u) / 32u, 32, 0, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out);
     g_launches = 1;

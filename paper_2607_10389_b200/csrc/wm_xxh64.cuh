@@ -126,20 +126,18 @@ static_assert(kXAhead + 2u <= kXSlots, "a slot is handed over before the ring co
 constexpr uint32_t kXFeeders = 4;                       // warps that bring the data in and multiply it
 constexpr uint32_t kXThreads = 256;                     // (warps 0, 1: chains; 2, 3, 6, 7: feeders, on the other two schedulers)
 
-// A warp's bounded wait for a phase of a barrier in shared memory; the answer is the same in every
-// lane.  The call has no result record to say that it failed, so a block that was merely descheduled
-// for a while must not be taken for one: a wait ends only when the budget has passed AND the barrier
-// has been tried 16,384 times (the warps that wait for each other are of one block and stand still
-// together).
+// A warp's wait for a phase of a barrier in shared memory, for at most the budget; the answer is the
+// same in every lane.  The call has no result record to say that it failed, and it cannot fail: when a
+// wait runs out, the block's warps leave the ring (`fail`) and the chain warp hashes its chunks with
+// loads of its own (x_walk).
 __device__ __forceinline__ bool x_wait(uint32_t bar, uint32_t parity, uint32_t budget_ns, volatile uint32_t* fail)
 {
     bool ok = mbar_try(bar, parity) != 0u;
     if (!ok) {
         const uint32_t t0 = now_ns();
-        uint32_t tries = 0;
         do {
             ok = mbar_try(bar, parity) != 0u;
-        } while (!ok && *fail == 0u && (++tries < 16384u || now_ns() - t0 <= budget_ns));
+        } while (!ok && *fail == 0u && now_ns() - t0 <= budget_ns);
     }
     ok = __all_sync(0xFFFFFFFFu, ok);
     if (!ok) *fail = 1u;
@@ -176,6 +174,22 @@ __device__ __forceinline__ void x_load16(unsigned long long (&x)[16], uint32_t a
     for (int i = 0; i < 16; i++) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(x[i]) : "r"(a + 32u * i));
 }
 
+// Accumulator k of a chunk from its start value, without the ring: sixteen stripes' loads at a time.  The
+// rare path of a wait that ran out; kept out of line.
+__device__ __noinline__ unsigned long long x_walk(unsigned long long v, const unsigned char* base, uint32_t stripes, uint32_t k)
+{
+    const unsigned long long* p = reinterpret_cast<const unsigned long long*>(base) + k;
+    for (uint32_t i = 0; i < stripes; i += 16u) {
+        unsigned long long in[16];
+#pragma unroll
+        for (uint32_t j = 0; j < 16u; j++) in[j] = i + j < stripes ? p[4ull * (i + j)] : 0ull;
+#pragma unroll
+        for (uint32_t j = 0; j < 16u; j++)
+            if (i + j < stripes) v = x_round(v, in[j]);
+    }
+    return v;
+}
+
 // One block per eight chunks.  n_sm: blocks up to that number are alone on their SM, the ones above
 // share one; their chains are walked by different warps, so that two chains never share a scheduler.
 // Measured (one chain step per 32-byte stripe): 34 ns a stripe with k_xxh64, 15 ns here with a block
@@ -184,7 +198,7 @@ __device__ __forceinline__ void x_load16(unsigned long long (&x)[16], uint32_t a
 // 12 ns) and the hand-over of a slot every 64 steps.
 __global__ void __launch_bounds__(kXThreads)
 k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk_bytes, uint32_t n_chunks,
-              unsigned long long seed, unsigned long long* __restrict__ out, uint32_t n_sm, uint32_t wait_ns)
+              unsigned long long seed, unsigned long long* __restrict__ out, uint32_t n_sm, uint32_t wait_ns, uint32_t inject)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_full[kXSlots], s_empty[kXSlots];
@@ -192,7 +206,8 @@ k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t
     const uint32_t warp = threadIdx.x / 32u, lane = threadIdx.x % 32u;
     const uint32_t chain_warp = (blockIdx.x / n_sm) & 1u;
     if (threadIdx.x == 0) {
-        for (uint32_t i = 0; i < kXSlots; i++) { mbar_init(&s_full[i], kXFeeders); mbar_init(&s_empty[i], 1); }
+        // (test hook: a slot waits for one feeder more than there are)
+        for (uint32_t i = 0; i < kXSlots; i++) { mbar_init(&s_full[i], kXFeeders + ((inject & kInjectNoCopy) ? 1u : 0u)); mbar_init(&s_empty[i], 1); }
         s_fail = 0;
     }
     __syncthreads();
@@ -305,15 +320,15 @@ k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t
         if (lane == 0) mbar_arrive_at(empty + 8u * slot);
         slot = n_slot; parity = n_parity; a = n_a;
     }
-    if (stripes) v = x_step(at_end, 0ull);
+    if (!ok) v = x_walk(v, cache + (uint64_t)(stripes ? c : 0u) * chunk_bytes, stripes, k);
+    else if (stripes) v = x_step(at_end, 0ull);
 
     // the quad's four accumulators to its first thread
     const uint32_t q0 = lane & ~3u;
     const unsigned long long v1 = __shfl_sync(0xFFFFFFFFu, v, q0), v2 = __shfl_sync(0xFFFFFFFFu, v, q0 + 1u),
                              v3 = __shfl_sync(0xFFFFFFFFu, v, q0 + 2u), v4 = __shfl_sync(0xFFFFFFFFu, v, q0 + 3u);
     if (k != 0u || c >= n_chunks) return;
-    // (fail closed: no hash of data that never arrived)
-    out[c] = ok ? x_finish(cache + (uint64_t)c * chunk_bytes, len, seed, v1, v2, v3, v4) : 0ull;
+    out[c] = x_finish(cache + (uint64_t)c * chunk_bytes, len, seed, v1, v2, v3, v4);
 }
 
 }  // namespace wm

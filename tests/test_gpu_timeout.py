@@ -204,3 +204,29 @@ def test_dirty_diff_leaves_a_clean_status_even_on_a_dirty_workspace(stalled):
     cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
     wm.wm_dirty_diff(cur, prev, chunk, dirty, None, cnt, ws)         # no waits inside: cannot time out
     assert wm.workspace_status(ws) == 0 and int(cnt.item()) == 1 and int(dirty[3].item()) == 1
+
+
+@pytest.mark.parametrize("n,chunk", [(5 * 65536 + 777, 65536), (40 * 16384 + 31, 16384), (9, 16384), (3 << 20, 1 << 20)])
+def test_xxh64_is_right_also_when_its_waits_run_out(stalled, n, chunk):
+    """The call has no record to report a failure in: a wait that runs out costs time (the budget, not more), not the hash."""
+    host = torch.randint(0, 256, (n,), dtype=torch.uint8, generator=torch.Generator().manual_seed(n))
+    cur = host.cuda()
+    out = torch.zeros(wm.num_chunks(n, chunk), dtype=torch.int64, device="cuda")
+    want = oracle.checksum_xxh64(host.numpy(), chunk, seed=77).tolist()
+
+    def timed():
+        torch.cuda.synchronize()
+        t0 = time.time()
+        wm.wm_checksum_xxh64(cur, chunk, 77, out)
+        torch.cuda.synchronize()
+        return time.time() - t0
+    timed()
+    assert out.cpu().numpy().view(np.uint64).tolist() == want
+    with stalled():
+        out.fill_(5)
+        spent = timed()
+    assert out.cpu().numpy().view(np.uint64).tolist() == want
+    assert spent < 1.0 and (n < 32 or spent >= BUDGET_MS / 1000)     # (a chunk without a whole stripe waits for nothing)
+    out.fill_(5)
+    timed()
+    assert out.cpu().numpy().view(np.uint64).tolist() == want
