@@ -159,3 +159,26 @@ def test_encode_around_the_numbers_of_teams(tiles, masked):
     r = wm.read_result(res)
     assert r.ok and r.wire_len == want.wire_len and np.array_equal(wire[: r.wire_len].cpu().numpy(), want_wire)
     assert np.array_equal(crc.cpu().numpy().view(np.uint32), want_crc)
+
+
+@pytest.mark.parametrize("tiles", [8 * 147 - 1, 8 * 147 + 147, 8 * 147 + 148, 12 * 147 + 5, 16 * 147, 16 * 147 + 1])
+@pytest.mark.parametrize("options", [0, wm.OPT_ENTROPY])
+@pytest.mark.parametrize("masked", [False, True])
+def test_encode_between_one_and_two_tiles_per_team(tiles, options, masked):
+    """Every block has the same number of tiles there, some teams a second one; capped at 37 blocks the same cache
+    has more than that.  With a mask the cache is larger and as many of its tiles are present."""
+    chunk_tiles = 1 if masked else 3
+    n, chunk = (tiles * 3 // 2 if masked else tiles) * 16384 - 5, chunk_tiles * 16384
+    g = torch.Generator("cuda").manual_seed(tiles + options)
+    cur = torch.randn((n + 1) // 2, generator=g, device="cuda").to(torch.bfloat16).view(torch.uint8)[:n].contiguous()
+    nc = wm.num_chunks(n, chunk)
+    mask = np.array([c % 3 != 2 for c in range(nc)], np.uint8) if masked else None
+    want_wire, want_crc, want = oracle.encode(cur.cpu().numpy(), chunk, dirty=mask, crc_in=np.zeros(nc, np.uint32), entropy=bool(options))
+    ws, res = wm.new_workspace(n, chunk), wm.new_result()
+    for blocks in (0, 37, 0):
+        crc = torch.zeros(nc, dtype=torch.int32, device="cuda")
+        wire = torch.zeros(wm.wire_bound(n, chunk), dtype=torch.uint8, device="cuda")
+        wm.wm_encode_opt(cur, chunk, None if mask is None else torch.from_numpy(mask).cuda(), crc, wire, ws, res, options | wm.opt_blocks(blocks))
+        r = wm.read_result(res)
+        assert r.ok and r.wire_len == want.wire_len and np.array_equal(wire[: r.wire_len].cpu().numpy(), want_wire), blocks
+        assert np.array_equal(crc.cpu().numpy().view(np.uint32), want_crc), blocks
