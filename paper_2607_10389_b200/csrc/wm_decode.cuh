@@ -836,15 +836,19 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
                     have_digest = true;
                 }
             } else if (decoded) {
-                // raw, zero and constant tiles: the sixteen words are there already
-                if (MODE != 1) {
-#pragma unroll
-                    for (int i = 0; i < 16; i++) put(i, w[i]);
-                }
+                // Raw, zero and constant tiles: the sixteen words are there already.  Digest first, then the
+                // stores: such a tile is mostly stores, and when all warps' stores go out right behind the
+                // barrier that also starts the next copy, the two hold each other up (1.68 GB of random
+                // bytes, back to back for seconds at the power limit: 585 us with the stores first, 584 with
+                // the two interleaved, 540 so; not limited, 516 either way).
                 if (MODE != 2) {
                     const uint32_t v = tile_digest_block(S, w, fold, warp, lane);
                     if (lane == 0) sts_now(tc_s + (uint32_t)offsetof(DecTeamCtl, wdig) + 32u * p + 4u * warp, v);
                     have_digest = true;
+                }
+                if (MODE != 1) {
+#pragma unroll
+                    for (int i = 0; i < 16; i++) put(i, w[i]);
                 }
             }
             };
