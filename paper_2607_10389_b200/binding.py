@@ -201,12 +201,18 @@ def _dev_u8(t: torch.Tensor, what: str) -> torch.Tensor:
 
 
 # The current stream's handle without making a Stream object of it: 0.2 us instead of 3.4, where a
-# small cache's call is 6 us of host work in all.
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# small cache's call is 6 us of host work in all.  The two functions are not public (a PyTorch without
+# CUDA has neither); the public way is taken where they are missing.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream) -> int:
-    return _raw_stream(_device()) if stream is None else stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
 def _check(rc: int, what: str) -> None:

@@ -53,3 +53,15 @@ def test_calls_refuse_to_run_without_a_device_or_on_host_tensors():
     a = torch.zeros(16384, dtype=torch.uint8)
     with pytest.raises(wm.WmError):
         wm.wm_checksum(a, 16384, torch.zeros(1, dtype=torch.int32), torch.zeros(1024, dtype=torch.uint8))
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_the_binding_imports_and_finds_the_stream_without_pytorch_private_functions(missing):
+    """A PyTorch without CUDA has neither of the two; a later one may rename them."""
+    import subprocess
+    import sys
+    code = ("import types, torch; hasattr(torch._C, %r) and delattr(torch._C, %r)\n"
+            "from paper_2607_10389_b200 import binding\n"
+            "torch.cuda.current_stream = lambda: types.SimpleNamespace(cuda_stream=77)\n"
+            "assert binding._stream(None) == 77 and binding._stream(types.SimpleNamespace(cuda_stream=5)) == 5\n" % (missing, missing))
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
