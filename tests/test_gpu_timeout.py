@@ -230,3 +230,29 @@ def test_xxh64_is_right_also_when_its_waits_run_out(stalled, n, chunk):
     out.fill_(5)
     timed()
     assert out.cpu().numpy().view(np.uint64).tolist() == want
+
+
+@pytest.mark.parametrize("tail", [0, 4097])
+def test_checksum_of_a_large_cache_fails_closed(stalled, tail):
+    """From 112 tiles per SM on a kernel of its own takes the cache, with a barrier per warp and eight waits per tile."""
+    n, chunk = 113 * torch.cuda.get_device_properties(0).multi_processor_count * 16384 + tail, 1 << 20
+    cur = torch.randint(0, 256, (n,), dtype=torch.uint8, device="cuda", generator=torch.Generator("cuda").manual_seed(tail))
+    nc = wm.num_chunks(n, chunk)
+    ws, crc = wm.new_workspace(n, chunk), torch.zeros(nc, dtype=torch.int32, device="cuda")
+
+    def checksum(fill, poly=None):
+        crc.fill_(fill)
+        if poly is None:
+            wm.wm_checksum(cur, chunk, crc, ws)
+        else:
+            wm.wm_checksum_poly(cur, chunk, poly, crc, ws)
+        return wm.workspace_status(ws)
+    assert checksum(0) == 0
+    want = crc.clone()
+    assert np.array_equal(want[-2:].cpu().numpy().view(np.uint32), oracle.checksum(cur[(nc - 2) * chunk:].cpu().numpy(), chunk))
+    for poly in (None, wm.POLY_ZLIB):
+        t0 = time.time()
+        with stalled():
+            assert checksum(0x1234, poly) == -10
+        assert bool((crc == 0).all()) and time.time() - t0 < 20
+        assert checksum(5) == 0 and torch.equal(crc, want)
