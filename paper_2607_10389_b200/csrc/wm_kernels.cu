@@ -431,7 +431,7 @@ static wm_status encode_any(const void* cache, const wm_leaf* leaves, uint32_t n
     const uint32_t init_blocks = (g.n_tiles + 1023) / 1024 < 1024 ? (g.n_tiles + 1023) / 1024 : 1024;
     launch_after(k_encode_init, init_blocks ? init_blocks : 1, 1024, 0, s, g, ws, w, dirty);
     if (leaves) {
-        const uint32_t map_blocks = (g.n_tiles + 1023) / 1024 < 148 ? (g.n_tiles + 1023) / 1024 : 148;      // a tile per thread
+        const uint32_t map_want = (g.n_tiles + 1023) / 1024, map_blocks = map_want < (uint32_t)ds->sm_count ? map_want : (uint32_t)ds->sm_count;      // a tile per thread
         launch_after(k_leaf_map, map_blocks ? map_blocks : 1, 1024, 0, s, leaves, n_leaves, g, ws, result, 0);
         launch_after(k_leaf_gather, 1024, 256, 0, s, leaves, n_leaves, g, ws);
     }
@@ -522,7 +522,7 @@ static wm_status decode_any(const void* wire, uint64_t wire_len, void* dst, cons
     const bool single = !leaves && 8ull * g.n_meta_slices + (g.n_chunks + per_warp - 1u) / per_warp <= 32u;      // one block checks, and clears
     if (!single) launch_after(k_decode_init, 1, 64, 0, s, ws);
     if (leaves) {
-        const uint32_t map_blocks = (g.n_tiles + 1023) / 1024 < 148 ? (g.n_tiles + 1023) / 1024 : 148;      // a tile per thread
+        const uint32_t map_want = (g.n_tiles + 1023) / 1024, map_blocks = map_want < (uint32_t)ds->sm_count ? map_want : (uint32_t)ds->sm_count;      // a tile per thread
         launch_after(k_leaf_map, map_blocks ? map_blocks : 1, 1024, 0, s, leaves, n_leaves, g, ws, result, 1);
     }
     // a wire shorter than the metadata is rejected by the header check before anything else is read
