@@ -20,7 +20,8 @@
  *   - Calls that share a workspace must be ordered on one stream (or by events).
  *   - A call enqueues a short chain of kernels, launched with programmatic stream
  *     serialization (a kernel may start while its predecessor on the stream drains and
- *     waits inside for its end before touching anything).  Work enqueued by the caller before
+ *     waits inside for its end before touching anything; wm_checksum_xxh64 is one kernel,
+ *     launched plainly).  Work enqueued by the caller before
  *     or after a call keeps ordinary stream order.
  *   - All integers in the wire image are little-endian.  Tile = 16384 bytes, group = 256
  *     bf16 elements; n_chunks = ceil(nbytes / chunk_bytes), n_tiles = ceil(nbytes / 16384).
@@ -76,13 +77,15 @@ uint64_t wm_workspace_bytes(uint64_t nbytes, uint32_t chunk_bytes);
 /*
  * wm_wait_budget_ms - upper bound of every device-side wait, in milliseconds.
  * Paper: fail-closed behaviour (Section 4.1: a move either completes verified or installs nothing).
- * The kernels wait in three places: for a bulk copy into shared memory, for the placement
- * scanner (encode: a tile's offset), and the scanner for the tiles' lengths.  Each wait is bounded
+ * The kernels wait for a bulk copy into shared memory, for the placement scanner (encode: a tile's
+ * offset), as the scanner for the tiles' lengths, for a tile's widths from the warps that measure it
+ * (encode), and for a slot of a ring in shared memory (wm_checksum_xxh64).  Each wait is bounded
  * by time on the GPU's own clock, not by a number of polls, so a kernel that shares the GPU with
  * other work and is descheduled for a while is not mistaken for a failure, and a real failure
  * never turns into a hang: when the budget has passed the kernel gives up, withdraws the
- * remaining work, returns, and the call reports WM_ERR_TIMEOUT (the CUDA context stays usable and
- * the next call on the same workspace starts clean).  Default 2000 ms; process-wide, read by each
+ * remaining work, waits once more, for a budget at most, for its own copies to land, returns, and the
+ * call reports WM_ERR_TIMEOUT (the CUDA context stays usable and the next call on the same workspace
+ * starts clean; wm_checksum_xxh64 finishes by a path without waits instead).  Default 2000 ms; process-wide, read by each
  * call when it is issued; 0 is taken as 1.
  */
 void wm_wait_budget_ms(uint32_t ms);
@@ -342,7 +345,7 @@ void wm_entropy_enable(int on);
  * 16-byte boundary below its first byte, the kernel shifts by the remainder; decoded tiles whose
  * destination is not four-byte aligned take halfword or byte stores, which is slower: put odd-sized
  * leaves last where the order is yours to choose).  A tile that crosses a leaf boundary, at most
- * two per leaf, is read and written byte by byte through the table.  No byte outside the leaves
+ * two per leaf, goes run by run through the table (whole words inside a run).  No byte outside the leaves
  * is ever read or written.
  * Everything else is as in wm_encode / wm_decode_verify.
  */

@@ -1,9 +1,10 @@
 // Device-side building blocks shared by the kernels: shared-memory table layout, the
 // word-strided CRC chain, GF(2) products, team barriers and small load/store helpers.
 //
-// Work unit: a "team" of 8 warps (256 threads) owns one 16 KiB tile at a time.  The tile is
-// seen as 128 rows of 128 bytes; warp w owns rows 16w .. 16w+15 and lane l owns the 32-bit
-// word l of each of those rows.  A lane therefore walks 16 words that are exactly 128 bytes
+// Work unit: a "team" of warps owns one 16 KiB tile at a time (eight warps in the decode kernel and the
+// checksum of smaller caches, four in the encode kernel, one in the checksum of large caches).  The
+// tile is seen as 128 rows of 128 bytes; a warp owns 16, 32 or all 128 consecutive rows and lane l owns
+// the 32-bit word l of each of those rows.  A lane therefore walks words that are exactly 128 bytes
 // apart, which makes its CRC contribution a Horner chain with ONE fixed multiplier
 // (x^1024, table G); the lane's place inside the row and the warp's place inside the tile
 // are folded in once per tile with two small nibble tables (NK, NW).
@@ -423,8 +424,8 @@ __device__ __forceinline__ void tmem_fence_before_sync() { asm volatile("tcgen05
 __device__ __forceinline__ void tmem_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // 16 registers -> 16 columns of this thread's lane, and back.  A store is waited for when the
-// next one is issued (a step later) and once more before the memory is handed back: its data is
-// fetched three steps on, with three such waits in between, so nobody stands still for it.
+// next one is issued and once more before the memory is handed back; its data is fetched two steps
+// on, behind a wait of its own (tmem_wait_stores in front of the fetch) that finds it long done.
 __device__ __forceinline__ void tmem_wait_stores() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_store16(uint32_t taddr, const uint32_t (&w)[16])
 {
@@ -476,8 +477,8 @@ __device__ __forceinline__ void read_staged_words_at(uint32_t stage_s, uint32_t 
 // tile.  When `first_in_chunk`, the chunk's first four bytes are complemented (the all-ones CRC
 // init).  `tile` is four-byte aligned; no byte behind its end is read.  A thread takes sixteen
 // words and has all of its loads under way together: the tile is one trip to memory long, where
-// fetching its words one after the other, byte by byte, took 8 us more (decode of 8 MB: 36.8 us, 28.7
-// now), which every call waited for at its end.
+// fetching its words one after the other, byte by byte, took 8 us more (decode of 8 MB: 36.8 us ->
+// 28.7; 18.6 with what came after), which every call waited for at its end.
 __device__ __forceinline__ void stage_ragged_tile(unsigned char* stage, const unsigned char* __restrict__ tile, uint32_t len,
                                                   bool first_in_chunk, uint32_t tt)
 {

@@ -5,9 +5,13 @@
 //   wm_dirty_diff    : k_diff_init -> k_diff -> k_diff_compact
 //   wm_encode        : k_encode_init -> k_encode (single pass; teams publish tile lengths, one
 //                      scanner warp turns them into payload offsets) -> k_encode_finish (directory, cache CRC, header)
-//                      -> k_meta_crc (metadata CRC, result)
-//   wm_decode_verify : k_decode_init -> k_decode_check (header, metadata CRC, structure: the gate)
+//                      -> k_meta_crc (metadata CRC, result); small caches: k_encode_close does both
+//   wm_decode_verify : k_decode_init -> k_decode_check (header, metadata CRC, structure: the gate; for small
+//                      caches one block, which clears the control block too, and no k_decode_init)
 //                      -> k_decode (unpack + CRC of decoded bytes) -> k_decode_finish
+//   leaf mode adds k_leaf_map and k_leaf_gather in front of k_encode, k_leaf_map in front of and
+//   k_leaf_scatter behind k_decode
+//   wm_checksum_xxh64: k_xxh64_paced (few chunks) or k_xxh64
 #include <cstdint>
 #include <cstdio>
 #include <cstring>

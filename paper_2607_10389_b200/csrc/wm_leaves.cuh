@@ -20,7 +20,7 @@ namespace wm {
 //     past the leaf) is a "walked" tile: it gets a 16 KiB slot in the workspace's side buffer and
 //     its address is the slot's.  k_leaf_gather fills the slots from the leaves before the encode
 //     kernel runs, k_leaf_scatter empties them into the leaves after the decode kernel has run,
-//     both run by run, byte by byte, so the main kernels see ordinary aligned tiles and carry no
+//     both run by run, whole words inside a run, so the main kernels see ordinary aligned tiles and carry no
 //     code for the exception.  There are at most two walked tiles per leaf; ws.wlist keeps their
 //     numbers, ctrl->n_walked their count.
 // Rules (a table that breaks one raises error bit 8; in decode mode it also closes the gate and
