@@ -545,13 +545,14 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         const bool one = per_block <= kEncTeams, many = per_block > 2u * kEncTeams;
         uint32_t k0 = 0xFFFFFFFFu, k1 = 0xFFFFFFFFu;
         if (team < per_block) k0 = next_ticket(ws.ctrl);
-        if (many) k1 = next_ticket(ws.ctrl);
+        if (many && k0 < n_hot) k1 = next_ticket(ws.ctrl);        // (behind the answer: the teams' second tiles come after most first ones)
         else if (team + kEncTeams < per_block) k1 = kEncTeams * (gridDim.x - 1u) + atomicAdd(&ws.ctrl->second, 1u);
         const uint32_t q0 = describe_tile<MASKED>(g, ws.plist, n_hot, k0);
         const uint32_t q1 = describe_tile<MASKED>(g, ws.plist, n_hot, k1);
         // (with a tile per team at most the next draw finds nothing, but it keeps the teams from their offsets
-        // until the scanner has them: without it 8 to 17 MB took 0.9 us longer, measured on four forms of this)
-        claiming = is_tile(many ? q1 : q0) && (one || many);
+        // until the scanner has them: without it 8 to 17 MB took 0.9 us longer, measured on four forms of this.
+        // Not with the entropy option, whose draws come too early for that and where it takes nothing.)
+        claiming = is_tile(many ? q1 : q0) && (many || (one && !ENT));
         if (MASKED) { tc->kring[0] = k0; tc->kring[1] = k1; }      // the steps in which they will be measured
         tc->next[0] = q0;
         tc->next[1] = q1;
@@ -588,19 +589,24 @@ k_encode(const unsigned char* __restrict__ cache, Geo g, const uint8_t* __restri
         }
         // Round trips to L2 are under way during a step whose answers are taken at its end: W's offset (asked
         // for by warp 2 in front of Y's second share) and the ticket of the tile to measure two steps on
-        // (the leader).  Tickets are claimed as late as that allows: the time from a claim to the tile's
-        // length, times how unevenly the teams run, is what an offset waits for.  With a mask or leaves a
-        // ticket is looked up once more (its chunk's number, its address): it is claimed at the start of
-        // the step and looked up where the others are claimed.
+        // (the leader).  Without mask, leaves and entropy option it is claimed as late as that allows, in the
+        // middle of the step: the time from a claim to the tile's length, times how unevenly the teams
+        // run, is what an offset waits for.  With a mask or leaves a ticket is looked up once more (its
+        // chunk's number, its address): it is claimed at the start of the step and looked up in the middle.
+        // With the entropy option it is claimed at the start as well: where tiles of very different lengths
+        // follow one another, teams that claim late stand at their offsets (a text model's window of
+        // 1.61 GB, three quarters zeros, 967 us late and 832 early, with zero tiles 1368 and 788, Gaussian
+        // and random pieces in turn 1318 and 892; attention caches 1076 and 1080).
+        constexpr bool kEarly = MASKED || LEAVES || ENT;
         uint32_t pv = 0, tk = 0xFFFFFFFFu, qC = kQNone, plA = 0;
         unsigned long long pA = 0;
-        if ((MASKED || LEAVES) && leader && claiming) tk = next_ticket(ws.ctrl);
+        if (kEarly && leader && claiming) tk = next_ticket(ws.ctrl);
         auto ask = [&]() {
             if (tt == 64u && is_tile(qW)) pv = ld_relaxed_u32(ws.lbk + place_of(step - 1u, qW));
             if (leader && claiming) {
-                if (!MASKED && !LEAVES) {
+                if (!kEarly) {
                     tk = next_ticket(ws.ctrl);
-                } else if (tk < n_hot) {
+                } else if ((MASKED || LEAVES) && tk < n_hot) {
                     if (LEAVES) { qC = describe_tile<MASKED>(g, ws.plist, n_hot, tk); pA = tile_src(qC & kQTile); }
                     else plA = __ldcg(ws.plist + chunk_of(g, tk));
                 }
