@@ -119,7 +119,7 @@ static const DeviceState* device_state()
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
     for (const void* f : {(const void*)k_meta_crc, (const void*)k_encode_close})
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, big) != cudaSuccess) return nullptr;
-    if (cudaFuncSetAttribute(k_xxh64_paced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXSmem) != cudaSuccess) return nullptr;
+    if (cudaFuncSetAttribute(k_xxh64_paced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2u * kXRing)) != cudaSuccess) return nullptr;
     for (int k = 0; k < 4; k++)
         for (int j = 0; j < 2; j++)
             if (cudaEventCreate(&s.ev[k][j]) != cudaSuccess) return nullptr;
@@ -314,15 +314,19 @@ wm_status wm_checksum_xxh64(const void* cache, uint64_t nbytes, uint32_t chunk_b
     const unsigned char* c = static_cast<const unsigned char*>(cache);
     unsigned long long* out = reinterpret_cast<unsigned long long*>(hash_out);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // The paced kernel takes eight chunks per block and two blocks per SM (its ring is 98 KiB): while
-    // all blocks fit at once, each chain runs at its step's latency: 162 us against 275 for 214 blocks
-    // (400 MB in 240 KiB chunks), 82 against 78 for 300, and from there on the other kernel is ahead
-    // (427 blocks: 311 against 289).
-    const uint32_t octets = (g.n_chunks + kXRows - 1u) / kXRows, n_sm = (uint32_t)ds->sm_count;
-    if (octets <= 2u * n_sm)
-        k_xxh64_paced<<<octets, kXThreads, kXSmem, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, n_sm, g.wait_ns, g.inject);
-    else
+    // The paced kernel takes up to 16 chunks per SM, the same number on every one, at 13.2 ns a stripe; with
+    // more chunks its blocks come in turns.  The other one takes 38 ns a stripe until it is bound by the
+    // memory rate (from about 7,000 chunks on), so it is ahead from three turns on.  Two turns and the other kernel: 3,000 chunks of 1 MiB 860 us and 1193,
+    // 3,542 of 240 KiB 209 and 289, 4,736 of 64 KiB 67 and 84.
+    const uint32_t n_sm = (uint32_t)ds->sm_count, turns = (g.n_chunks + 2u * kXRows * n_sm - 1u) / (2u * kXRows * n_sm);
+    const uint32_t rows = (g.n_chunks + turns * n_sm - 1u) / (turns * n_sm);
+    if (turns <= 2u) {
+        const uint32_t rows0 = rows <= kXRows ? rows : (rows + 1u) / 2u;
+        k_xxh64_paced<<<(g.n_chunks + rows - 1u) / rows, kXThreads, rows <= kXRows ? kXRing : 2u * kXRing, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, rows, rows0,
+                                                                                                                g.wait_ns, g.inject);
+    } else {
         k_xxh64<<<(4u * g.n_chunks + 31u) / 32u, 32, 0, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out);
+    }
     g_launches = 1;
     return launch_status();
 }

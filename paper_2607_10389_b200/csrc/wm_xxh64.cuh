@@ -115,16 +115,16 @@ k_xxh64(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk
 }
 
 // ---- few chunks: one warp walks the chains, the others feed it
-constexpr uint32_t kXRows = 8;                          // chunks a block works on at a time
+constexpr uint32_t kXRows = 8;                          // chunks a chain warp walks at a time, at most
 constexpr uint32_t kXSeg = 64;                          // stripes of every chunk in one slot of the ring
 constexpr uint32_t kXRowBytes = 32u * kXSeg;
 constexpr uint32_t kXPitch = kXRowBytes + 32u;          // (rows 32 bytes apart modulo 128: the chains' reads meet no bank twice)
 constexpr uint32_t kXSlot = kXRows * kXPitch;
-constexpr uint32_t kXSlots = 6, kXAhead = 4;            // slots of the ring; slots whose copies are under way
-constexpr uint32_t kXSmem = kXSlots * kXSlot;
-static_assert(kXAhead + 2u <= kXSlots, "a slot is handed over before the ring comes round to it");
+constexpr uint32_t kXSlots = 3;                         // slots of a ring (4: 13.4 ns a step, 3: 13.1)
+constexpr uint32_t kXRing = kXSlots * kXSlot;
 constexpr uint32_t kXFeeders = 4;                       // warps that bring the data in and multiply it
-constexpr uint32_t kXThreads = 256;                     // (warps 0, 1: chains; 2, 3, 6, 7: feeders, on the other two schedulers)
+constexpr uint32_t kXSets = 3;                          // slots' data that a feeder has under way in registers
+constexpr uint32_t kXThreads = 512;                     // (warps 0, 1: chains; 2, 3, 6, 7 and 10, 11, 14, 15: their feeders, on the other two schedulers)
 
 // A warp's wait for a phase of a barrier in shared memory, for at most the budget; the answer is the
 // same in every lane.  The call has no result record to say that it failed, and it cannot fail: when a
@@ -168,11 +168,7 @@ constexpr unsigned long long x_inverse(unsigned long long p)      // modulo 2^64
 constexpr unsigned long long kXP1Inverse = x_inverse(kXP1);
 __device__ __forceinline__ unsigned long long x_before(unsigned long long v) { return x_rotl(v * kXP1Inverse, 33); }
 
-__device__ __forceinline__ void x_load16(unsigned long long (&x)[16], uint32_t a)
-{
-#pragma unroll
-    for (int i = 0; i < 16; i++) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(x[i]) : "r"(a + 32u * i));
-}
+__device__ __forceinline__ void x_load1(unsigned long long& x, uint32_t a) { asm volatile("ld.shared.u64 %0, [%1];" : "=l"(x) : "r"(a)); }
 
 // Accumulator k of a chunk from its start value, without the ring: sixteen stripes' loads at a time.  The
 // rare path of a wait that ran out; kept out of line.
@@ -190,86 +186,87 @@ __device__ __noinline__ unsigned long long x_walk(unsigned long long v, const un
     return v;
 }
 
-// One block per eight chunks.  n_sm: blocks up to that number are alone on their SM, the ones above
-// share one; their chains are walked by different warps, so that two chains never share a scheduler.
-// Measured (one chain step per 32-byte stripe): 34 ns a stripe with k_xxh64, 15 ns here with a block
-// alone on its SM and 18 ns with two; 1.67 GB in 1 MiB chunks (200 blocks) 1.14 -> 0.61 ms, 8 GiB
-// of 4 MiB chunks is bound by the same chain.  What is left is the step's own latency (23 cycles,
-// 12 ns) and the hand-over of a slot every 64 steps.
-__global__ void __launch_bounds__(kXThreads)
+// One block per SM.  A block takes `rows` chunks: up to eight by one chain warp, up to sixteen by two
+// (the first has rows0 of them), each with a ring and feeders of its own.  The chains stand on schedulers
+// of their own, and every SM has the same number of chunks: a second chain on an SM costs both of them.
+// What bounds it is the latency of a step, 23 cycles (11.7 ns); it takes 13.1 ns one chain to an SM and 13.2 with
+// two (1.67 GB in 1 MiB chunks 605 -> 432 us, 2.48 GB 640 -> 434).  Before, a block had eight chunks and one chain,
+// two such blocks could stand on an SM, and wherever the second one's warps came to stand they shared the
+// first one's scheduler: 14.8 ns alone, 18.4 together.
+__global__ void __launch_bounds__(kXThreads, 1)
 k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk_bytes, uint32_t n_chunks,
-              unsigned long long seed, unsigned long long* __restrict__ out, uint32_t n_sm, uint32_t wait_ns, uint32_t inject)
+              unsigned long long seed, unsigned long long* __restrict__ out, uint32_t rows, uint32_t rows0, uint32_t wait_ns, uint32_t inject)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long s_full[kXSlots], s_empty[kXSlots];
+    __shared__ __align__(8) unsigned long long s_full[2][kXSlots], s_empty[2][kXSlots];
     __shared__ uint32_t s_fail;
     const uint32_t warp = threadIdx.x / 32u, lane = threadIdx.x % 32u;
-    const uint32_t chain_warp = (blockIdx.x / n_sm) & 1u;
-    if (threadIdx.x == 0) {
+    const uint32_t half = (warp & 2u) ? warp >> 3 : warp & 1u;           // whose chain this warp belongs to
+    const uint32_t c0 = blockIdx.x * rows + (half ? rows0 : 0u), my_rows = half ? rows - rows0 : rows0;      // the chain's chunks
+    if (threadIdx.x < 2u * kXSlots) {
         // (test hook: a slot waits for one feeder more than there are)
-        for (uint32_t i = 0; i < kXSlots; i++) { mbar_init(&s_full[i], kXFeeders + ((inject & kInjectNoCopy) ? 1u : 0u)); mbar_init(&s_empty[i], 1); }
+        mbar_init(&s_full[0][threadIdx.x], kXFeeders + ((inject & kInjectNoCopy) ? 1u : 0u));
+        mbar_init(&s_empty[0][threadIdx.x], 1);
         s_fail = 0;
     }
     __syncthreads();
-    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem);
-    const uint32_t full = (uint32_t)__cvta_generic_to_shared(s_full), empty = (uint32_t)__cvta_generic_to_shared(s_empty);
-    auto length = [&](uint32_t c) -> uint32_t {          // bytes of chunk c (0: there is none)
-        if (c >= n_chunks) return 0u;
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem) + half * kXRing;
+    const uint32_t full = (uint32_t)__cvta_generic_to_shared(s_full[half]), empty = (uint32_t)__cvta_generic_to_shared(s_empty[half]);
+    auto length = [&](uint32_t row) -> uint32_t {        // bytes of the chain's row-th chunk (0: there is none)
+        const uint32_t c = c0 + row;
+        if (row >= my_rows || c >= n_chunks) return 0u;
         const uint64_t left = nbytes - (uint64_t)c * chunk_bytes;
         return left < chunk_bytes ? (uint32_t)left : chunk_bytes;
     };
-    const uint32_t n_seg = (length(blockIdx.x * kXRows) / 32u + kXSeg - 1u) / kXSeg;      // (the first of the eight is the longest)
+    const uint32_t n_seg = (length(0u) / 32u + kXSeg - 1u) / kXSeg;      // (the first chunk is the longest)
 
     if (warp & 2u) {
         // ---- the warps that feed the ring, two chunks each: sixteen lanes take 256 consecutive bytes of
-        // one chunk, and every lane waits for its own copies only
-        const uint32_t feeder = (warp & 1u) + (warp >> 2) * 2u;
+        // one chunk at a time, straight into registers, kXSets slots ahead; the products go to the ring.
+        // (Copied into the ring first and multiplied there, every byte passed through shared memory four
+        // times, and that was what two blocks on one SM shared: 18.4 ns a step.)
+        const uint32_t feeder = (warp & 1u) + ((warp >> 2) & 1u) * 2u;
         const uint32_t row = 2u * feeder + lane / 16u, col = 16u * (lane % 16u);
         const uint32_t mine = ring + row * kXPitch + col;
         constexpr uint32_t kUnits = kXRowBytes / 256u;   // 16-byte pieces of a slot per lane
-        const uint32_t c = blockIdx.x * kXRows + row;
-        const uint32_t whole = length(c) & ~31u;         // bytes in whole stripes
-        const unsigned char* p = cache + (uint64_t)(whole ? c : 0u) * chunk_bytes + col;
-        auto hand_over = [&](uint32_t s) {               // the products, in place (all loads before the first store)
-            const uint32_t a = mine + (s % kXSlots) * kXSlot;
-            unsigned long long u[kUnits], v[kUnits];
-#pragma unroll
-            for (uint32_t i = 0; i < kUnits; i++) asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(u[i]), "=l"(v[i]) : "r"(a + 256u * i));
-#pragma unroll
-            for (uint32_t i = 0; i < kUnits; i++)
-                asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a + 256u * i), "l"(u[i] * kXP2), "l"(v[i] * kXP2) : "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive_at(full + 8u * (s % kXSlots));
-        };
-        uint32_t done = 0;
-        for (uint32_t s = 0; s < n_seg; s++) {
-            if (s >= kXSlots && !x_wait(empty + 8u * (s % kXSlots), ((s / kXSlots) & 1u) ^ 1u, wait_ns, &s_fail)) {
-                cp_async_wait_all();
-                return;
-            }
-            const uint32_t a = mine + (s % kXSlots) * kXSlot;
+        const uint32_t whole = length(row) & ~31u;       // bytes in whole stripes
+        const unsigned char* const p = cache + (uint64_t)(whole ? c0 + row : 0u) * chunk_bytes + col;
+        ulonglong2 in[kXSets][kUnits];
+        auto fetch = [&](ulonglong2 (&x)[kUnits], uint32_t s) {
             const uint32_t at = s * kXRowBytes;
 #pragma unroll
             for (uint32_t i = 0; i < kUnits; i++)
-                if (at + 256u * i + col < whole)
-                    asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(a + 256u * i), "l"(p + at + 256u * i) : "memory");
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            if (s + 1u - done > kXAhead) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(kXAhead) : "memory");
-                hand_over(done++);
+                x[i] = at + 256u * i + col < whole ? __ldcs(reinterpret_cast<const ulonglong2*>(p + at + 256u * i)) : make_ulonglong2(0ull, 0ull);
+        };
+#pragma unroll
+        for (uint32_t j = 0; j < kXSets; j++) fetch(in[j], j);
+        uint32_t slot = 0, parity = 1u;                  // (a barrier's phase before its first counts as complete)
+        for (uint32_t s0 = 0; s0 < n_seg; s0 += kXSets) {
+#pragma unroll
+            for (uint32_t j = 0; j < kXSets; j++) {
+                const uint32_t s = s0 + j;
+                if (s >= n_seg) return;
+                if (!x_wait(empty + 8u * slot, parity, wait_ns, &s_fail)) return;
+                const uint32_t a = mine + slot * kXSlot;
+#pragma unroll
+                for (uint32_t i = 0; i < kUnits; i++)
+                    asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a + 256u * i), "l"(in[j][i].x * kXP2), "l"(in[j][i].y * kXP2) : "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive_at(full + 8u * slot);
+                fetch(in[j], s + kXSets);
+                slot = slot + 1u == kXSlots ? 0u : slot + 1u;
+                if (slot == 0u) parity ^= 1u;
             }
         }
-        cp_async_wait_all();
-        while (done < n_seg) hand_over(done++);
         return;
     }
-    if (warp != chain_warp) return;
+    if (warp > 1u) return;
 
     // ---- the chains: lane 4 r + k is accumulator k of chunk r of the eight
     const uint32_t k = lane & 3u, row = lane >> 2;
     const uint32_t mine = ring + row * kXPitch + 8u * k;
-    const uint32_t c = blockIdx.x * kXRows + row;
-    const uint32_t len = length(c), stripes = len / 32u;
+    const uint32_t c = c0 + row;
+    const uint32_t len = length(row), stripes = len / 32u;
     // A segment in whose midst a chunk ends (only the cache's last chunk can) is walked with a test
     // per stripe.  Behind its chunk's end a chain runs on with whatever lies in its row, its result
     // having been put aside.
@@ -279,46 +276,60 @@ k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t
     unsigned long long v = k == 0u ? seed + kXP1 + kXP2 : k == 1u ? seed + kXP2 : k == 2u ? seed : seed - kXP1;
     unsigned long long s = x_before(v), at_end = 0ull;
     unsigned long long x0[16], x1[16];
-    auto steps = [&](const unsigned long long (&x)[16]) {
+    // sixteen steps, the loads of the next sixteen between them (in one run in front of the steps they held the
+    // chain up)
+    auto steps = [&](const unsigned long long (&x)[16], unsigned long long (&next)[16], uint32_t from) {
 #pragma unroll
-        for (int i = 0; i < 16; i++) s = x_step(s, x[i]);
+        for (int i = 0; i < 16; i++) {
+            s = x_step(s, x[i]);
+            x_load1(next[i], from + 32u * i);
+        }
     };
+    const uint32_t end_seg = (stripes + kXSeg - 1u) / kXSeg;         // of this lane's chunk
     bool ok = n_seg == 0u || x_wait(full, 0u, wait_ns, &s_fail);
-    if (n_seg) x_load16(x0, mine);
     uint32_t slot = 0, parity = 0, a = mine;             // of segment g
-    for (uint32_t g = 0; g < n_seg && ok; g++) {
+    uint32_t n_slot = 0, n_parity = 0, n_a = 0;          // of the one behind it
+    auto look_ahead = [&]() {
         const bool wrap = slot + 1u == kXSlots;
-        const uint32_t n_slot = wrap ? 0u : slot + 1u, n_parity = parity ^ (wrap ? 1u : 0u), n_a = wrap ? mine : a + kXSlot;
-        const bool more = g + 1u < n_seg;
-        // whether the next segment is there is asked, and its first words are fetched, while this one's
-        // last quarter is still to be walked: nothing waits at the seam
-        uint32_t ready = 1u;
-        if (g != odd_seg) {
-            x_load16(x1, a + 512u);
-            steps(x0);
-            x_load16(x0, a + 1024u);
-            steps(x1);
-            x_load16(x1, a + 1536u);
-            if (more) ready = mbar_test(full + 8u * n_slot, n_parity);
-            steps(x0);
-        } else {
-            ready = 0u;
-            for (uint32_t i = 0; i < kXSeg; i++) {
-                unsigned long long x;
-                asm volatile("ld.shared.u64 %0, [%1];" : "=l"(x) : "r"(a + 32u * i));
-                const unsigned long long n = x_step(s, x);
-                if (g * kXSeg + i < stripes) s = n;
-            }
-        }
-        if (more) {
-            if (!__all_sync(0xFFFFFFFFu, ready != 0u)) ok = x_wait(full + 8u * n_slot, n_parity, wait_ns, &s_fail);
-            x_load16(x0, n_a);
-        }
-        if (g != odd_seg) steps(x1);
-        if ((stripes + kXSeg - 1u) / kXSeg == g + 1u) at_end = s;
+        n_slot = wrap ? 0u : slot + 1u;
+        n_parity = parity ^ (wrap ? 1u : 0u);
+        n_a = wrap ? mine : a + kXSlot;
+    };
+    auto done = [&](uint32_t g) {                        // with segment g
+        if (end_seg == g + 1u) at_end = s;
         __syncwarp();
         if (lane == 0) mbar_arrive_at(empty + 8u * slot);
         slot = n_slot; parity = n_parity; a = n_a;
+    };
+    for (uint32_t g = 0; g < n_seg && ok;) {
+        if (g == odd_seg) {
+            look_ahead();
+            for (uint32_t i = 0; i < kXSeg; i++) {
+                unsigned long long x;
+                x_load1(x, a + 32u * i);
+                const unsigned long long n = x_step(s, x);
+                if (g * kXSeg + i < stripes) s = n;
+            }
+            if (g + 1u < n_seg) ok = x_wait(full + 8u * n_slot, n_parity, wait_ns, &s_fail);
+            done(g++);
+            continue;
+        }
+        const uint32_t g1 = g < odd_seg ? min(odd_seg, n_seg) : n_seg;       // the segments up to here have no chunk's end in their midst
+#pragma unroll
+        for (int i = 0; i < 16; i++) x_load1(x0[i], a + 32u * i);
+        for (; g < g1 && ok; g++) {
+            // whether the next segment is there is asked while this one's third quarter is still to be walked,
+            // and its first words are fetched during the last: nothing waits at the seam.  (Behind the last
+            // segment they are fetched from a slot that holds something else, and not used.)
+            look_ahead();
+            steps(x0, x1, a + 512u);
+            steps(x1, x0, a + 1024u);
+            const uint32_t ready = g + 1u < n_seg ? mbar_test(full + 8u * n_slot, n_parity) : 1u;
+            steps(x0, x1, a + 1536u);
+            if (!__all_sync(0xFFFFFFFFu, ready != 0u)) ok = x_wait(full + 8u * n_slot, n_parity, wait_ns, &s_fail);
+            steps(x1, x0, n_a);
+            done(g);
+        }
     }
     if (!ok) v = x_walk(v, cache + (uint64_t)(stripes ? c : 0u) * chunk_bytes, stripes, k);
     else if (stripes) v = x_step(at_end, 0ull);
@@ -327,7 +338,7 @@ k_xxh64_paced(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t
     const uint32_t q0 = lane & ~3u;
     const unsigned long long v1 = __shfl_sync(0xFFFFFFFFu, v, q0), v2 = __shfl_sync(0xFFFFFFFFu, v, q0 + 1u),
                              v3 = __shfl_sync(0xFFFFFFFFu, v, q0 + 2u), v4 = __shfl_sync(0xFFFFFFFFu, v, q0 + 3u);
-    if (k != 0u || c >= n_chunks) return;
+    if (k != 0u || row >= my_rows || c >= n_chunks) return;
     out[c] = x_finish(cache + (uint64_t)c * chunk_bytes, len, seed, v1, v2, v3, v4);
 }
 

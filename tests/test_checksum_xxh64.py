@@ -78,3 +78,18 @@ def test_gpu_xxh64_octets_and_ring_edges(n_chunks, last):
     wm.wm_checksum_xxh64(torch.from_numpy(a).cuda(), TILE, 99, out)
     want = [xxhash.xxh64(a[o:o + TILE].tobytes(), seed=99).intdigest() for o in range(0, n, TILE)]
     assert out.cpu().numpy().view(np.uint64).tolist() == want
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_chunks", [148, 149, 8 * 148, 8 * 148 + 1, 16 * 148, 16 * 148 + 1, 32 * 148, 32 * 148 + 1])
+@pytest.mark.parametrize("last", [17, 32, TILE - 32 * 64, TILE])
+def test_gpu_xxh64_chunks_per_sm(n_chunks, last):
+    """One and two chains on an SM, one and two turns, the other kernel; the chains' shares differ by a chunk."""
+    import torch
+    from paper_2607_10389_b200 import binding as wm
+    n = (n_chunks - 1) * TILE + last
+    a = _bytes(n, n_chunks + last)
+    out = torch.full((n_chunks + 1,), 5, dtype=torch.int64, device="cuda")
+    wm.wm_checksum_xxh64(torch.from_numpy(a).cuda(), TILE, 2 ** 63 + 1, out[:n_chunks])
+    want = [xxhash.xxh64(a[o:o + TILE].tobytes(), seed=2 ** 63 + 1).intdigest() for o in range(0, n, TILE)]
+    assert out.cpu().numpy().view(np.uint64).tolist() == want + [5]
