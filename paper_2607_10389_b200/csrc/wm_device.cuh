@@ -359,16 +359,6 @@ __device__ __forceinline__ void bulk_load_at(uint32_t d, const void* gsrc, uint3
                      ::"r"(d), "l"(gsrc), "r"(bytes), "r"(b) : "memory");
 }
 
-// Its two halves, for a stage that several copies fill.
-__device__ __forceinline__ void mbar_expect(uint32_t b, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_copy_at(uint32_t d, const void* gsrc, uint32_t bytes, uint32_t b)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d), "l"(gsrc), "r"(bytes), "r"(b) : "memory");
-}
-
 // The low 32 bits of the GPU's wall clock in nanoseconds (they wrap every 4.29 s).  Every
 // device-side wait is bounded by TIME against the call's budget (Geo::wait_ns, two seconds unless
 // the caller set another, never more than four), not by a number of polls: a block that shares
@@ -458,10 +448,6 @@ __device__ __forceinline__ void tmem_load16(uint32_t taddr, uint32_t (&w)[16])
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 

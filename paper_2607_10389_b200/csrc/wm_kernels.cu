@@ -31,8 +31,6 @@
 #include "wm_leaves.cuh"
 #include "wm_encode.cuh"
 #include "wm_meta.cuh"
-#include "wm_unpack.cuh"
-#include "wm_decode_stream.cuh"
 #include "wm_decode.cuh"
 #include "wm_xxh64.cuh"
 
