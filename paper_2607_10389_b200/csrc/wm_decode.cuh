@@ -500,13 +500,15 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         const uint32_t j = chunk_of(g, k);
         return ws.plist[j] * g.tiles_per_chunk + (k - j * g.tiles_per_chunk);
     };
+    const uint32_t teams = gridDim.x * TEAMS;
+    auto draw = [&]() -> uint32_t { return 3u * teams + atomicAdd(&ws.ctrl->ticket, 1u); };     // (three a team are dealt out)
     auto claim = [&]() -> uint32_t {
-        uint32_t k = atomicAdd(&ws.ctrl->ticket, 1u);
+        uint32_t k = draw();
         if (!masked) return k;
         while (k < n_tickets) {
             const uint32_t t = tile_of(k);
             if (t < g.n_full_tiles) return t;
-            k = atomicAdd(&ws.ctrl->ticket, 1u);
+            k = draw();
         }
         return kNone;
     };
@@ -549,24 +551,28 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
     }
     if (leader) {
         mbar_init(&tc->mbar, 1);
-        uint32_t ta, tb, tn;               // the tiles of the first three steps
-        const uint32_t n_claim = masked ? n_tickets : g.n_full_tiles, teams = gridDim.x * TEAMS;
+        // The tiles of the first three steps are dealt out: tickets k, k + teams, k + 2 teams for team k, the
+        // blocks' first teams before their second ones, and draws begin behind those.  With few tiles per team
+        // the teams', and the blocks', shares then differ by one, and nobody starts with a trip for a ticket.
+        // (Three consecutive tickets drawn at once gave some teams three tiles and others none: 10, 12, 16 and 18 MB
+        // in 64 KiB chunks 25.6, 26.8, 28.8 and 28.8 us, now 21.7, 22.5, 25.5 and 25.8; 12 MB with the entropy option
+        // 36.7 and 30.1, in 45 tensors 45.7 and 38.0, 16 MB with 60 % of it present 27.8 and 24.4; above 24 MB 1 to 3 %.)
+        const uint32_t n_claim = masked ? n_tickets : g.n_full_tiles, k = blockIdx.x + gridDim.x * team;
+        auto dealt = [&](uint32_t kk) -> uint32_t {
+            if (kk >= n_claim) return kNone;
+            if (!masked) return kk;
+            const uint32_t t = tile_of(kk);
+            return t < g.n_full_tiles ? t : claim();       // (masked: behind the end of the cache's short last chunk)
+        };
+        uint32_t ta = kNone, tb = kNone, tn = kNone;
         if (n_claim <= teams) {
-            // A tile per team at most: dealt out evenly over the blocks, nobody draws a second one.
-            // (Above that a team draws three consecutive tickets at once, which shares out a few tiles
-            // per team unevenly but saves two trips: calls of 9.3, 16, 20 and 28 MB in 64 KiB chunks take
-            // 25.4, 28.8, 29.7 and 31.5 us; 29.5, 32.8, 34.3 and 37.4 with one draw after the other and without
-            // the steps that came with this one.  Even shares are not tried there.)
-            const uint32_t k = blockIdx.x + gridDim.x * team;
-            ta = k < n_claim ? tile_of(k) : kNone;
-            tb = tn = kNone;
-        } else if (!masked) {
-            ta = atomicAdd(&ws.ctrl->ticket, 3u);
-            tb = ta + 1u;
-            tn = ta + 2u;
+            if (k < n_claim) ta = tile_of(k);
         } else {
-            ta = claim(); tb = claim(); tn = claim();
+            ta = dealt(k); tb = dealt(k + teams); tn = dealt(k + 2u * teams);
         }
+        // (a ticket without a tile, and no draw left in its place, must not stand before one that has a tile)
+        if (masked && tb == kNone) { tb = tn; tn = kNone; }
+        if (masked && ta == kNone) { ta = tb; tb = tn; tn = kNone; }
         lookup2(ta, tb);
         tc->slot[2].t = tn;                // its look-ups happen in the first step
         start_copy(tc->slot[0]);

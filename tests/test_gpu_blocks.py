@@ -182,3 +182,34 @@ def test_encode_between_one_and_two_tiles_per_team(tiles, options, masked):
         r = wm.read_result(res)
         assert r.ok and r.wire_len == want.wire_len and np.array_equal(wire[: r.wire_len].cpu().numpy(), want_wire), blocks
         assert np.array_equal(crc.cpu().numpy().view(np.uint32), want_crc), blocks
+
+
+@pytest.mark.parametrize("tiles", [1, 3, 4, 5, 8, 9, 12, 13, 14, 17])
+@pytest.mark.parametrize("tail", [0, 777])
+@pytest.mark.parametrize("chunk_tiles", [3, 4])
+def test_decode_of_one_to_four_tiles_per_team(tiles, tail, chunk_tiles):
+    """One block has four teams; the first three tickets of each are dealt out.  The sizes are the edges of that;
+    with a mask a ticket may fall behind the cache's short last chunk, wherever that stands in the list."""
+    TILE = 16384
+    chunk, n = chunk_tiles * TILE, tiles * TILE + tail
+    host = inputs.make_cache(inputs.CONFIGS["engine_small"])[:n].contiguous()
+    cur, nc = host.cuda(), wm.num_chunks(n, chunk)
+    ws, res = wm.new_workspace(n, chunk), wm.new_result()
+    last = np.zeros(nc, np.uint8)
+    last[-1] = 1
+    half = (np.arange(nc) % 2 == (nc - 1) % 2).astype(np.uint8)
+    for mask in (None, np.ones(nc, np.uint8), last, half):
+        crc = torch.zeros(nc, dtype=torch.int32, device="cuda")
+        wm.wm_checksum(cur, chunk, crc, ws)
+        wire = torch.zeros(wm.wire_bound(n, chunk), dtype=torch.uint8, device="cuda")
+        wm.wm_encode(cur, chunk, None if mask is None else torch.from_numpy(mask).cuda(), crc, wire, ws, res)
+        r = wm.read_result(res)
+        assert r.ok
+        present = np.repeat(np.ones(nc, bool) if mask is None else mask != 0, chunk)[:n]
+        start = np.where(present, 0xEE, host.numpy()).astype(np.uint8)
+        for opt in (0, wm.OPT_STRICT):
+            for blocks in (1, 2):
+                dst, dst_crc = torch.from_numpy(start).cuda(), crc.clone()
+                wm.wm_decode_verify_opt(wire, r.wire_len, dst, chunk, dst_crc, ws, res, opt | wm.opt_blocks(blocks))
+                assert wm.read_result(res).ok and torch.equal(dst, cur), (opt, blocks)
+                assert torch.equal(dst_crc, crc)
