@@ -8,9 +8,9 @@
 //   k_xxh64        a warp loads its chunks' data into registers two batches ahead and walks the
 //                  chains.  With many chunks (64 KiB each, say) there are chains enough to cover
 //                  the loads and the products, and it runs at the memory rate (6.2 TB/s).
-//   k_xxh64_paced  for few chunks, where a scheduler has one chain warp at most and the latency of
-//                  one chain step bounds the call: the chain warp does nothing but chain steps,
-//                  other warps bring the data in and take the products.
+//   k_xxh64_paced  for few chunks, where the latency of one chain step bounds the call: a chain warp
+//                  has a scheduler to itself and does nothing but chain steps, other warps bring the
+//                  data in and take the products.
 #pragma once
 
 namespace wm {

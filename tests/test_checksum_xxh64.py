@@ -67,7 +67,7 @@ def test_gpu_xxh64_engine_cache_and_bad_arguments():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n_chunks", [7, 8, 9, 2 * 148 * 8, 2 * 148 * 8 + 11])       # eight chunks a block; the last size takes the other kernel
+@pytest.mark.parametrize("n_chunks", [7, 8, 9, 2 * 148 * 8, 2 * 148 * 8 + 11])       # eight chunks a chain, sixteen an SM; the last size takes two turns
 @pytest.mark.parametrize("last", [5, 31, 2047, 2048 + 32, TILE - 9, TILE])             # the ring's slots hold 2048 bytes of a chunk
 def test_gpu_xxh64_octets_and_ring_edges(n_chunks, last):
     import torch
