@@ -315,19 +315,12 @@ wm_status wm_checksum_xxh64(const void* cache, uint64_t nbytes, uint32_t chunk_b
     const unsigned char* c = static_cast<const unsigned char*>(cache);
     unsigned long long* out = reinterpret_cast<unsigned long long*>(hash_out);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // The paced kernel takes up to 16 chunks per SM, the same number on every one, at 13.2 ns a stripe; with
-    // more chunks its blocks come in turns.  The other one takes 38 ns a stripe until it is bound by the
-    // memory rate (from about 7,000 chunks on), so it is ahead from three turns on.  Two turns and the other kernel: 3,000 chunks of 1 MiB 860 us and 1193,
-    // 3,542 of 240 KiB 209 and 289, 4,736 of 64 KiB 67 and 84.
-    const uint32_t n_sm = (uint32_t)ds->sm_count, turns = (g.n_chunks + 2u * kXRows * n_sm - 1u) / (2u * kXRows * n_sm);
-    const uint32_t rows = (g.n_chunks + turns * n_sm - 1u) / (turns * n_sm);
-    if (turns <= 2u) {
-        const uint32_t rows0 = rows <= kXRows ? rows : (rows + 1u) / 2u;
-        k_xxh64_paced<<<(g.n_chunks + rows - 1u) / rows, kXThreads, rows <= kXRows ? kXRing : 2u * kXRing, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, rows, rows0,
-                                                                                                                g.wait_ns, g.inject);
-    } else {
-        k_xxh64<<<(4u * g.n_chunks + 31u) / 32u, 32, 0, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out);
-    }
+    const XxhPlan p = xxh64_plan(g.n_chunks, (uint32_t)ds->sm_count);
+    if (p.paced)
+        k_xxh64_paced<<<p.blocks, kXThreads, p.rows <= kXRows ? kXRing : 2u * kXRing, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out, p.rows, p.rows0,
+                                                                                           g.wait_ns, g.inject);
+    else
+        k_xxh64<<<p.blocks, 32, 0, s>>>(c, nbytes, chunk_bytes, g.n_chunks, seed, out);
     g_launches = 1;
     return launch_status();
 }

@@ -12,6 +12,7 @@
 //                  has a scheduler to itself and does nothing but chain steps, other warps bring the
 //                  data in and take the products.
 #pragma once
+#include "wm_xxh64_plan.h"
 
 namespace wm {
 
@@ -62,8 +63,7 @@ __global__ void __launch_bounds__(32)
 k_xxh64(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk_bytes, uint32_t n_chunks,
         unsigned long long seed, unsigned long long* __restrict__ out)
 {
-    const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t c = gt >> 2, k = gt & 3u;
+    const uint32_t c = 8u * blockIdx.x + threadIdx.x / 4u, k = threadIdx.x & 3u;       // (a chunk's number: 4 c need not fit 32 bits)
     const bool live = c < n_chunks;                     // (a quad is live or dead as a whole)
     const unsigned char* base = cache;
     uint64_t len = 0;
@@ -115,7 +115,6 @@ k_xxh64(const unsigned char* __restrict__ cache, uint64_t nbytes, uint32_t chunk
 }
 
 // ---- few chunks: one warp walks the chains, the others feed it
-constexpr uint32_t kXRows = 8;                          // chunks a chain warp walks at a time, at most
 constexpr uint32_t kXSeg = 64;                          // stripes of every chunk in one slot of the ring
 constexpr uint32_t kXRowBytes = 32u * kXSeg;
 constexpr uint32_t kXPitch = kXRowBytes + 32u;          // (rows 32 bytes apart modulo 128: the chains' reads meet no bank twice)
