@@ -2,6 +2,7 @@
 // (leaves, strict passes, entropy option) and the verdict (k_decode_finish).
 // Part of the one translation unit wm_kernels.cu (included there, in this order).
 #pragma once
+#include "wm_deal.h"
 
 namespace wm {
 
@@ -415,6 +416,17 @@ __device__ __forceinline__ bool all_of_width_4(uint2 dd)
     return (w | over) == 0u;
 }
 
+// What k_decode's prologue does for an image with a dirty mask, out of its way (see there).
+__device__ __noinline__ FirstTiles deal_masked(uint32_t k, uint32_t teams, uint32_t n_tickets, uint32_t n_full, uint32_t tiles_per_chunk,
+                                               uint32_t tpc_shift, const uint32_t* plist, uint32_t* ticket)
+{
+    auto tile_of = [&](uint32_t kk) {
+        const uint32_t j = tpc_shift < 32u ? kk >> tpc_shift : kk / tiles_per_chunk;
+        return plist[j] * tiles_per_chunk + (kk - j * tiles_per_chunk);
+    };
+    return deal_first_tiles(k, teams, n_tickets, n_full, tile_of, [&]() { return 3u * teams + atomicAdd(ticket, 1u); });
+}
+
 // Unpack + checksum of the decoded bytes.  Tiles are claimed by ticket.  The team owns one
 // 16 KiB stage in shared memory; the encoded tile arrives there by one bulk copy (TMA) that is
 // started a tile ahead, each lane takes what it needs (descriptors, its 8 sign-mantissa bytes
@@ -554,27 +566,26 @@ k_decode(const unsigned char* __restrict__ wire, Geo g, unsigned char* __restric
         // The tiles of the first three steps are dealt out: tickets k, k + teams, k + 2 teams for team k, the
         // blocks' first teams before their second ones, and draws begin behind those.  With few tiles per team
         // the teams', and the blocks', shares then differ by one, and nobody starts with a trip for a ticket.
-        // (Three consecutive tickets drawn at once gave some teams three tiles and others none: 10, 12, 16 and 18 MB
-        // in 64 KiB chunks 25.6, 26.8, 28.8 and 28.8 us, now 21.7, 22.5, 25.5 and 25.8; 12 MB with the entropy option
-        // 36.7 and 30.1, in 45 tensors 45.7 and 38.0, 16 MB with 60 % of it present 27.8 and 24.4; above 24 MB 1 to 3 %.)
-        const uint32_t n_claim = masked ? n_tickets : g.n_full_tiles, k = blockIdx.x + gridDim.x * team;
-        auto dealt = [&](uint32_t kk) -> uint32_t {
-            if (kk >= n_claim) return kNone;
-            if (!masked) return kk;
-            const uint32_t t = tile_of(kk);
-            return t < g.n_full_tiles ? t : claim();       // (masked: behind the end of the cache's short last chunk)
-        };
-        uint32_t ta = kNone, tb = kNone, tn = kNone;
-        if (n_claim <= teams) {
-            if (k < n_claim) ta = tile_of(k);
-        } else {
-            ta = dealt(k); tb = dealt(k + teams); tn = dealt(k + 2u * teams);
-        }
-        // (a ticket without a tile, and no draw left in its place, must not stand before one that has a tile)
-        if (masked && tb == kNone) { tb = tn; tn = kNone; }
-        if (masked && ta == kNone) { ta = tb; tb = tn; tn = kNone; }
-        lookup2(ta, tb);
-        tc->slot[2].t = tn;                // its look-ups happen in the first step
+        // Three consecutive tickets drawn at once gave some teams three tiles and others none: 10, 16, 24 and 40 MB in
+        // 64 KiB chunks 25.3, 28.5, 31.1 and 36.4 us, dealt out 20.2, 23.8, 29.0 and 35.0; 100 and 400 MB 59.0 and 157, 57.7
+        // and 156; nothing from 1.6 GB on.  The price: a block that gets its SM late, because another stream's kernel has
+        // it, still owns its tiles.  With 20 SMs held for the whole call 24, 100 and 400 MB take 67, 101 and 208 us
+        // (drawn 61, 94 and 201); with the blocks capped to the free SMs 55 and 88 (drawn 58 and 90).
+        // Without a mask a ticket is its tile's number (n_full_tiles or more: none), and there is nothing to ask; what
+        // a mask needs is a call, so that calls without one do not carry it: with it inline 2 and 8 MB took 18.64 and 18.75
+        // us, so 18.2 and 18.4 (drawn 18.35 and 18.50).  Two cases keep code of their own: a mask with a ticket per
+        // team (8 MB, half of it present: 0.2 us), and a strict call's first pass, whose loop comes out 2 % slower
+        // beside the call (1.6 GB strict 913 us, so 898).
+        const uint32_t k = blockIdx.x + gridDim.x * team;
+        FirstTiles f = {k, k + teams, k + 2u * teams};
+        if (MODE == 1)
+            f = deal_first_tiles_inline(k, teams, masked ? n_tickets : g.n_full_tiles, g.n_full_tiles, masked, tile_of, draw);
+        else if (MODE == 0 && masked && n_tickets <= teams)
+            f = {k < n_tickets ? tile_of(k) : kNone, kNone, kNone};
+        else if (masked)
+            f = deal_masked(k, teams, n_tickets, g.n_full_tiles, g.tiles_per_chunk, g.tpc_shift, ws.plist, &ws.ctrl->ticket);
+        lookup2(f.a, f.b);
+        tc->slot[2].t = f.c;               // its look-ups happen in the first step
         start_copy(tc->slot[0]);
     }
     team_bar(team);
