@@ -25,15 +25,14 @@
 #include "wm_device.cuh"
 
 // The kernels, one file per call (a single translation unit: the host side below launches them).
-// (Their order is their place in the library: with the xxh64 kernels last an encode call of 8 MB took 1.3 % more.)
 #include "wm_layout.cuh"
 #include "wm_checksum.cuh"
-#include "wm_xxh64.cuh"
 #include "wm_diff.cuh"
 #include "wm_leaves.cuh"
 #include "wm_encode.cuh"
 #include "wm_meta.cuh"
 #include "wm_decode.cuh"
+#include "wm_xxh64.cuh"
 
 // Scratch and tables of wm_checksum_noalloc live in the library image itself: two file-scope
 // __device__ arrays that every GPU loading the library carries until the process exits.  In host
