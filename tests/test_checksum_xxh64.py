@@ -67,7 +67,7 @@ def test_gpu_xxh64_engine_cache_and_bad_arguments():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n_chunks", [7, 8, 9, 2 * 148 * 8, 2 * 148 * 8 + 11])       # eight chunks a chain, sixteen an SM; the last size takes two turns
+@pytest.mark.parametrize("n_chunks", [7, 8, 9, 2 * 148 * 8, 2 * 148 * 8 + 11])       # a chunk a block; sixteen, and two turns (of 148 SMs)
 @pytest.mark.parametrize("last", [5, 31, 2047, 2048 + 32, TILE - 9, TILE])             # the ring's slots hold 2048 bytes of a chunk
 def test_gpu_xxh64_octets_and_ring_edges(n_chunks, last):
     import torch
@@ -81,12 +81,13 @@ def test_gpu_xxh64_octets_and_ring_edges(n_chunks, last):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n_chunks", [148, 149, 8 * 148, 8 * 148 + 1, 16 * 148, 16 * 148 + 1, 32 * 148, 32 * 148 + 1])
+@pytest.mark.parametrize("per_sm,more", [(1, 0), (1, 1), (7, 1), (8, 0), (8, 1), (16, 0), (16, 1), (32, 0), (32, 1)])
 @pytest.mark.parametrize("last", [17, 32, TILE - 32 * 64, TILE])
-def test_gpu_xxh64_chunks_per_sm(n_chunks, last):
+def test_gpu_xxh64_chunks_per_sm(per_sm, more, last):
     """One and two chains on an SM, one and two turns, the other kernel; the chains' shares differ by a chunk."""
     import torch
     from paper_2607_10389_b200 import binding as wm
+    n_chunks = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
     n = (n_chunks - 1) * TILE + last
     a = _bytes(n, n_chunks + last)
     out = torch.full((n_chunks + 1,), 5, dtype=torch.int64, device="cuda")

@@ -206,9 +206,17 @@ def test_dirty_diff_leaves_a_clean_status_even_on_a_dirty_workspace(stalled):
     assert wm.workspace_status(ws) == 0 and int(cnt.item()) == 1 and int(dirty[3].item()) == 1
 
 
-@pytest.mark.parametrize("n,chunk", [(5 * 65536 + 777, 65536), (40 * 16384 + 31, 16384), (9, 16384), (3 << 20, 1 << 20)])
+@pytest.mark.parametrize("n,chunk", [(5 * 65536 + 777, 65536), (40 * 16384 + 31, 16384), (9, 16384), (3 << 20, 1 << 20),
+                                     (-2, 16384), (-8, 16384), (-16, 16384)])
 def test_xxh64_is_right_also_when_its_waits_run_out(stalled, n, chunk):
-    """The call has no record to report a failure in: a wait that runs out costs time (the budget, not more), not the hash."""
+    """The call has no record to report a failure in: a wait that runs out costs time (the budget, not more), not the hash.
+    -k: a chunk more than k for every SM, the last one short (a block of several chunks; of two chains, which share
+    the word that says a wait has run out; blocks in two turns)."""
+    turns = 1
+    if n < 0:
+        n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+        turns = 2 if n == -16 else 1
+        n = -n * n_sm * chunk + 4097
     host = torch.randint(0, 256, (n,), dtype=torch.uint8, generator=torch.Generator().manual_seed(n))
     cur = host.cuda()
     out = torch.zeros(wm.num_chunks(n, chunk), dtype=torch.int64, device="cuda")
@@ -226,7 +234,7 @@ def test_xxh64_is_right_also_when_its_waits_run_out(stalled, n, chunk):
         out.fill_(5)
         spent = timed()
     assert out.cpu().numpy().view(np.uint64).tolist() == want
-    assert spent < 1.0 and (n < 32 or spent >= BUDGET_MS / 1000)     # (a chunk without a whole stripe waits for nothing)
+    assert spent < 1.0 * turns and (n < 32 or spent >= BUDGET_MS / 1000)     # (a chunk without a whole stripe waits for nothing)
     out.fill_(5)
     timed()
     assert out.cpu().numpy().view(np.uint64).tolist() == want
