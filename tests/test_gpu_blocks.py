@@ -189,7 +189,7 @@ def test_encode_between_one_and_two_tiles_per_team(tiles, options, masked):
 @pytest.mark.parametrize("chunk_tiles", [3, 4])
 def test_decode_of_one_to_four_tiles_per_team(tiles, tail, chunk_tiles):
     """One block has four teams; the first three tickets of each are dealt out.  The sizes are the edges of that;
-    with a mask a ticket may fall behind the cache's short last chunk, wherever that stands in the list."""
+    with a mask the last tickets may fall behind the cache's short last chunk (one warp lists these few chunks, in order)."""
     TILE = 16384
     chunk, n = chunk_tiles * TILE, tiles * TILE + tail
     host = inputs.make_cache(inputs.CONFIGS["engine_small"])[:n].contiguous()
@@ -213,3 +213,37 @@ def test_decode_of_one_to_four_tiles_per_team(tiles, tail, chunk_tiles):
                 wm.wm_decode_verify_opt(wire, r.wire_len, dst, chunk, dst_crc, ws, res, opt | wm.opt_blocks(blocks))
                 assert wm.read_result(res).ok and torch.equal(dst, cur), (opt, blocks)
                 assert torch.equal(dst_crc, crc)
+
+
+@pytest.mark.parametrize("rest,tail", [(1, 0), (2, 777), (0, 5)])
+@pytest.mark.parametrize("leaves", [False, True])
+@pytest.mark.parametrize("options", [0, wm.OPT_STRICT, wm.OPT_ENTROPY, wm.OPT_ENTROPY | wm.OPT_STRICT])
+def test_masked_decode_of_few_tickets_per_team(rest, tail, leaves, options):
+    """Chunks of more than 16 tiles have a warp each in the check, so the short last chunk may stand anywhere in the list of
+    present chunks and its tickets without a tile among the first ones.  The block counts are around one and three tickets
+    per team.  (Every place in the list, one after the other: tests/test_deal.py.)"""
+    TILE, tpc = 16384, 64
+    chunk, n = tpc * TILE, (3 * tpc + rest) * TILE + tail
+    host = inputs.make_cache(inputs.CONFIGS["tiny8m"])[:n].contiguous()
+    cur, nc = host.cuda(), wm.num_chunks(n, chunk)
+    ws, res, entropy = wm.new_workspace(n, chunk), wm.new_result(), options & wm.OPT_ENTROPY
+    crc = torch.zeros(nc, dtype=torch.int32, device="cuda")
+    wm.wm_checksum(cur, chunk, crc, ws)
+    cuts = [0, 3 * TILE + 100, 40 * TILE + 102, 100 * TILE + 7, n] if leaves else [0, n]
+    for mask in ([1, 1, 1, 1], [0, 1, 0, 1], [0, 0, 0, 1], [1, 0, 1, 0]):
+        m = np.array(mask, np.uint8)
+        wire = torch.zeros(wm.wire_bound(n, chunk), dtype=torch.uint8, device="cuda")
+        wm.wm_encode_opt(cur, chunk, torch.from_numpy(m).cuda(), crc.clone(), wire, ws, res, entropy)
+        r = wm.read_result(res)
+        assert r.ok
+        start = torch.from_numpy(np.where(np.repeat(m != 0, chunk)[:n], 0xEE, host.numpy()).astype(np.uint8)).cuda()
+        tickets = tpc * int(m.sum())
+        for blocks in sorted({1, tickets // 12 - 1, tickets // 12, -(-tickets // 12), tickets // 4 - 1, tickets // 4} - {0}):
+            for _ in range(3):
+                pieces = [start[a:b].clone() for a, b in zip(cuts, cuts[1:])]
+                table = wm.make_leaf_table(pieces) if leaves else None
+                dst_crc = crc.clone()
+                wm.wm_decode_verify_opt(wire, r.wire_len, None if leaves else pieces[0], chunk, dst_crc, ws, res, options | wm.opt_blocks(blocks),
+                                        leaf_table=table, nbytes=n)
+                rd = wm.read_result(res)
+                assert rd.ok and torch.equal(torch.cat(pieces), cur) and torch.equal(dst_crc, crc), (mask, blocks)
