@@ -201,7 +201,7 @@ def _dev_u8(t: torch.Tensor, what: str) -> torch.Tensor:
 
 
 # The current stream's handle without making a Stream object of it: 0.2 us instead of 3.4, where a
-# small cache's call is 6 us of host work in all.  The two functions are not public (a PyTorch without
+# small cache's call is 4 us of host work in all.  The two functions are not public (a PyTorch without
 # CUDA has neither); the public way is taken where they are missing.
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 _device = getattr(torch._C, "_cuda_getDevice", None)

@@ -72,7 +72,8 @@ static_assert(sizeof(Ctrl) == 256, "control block is 256 bytes");
 
 // Give up: the call has failed.  The error word says why (bit 1: a wait ran out), waits end early
 // once the poison flag is up, and the ticket counter jumps past every tile, so that nobody claims
-// another one (claiming itself never has to look at a flag).
+// another one (claiming itself never has to look at a flag; decode teams still go through the tiles they
+// were dealt, three at most).
 __device__ __forceinline__ void give_up(Ctrl* ctrl)
 {
     atomicOr(&ctrl->err, 2u);

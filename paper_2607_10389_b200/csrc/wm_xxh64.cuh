@@ -185,9 +185,10 @@ __device__ __noinline__ unsigned long long x_walk(unsigned long long v, const un
     return v;
 }
 
-// One block per SM.  A block takes `rows` chunks: up to eight by one chain warp, up to sixteen by two
-// (the first has rows0 of them), each with a ring and feeders of its own.  The chains stand on schedulers
-// of their own, and every SM has the same number of chunks: a second chain on an SM costs both of them.
+// One block at a time on an SM: its 512 threads' registers (126 each) leave no room for a second one; with 64
+// or fewer two would fit, and four chains would meet on two schedulers.  A block takes `rows` chunks, the last one what
+// is left: up to eight by one chain warp, up to sixteen by two (the first has rows0 of them), each with a ring and feeders
+// of its own.  The chains stand on schedulers of their own: a second chain on the same one costs both of them.
 // What bounds it is the latency of a step, 23 cycles (11.7 ns); it takes 13.1 ns one chain to an SM and 13.2 with
 // two (1.67 GB in 1 MiB chunks 605 -> 432 us, 2.48 GB 640 -> 434).  Before, a block had eight chunks and one chain,
 // two such blocks could stand on an SM, and wherever the second one's warps came to stand they shared the

@@ -12,10 +12,12 @@ struct XxhPlan {
     uint32_t rows, rows0;     // chunks a block takes, and how many of them its first chain takes
 };
 
-// The paced kernel takes up to 16 chunks per SM, the same number on every one, at 13.2 ns a stripe; with
-// more chunks its blocks come in turns.  The other one takes 38 ns a stripe until it is bound by the
-// memory rate (from about 7,000 chunks on), so it is ahead from three turns on.  Two turns and the other kernel: 3,000 chunks of 1 MiB 860 us and 1193,
-// 3,542 of 240 KiB 209 and 289, 4,736 of 64 KiB 67 and 84.
+// The paced kernel takes up to 16 chunks per block, a block per SM at a time, at 13.2 ns a stripe; rows are
+// rounded up, so some SMs may have no block (149 chunks: 75 blocks of two).  With more chunks its blocks come in
+// turns.  The other one takes 36 to 38 ns a stripe with 2,400 chunks, 41 to 44 with 4,700, until it is bound by
+// the memory rate (from about 7,000 chunks on), so it is ahead from three turns on.  Two turns and the other kernel:
+// 3,000 chunks of 1 MiB 857 us and 1196, 3,600 of 240 KiB 210 and 294, 4,736 of 64 KiB 68 and 88, of 16 KiB 25.1
+// and 26.7 (2,369 of 16 KiB: 22.9 either way).
 // (Divided first: for the largest counts that 32 bits hold, a sum in front of the division wraps.  n_chunks >= 1.)
 inline XxhPlan xxh64_plan(uint32_t n_chunks, uint32_t n_sm)
 {
