@@ -666,7 +666,7 @@ def main():
     ap.add_argument("--no-loop", action="store_true", help="skip the pre-copy step loop")
     ap.add_argument("--zero-tiles", action="store_true", help="encoder option: all-zero tiles as table entries")
     ap.add_argument("--entropy", action="store_true", help="codec option: entropy-coded exponents (ENT tiles) in every call")
-    ap.add_argument("--variant", default="plain", choices=["plain", "masked", "leaves", "paper_leaves", "xxh64", "xxh64_64k"],
+    ap.add_argument("--variant", default="plain", choices=["plain", "masked", "leaves", "paper_leaves", "xxh64", "xxh64_64k", "xxh64_16k"],
                     help="with --profile: which calls make up a step (for profiler captures of the other kernel variants)")
     ap.add_argument("--profile", action="store_true",
                     help="profiler capture mode: round-trip check, warm-up and timed steps only")
@@ -791,7 +791,7 @@ def main():
                 wm.wm_encode_leaves(ts, n_l, C, None, crc_b, wire, ws, res_e)
                 wm.wm_decode_verify_leaves(wire, wl, td, n_l, C, crc_dst, ws, res_d)
         else:
-            xc = C if args.variant == "xxh64" else 65536
+            xc = {"xxh64": C, "xxh64_64k": 65536, "xxh64_16k": 16384}[args.variant]
             hashes = torch.zeros(wm.num_chunks(N, xc), dtype=torch.int64, device=dev)
 
             def step():
